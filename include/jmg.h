@@ -121,6 +121,13 @@ void jmg_default_options(jmg_options* opt);
 /* Bytes of `work` that the call (op, n, nrhs, dtype, opt) needs; 0 is valid. */
 size_t jmg_workspace_size(int op, int n, int nrhs, int dtype, const jmg_options* opt);
 
+/* Bytes of `work` with which the same call takes its fastest route: never less
+ * than jmg_workspace_size().  More than that only for the plain FP64 calls with a
+ * factorisation (potrf, posv and posv_host, prec NATIVE), whose trailing updates
+ * then run on the tensor cores in error-free slices (about 7.2 KB per row of A),
+ * with a 256-byte aligned `work`; with less, they run on the FP64 CUDA cores. */
+size_t jmg_workspace_fast(int op, int n, int nrhs, int dtype, const jmg_options* opt);
+
 /*
  * potrf -- Cholesky factorisation A = L L^T in place (paper: "Software design",
  * the factorisation step of potrs).
@@ -131,7 +138,8 @@ size_t jmg_workspace_size(int op, int n, int nrhs, int dtype, const jmg_options*
  *           arithmetic and rounded to FP32)
  *   info    device int, written asynchronously (see above); may not be NULL
  *   opt     NULL or options (prec must be NATIVE)
- *   work    may be NULL when jmg_workspace_size(JMG_OP_POTRF, ...) is 0
+ *   work    may be NULL when jmg_workspace_size(JMG_OP_POTRF, ...) is 0;
+ *           jmg_workspace_fast(JMG_OP_POTRF, ...) bytes make FP64 fast
  * Asynchronous: returns once the kernels are queued on `stream`.
  */
 int jmg_potrf(int n, void* A, int lda, int dtype, int* info, const jmg_options* opt,

@@ -249,6 +249,17 @@ static int factor_mixed(int n, float* W, int ldw, const jmg_options& o, const Pl
   return sv_prepare(n, W, ldw, at<float>(work, p.off_SV), s);
 }
 
+// Plain factorisation by the scratch at hand: FP64 with room for the slices runs
+// its updates on the tensor cores, everything else on the CUDA cores.
+static int potrf_native(int n, void* A, int lda, int dtype, int nb, int* info, void* work,
+                        size_t lwork, cudaStream_t s) {
+  if (dtype == JMG_F32) return potrf_plain<float>(n, (float*)A, lda, nb, info, s);
+  const size_t fast = ozf_workspace(n);
+  if (fast > 0 && work && lwork >= fast && !(reinterpret_cast<uintptr_t>(work) & 255))
+    return potrf_split(n, (double*)A, lda, info, work, s);
+  return potrf_plain<double>(n, (double*)A, lda, nb, info, s);
+}
+
 // column max of |B| into colmax_r and R = B (start of refinement from X = 0)
 __global__ void k_copy_colmax(int n, const double* __restrict__ B, int ldb, double* __restrict__ R,
                               double* __restrict__ colmax) {
@@ -713,6 +724,16 @@ size_t jmg_workspace_size(int op, int n, int nrhs, int dtype, const jmg_options*
   return 0;
 }
 
+size_t jmg_workspace_fast(int op, int n, int nrhs, int dtype, const jmg_options* opt) {
+  jmg_options o;
+  opts_or_default(opt, &o);
+  const size_t base = jmg_workspace_size(op, n, nrhs, dtype, &o);
+  if (n <= 0 || dtype != JMG_F64 || o.prec != JMG_PREC_NATIVE) return base;
+  if (op == JMG_OP_POTRF || op == JMG_OP_POSV || op == JMG_OP_POSV_HOST)
+    return round_up(base, 256) + ozf_workspace(n);
+  return base;
+}
+
 const char* jmg_status_string(int st) {
   switch (st) {
     case JMG_OK: return "ok";
@@ -729,8 +750,6 @@ const char* jmg_status_string(int st) {
 
 int jmg_potrf(int n, void* A, int lda, int dtype, int* info, const jmg_options* opt, void* work,
               size_t lwork, void* stream) {
-  (void)work;
-  (void)lwork;
   JMG_TRY(check_common(n, lda, dtype));
   if (!info) return -5;
   if (n > 0 && !A) return -2;
@@ -740,8 +759,7 @@ int jmg_potrf(int n, void* A, int lda, int dtype, int* info, const jmg_options* 
   if (o.prec != JMG_PREC_NATIVE) return JMG_ERR_UNSUPPORTED;
   cudaStream_t s = (cudaStream_t)stream;
   JMG_CUDA(cudaMemsetAsync(info, 0, sizeof(int), s));
-  if (dtype == JMG_F32) return potrf_plain<float>(n, (float*)A, lda, o.nb, info, s);
-  return potrf_plain<double>(n, (double*)A, lda, o.nb, info, s);
+  return potrf_native(n, A, lda, dtype, o.nb, info, work, lwork, s);
 }
 
 int jmg_potrs(int n, int nrhs, const void* L, int lda, void* B, int ldb, int dtype, void* work,
@@ -786,14 +804,16 @@ int jmg_posv(int n, int nrhs, void* A, int lda, void* B, int ldb, int dtype, int
     if (nrhs > 0 && (!work || lwork < plain_solve_bytes(n, nrhs))) return JMG_ERR_WORKSPACE;
     if (reinterpret_cast<uintptr_t>(work) & 15) return JMG_ERR_ALIGN;
     JMG_CUDA(cudaMemsetAsync(info, 0, sizeof(int), s));
+    // the solve's tickets and flags first, the factor's scratch behind them
+    const size_t sb = plain_solve_bytes(n, nrhs);
+    JMG_TRY(potrf_native(n, A, lda, dtype, o.nb, info, work ? static_cast<char*>(work) + sb : nullptr,
+                         lwork > sb ? lwork - sb : 0, s));
     if (dtype == JMG_F32) {
-      JMG_TRY(potrf_plain<float>(n, (float*)A, lda, o.nb, info, s));
       if (nrhs > 0)
         JMG_TRY(solve_llt<float>(n, nrhs, (const float*)A, lda, (float*)B, ldb, (int*)work, info,
                                  s));
       return JMG_OK;
     }
-    JMG_TRY(potrf_plain<double>(n, (double*)A, lda, o.nb, info, s));
     if (nrhs > 0)
       JMG_TRY(solve_llt<double>(n, nrhs, (const double*)A, lda, (double*)B, ldb, (int*)work, info,
                                 s));

@@ -73,6 +73,7 @@ _SZ = ctypes.c_size_t
 _SIGS = {
     "jmg_default_options": (None, [ctypes.POINTER(Options)]),
     "jmg_workspace_size": (_SZ, [_I, _I, _I, _I, ctypes.POINTER(Options)]),
+    "jmg_workspace_fast": (_SZ, [_I, _I, _I, _I, ctypes.POINTER(Options)]),
     "jmg_potrf": (_I, [_I, _P, _I, _I, _P, ctypes.POINTER(Options), _P, _SZ, _P]),
     "jmg_potrs": (_I, [_I, _I, _P, _I, _P, _I, _I, _P, _SZ, _P]),
     "jmg_potrs_static": (_I, [_I, _I, _P, _I, _P, _I, _I, _P]),
@@ -190,8 +191,16 @@ def workspace_size(op: int, n: int, nrhs: int, opts: Options | None = None,
 
 def workspace(op: int, n: int, nrhs: int, opts: Options | None, device,
               dtype: int = JMG_F64) -> torch.Tensor:
-    nbytes = workspace_size(op, n, nrhs, opts, dtype)
-    return torch.empty(max(nbytes, 256), dtype=torch.uint8, device=device)
+    """Scratch of one call: enough for its fastest route, or what it needs at least
+    when the device has no room for that."""
+    need = workspace_size(op, n, nrhs, opts, dtype)
+    fast = int(load().jmg_workspace_fast(op, n, nrhs, dtype, ctypes.byref(opts) if opts else None))
+    if fast > need:
+        try:
+            return torch.empty(fast, dtype=torch.uint8, device=device)
+        except torch.cuda.OutOfMemoryError:
+            pass
+    return torch.empty(max(need, 256), dtype=torch.uint8, device=device)
 
 
 # ------------------------------------------------------------------ tensor helpers
@@ -215,8 +224,9 @@ def potrf_(A: torch.Tensor, *, nb: int = 128, info: torch.Tensor | None = None) 
     if info is None:
         info = torch.zeros(1, dtype=torch.int32, device=A.device)
     o = default_options(nb=nb)
-    st = load().jmg_potrf(n, p, lda, dt, info.data_ptr(), ctypes.byref(o), None, 0,
-                          _stream(A.device))
+    work = workspace(OP_POTRF, n, 1, o, A.device, dt)
+    st = load().jmg_potrf(n, p, lda, dt, info.data_ptr(), ctypes.byref(o), work.data_ptr(),
+                          work.numel(), _stream(A.device))
     _chk(st, "jmg_potrf")
     return info
 
@@ -313,7 +323,7 @@ def posv(A: torch.Tensor, B: torch.Tensor, *, prec: str = "fp64", words: int = 1
     info = (torch.zeros if o.prec == 0 else torch.empty)(1, dtype=torch.int32, device=A.device)
     stats = Stats()
     if work is None:
-        work = workspace(OP_POSV, n, nrhs, o, A.device)
+        work = workspace(OP_POSV, n, nrhs, o, A.device, dt)
     wp, wl = (work.data_ptr(), work.numel()) if work is not None else (None, 0)
     st = load().jmg_posv(n, nrhs, pa, lda, px, ldx, dt, info.data_ptr(), ctypes.byref(o),
                          ctypes.byref(stats), wp, wl, _stream(A.device))
