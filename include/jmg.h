@@ -168,7 +168,7 @@ int jmg_potrs(int n, int nrhs, const void* L, int lda, void* B, int ldb, int dty
  * handed out at start-up, a host framework that owns every device byte through
  * its own pool, or plain C callers without a device allocator -- and so cannot
  * pass the scratch that jmg_potrs wants.  It allocates nothing (no cudaMalloc,
- * no cudaFree, no allocating library routine); its scratch is a fixed 256 KiB
+ * no cudaFree, no allocating library routine); its scratch is a fixed 512 KiB
  * array in device memory that every GPU loading the library keeps until the
  * process exits.
  *   Arguments and results as jmg_potrs (FP64 only).

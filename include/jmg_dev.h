@@ -109,8 +109,8 @@ unsigned long long jmg_dev_set_wait_limit_ns(unsigned long long ns);
  * limit and the kernel leaves through its abort path (no trap, no fault):
  *
  * trsv_leaderless: the one-launch forward solve L Y = B (dtype JMG_F64 or
- *   JMG_F32) with every ticket offset by one, so that no CTA takes the leading
- *   role and no block of Y is ever published: every helper's flag wait runs
+ *   JMG_F32) with every ticket offset past the leaders, so that no CTA leads
+ *   and no block of Y is ever published: every helper's flag wait runs
  *   out.  `sync` holds jmg_workspace_size(JMG_OP_POTRS, n, nrhs, dtype, NULL)
  *   bytes; afterwards sync[0] == JMG_ERR_TIMEOUT and *info == -1 (info may be
  *   NULL).  B is left partly overwritten.

@@ -17,12 +17,15 @@
 namespace jmg {
 namespace {
 
-// Fixed scratch: 65536 ints (256 KiB), resident on every GPU that loads the
-// library until the process exits.  Every call shares it and it keeps the last
+// Fixed scratch: 131072 ints (512 KiB), resident on every GPU that loads the
+// library until the process exits: what the solve wants for every call within
+// the documented limit, g (2 + b) + 1 <= 65536 for g groups of 16 right-hand
+// sides and b blocks of 32 rows (it wants g (5 + b) + 1, or b + 18 when g = 1).  Every call shares it and it keeps the last
 // call's contents; the solve launcher clears the part it uses before each
 // launch (word 0, the outcome, only before the forward solve, so that it
 // carries a timeout of either direction to jmg_potrs_static_status).
-constexpr int kStaticScratchInts = 65536;
+constexpr int kStaticScratchInts = 131072;
+constexpr size_t kStaticLimit = 65536;
 static __device__ __align__(256) int g_solve_scratch[kStaticScratchInts];
 
 // Host-side device address of g_solve_scratch, one per device, looked up on the
@@ -61,7 +64,9 @@ extern "C" int jmg_potrs_static(int n, int nrhs, const void* L, int lda, void* B
   if (n == 0 || nrhs == 0) return JMG_OK;
   if (!L) return -3;
   if (!B) return -5;
-  if (trsv_sync_ints(n, nrhs) > (size_t)kStaticScratchInts) return JMG_ERR_WORKSPACE;
+  if (1 + (size_t)cdiv(nrhs, 16) * (2 + cdiv(n, 32)) > kStaticLimit ||
+      trsv_sync_ints(n, nrhs) > (size_t)kStaticScratchInts)
+    return JMG_ERR_WORKSPACE;
   int* scratch = nullptr;
   JMG_TRY(scratch_for_current_device(&scratch));
   return solve_llt<double>(n, nrhs, static_cast<const double*>(L), lda, static_cast<double*>(B),

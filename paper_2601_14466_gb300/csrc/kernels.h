@@ -50,13 +50,13 @@ int posv_small_batched(int n, int nrhs, int batch, T* A, int lda, long long sA, 
 // trsv_sync_ints(n, nrhs) ints of scratch: sync[0] is the error word (0, or
 // JMG_ERR_TIMEOUT once a device-side wait ran out; the forward solve clears it,
 // the backward solve keeps it and does nothing if it is set), then tickets,
-// finished-block counters and per-block flags.  tkt0 != 0 is a test hook: every
-// ticket is offset by tkt0, so no CTA leads and the helpers' bounded waits run
-// out (g_wait_ns).
+// finished-block counters and per-block flags.  hold != 0 is a test hook: every
+// ticket is offset past the leaders, so no CTA leads and the helpers' bounded
+// waits run out (g_wait_ns).
 size_t trsv_sync_ints(int n, int nrhs);
 template <typename T>
 int launch_trsv_persist(int n, int nrhs, const T* L, int lda, T* B, int ldb, int trans, int* sync,
-                        int* info, cudaStream_t s, int tkt0 = 0);
+                        int* info, cudaStream_t s, int hold = 0);
 // (L L^T) X = B: forward then backward with launch_trsv_persist.
 template <typename T>
 int solve_llt(int n, int nrhs, const T* L, int lda, T* B, int ldb, int* sync, int* info,
