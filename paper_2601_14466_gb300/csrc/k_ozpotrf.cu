@@ -21,10 +21,12 @@
 // Two-level right-looking blocking: panels of 64 columns inside blocks of NB = 512,
 // one update of the block's remaining columns per panel (depth 64) and one of the
 // whole trailing matrix per block (depth 512, sliced again with one exponent per
-// row over the block).  Factor alone on one GB300, before -> now: n = 1024
-// 3.66 -> 1.92 ms, 3000 18.6 -> 6.1, 5000 53 -> 11.2, 16384 1260 -> 84 ms (there the
-// tensor cores do 28 products of slices for one of FP64: 490 TFLOP/s over the
-// whole factorisation).
+// row over the block); the CTA that updates the next diagonal block factors it in
+// the same launch, so a panel is two launches.  Factor alone on one GB300, FP64
+// CUDA-core updates -> here: n = 1024 3.66 -> 1.10 ms, 3000 18.6 -> 3.6, 5000
+// 53 -> 7.1, 16384 1260 -> 66.6 ms (there the tensor cores do 28 products of slices
+// for one of FP64: 620 TFLOP/s over the whole factorisation).  Per panel, small
+// trailing matrix: 51 us tile + diagonal block, 19 us panel solve.
 #include <algorithm>
 
 #include "kernels.h"
@@ -45,6 +47,7 @@ constexpr int B_BUF = S * B_TILE;
 constexpr int SMEM = 2 * B_BUF + ASTAGES * A_TILE + 1024 + 256;
 constexpr uint32_t TCOLS = 512;      // 7 levels x 64 columns, rounded up
 constexpr int PW = 64;               // panel width
+constexpr int PT = 256;              // threads of the panel solve
 constexpr int GROUP = 8;             // row tiles per raster group
 constexpr int E_BAD = 1 << 20;       // exponent of a row that is not finite
 
@@ -116,26 +119,217 @@ static long long tile_count(int TI, int TJ) {
   return (long long)GROUP * W * gt * (gt + 1) / 2 + (long long)(G - gt) * GROUP * TJ;
 }
 
-// c - v 2^ex with one FP64 subtraction: v is rounded once to FP64 and its
-// exponent field is moved by integer addition where it stays normal.
-JMG_DEV double sub_scaled(double c, long long v, int ex) {
-  if (v == 0) return c;
-  double d = (double)v;
-  const int E = ((__double2hiint(d) >> 20) & 0x7FF) + ex;
-  if (E > 0 && E < 0x7FF)
-    d = __hiloint2double(__double2hiint(d) + (ex << 20), __double2loint(d));
-  else
-    d = ldexp(d, ex);
-  return c - d;
+// v 2^ex rounded once to FP64 (to nearest even), in integer operations: a
+// conversion holds the FP64 pipe as long as an FMA.
+JMG_DEV double scaled_double(long long v, int ex) {
+  if (v == 0) return 0.0;
+  const unsigned long long u = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
+  const int lz = __clzll((long long)u);
+  const unsigned long long m = u << lz;  // leading bit at 63
+  const int E = 1086 - lz + ex;          // exponent field
+  if (E < 1 || E > 2045) return ldexp((double)v, ex);
+  unsigned long long q = m >> 11;
+  const unsigned rem = (unsigned)m & 0x7FFu;
+  q += (rem > 0x400u || (rem == 0x400u && (q & 1))) ? 1 : 0;
+  // (a carry out of the significand moves into the exponent)
+  const unsigned long long bits = ((unsigned long long)(E - 1) << 52) + q;
+  return __longlong_as_double((long long)(bits | ((unsigned long long)v & (1ull << 63))));
 }
 
+// ---------------------------------------------------------------------------
+// 1 / d for normal d > 0 with a normal result, to within 0.501 ulp, on the integer
+// pipe (an FP64 division holds the FP64 pipe for several hundred clocks).  With
+// x = m / 2 in [1/2, 1) from the significand m and a 24-bit y0 ~ 1 / x from the
+// FP32 reciprocal, e = 1 - x y0 is formed exactly enough in 64-bit fixed point
+// (|e| < 2^-22) and 1 / x = y0 (1 + e + e^2) up to e^3 < 2^-66.
+JMG_DEV double rcp_fixed(double d) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(d);
+  const int ex = (int)(b >> 52);
+  const unsigned long long m = (b & ((1ull << 52) - 1)) | (1ull << 52), X = m << 11;
+  const unsigned xh = (unsigned)(X >> 32), xl = (unsigned)X;
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(__uint2float_rn(xh) * 0x1p-32f));
+  const unsigned Y0 = __float2uint_rz(y * 0x1p31f);
+  const unsigned long long P = (unsigned long long)xh * Y0 + __umulhi(xl, Y0);
+  const long long E = (long long)((1ull << 63) - P);  // e 2^63
+  const int Es = (int)(E >> 20);
+  const long long F = E + (((long long)Es * Es) >> 23);
+  const unsigned long long R = ((unsigned long long)Y0 << 32) +
+                               (unsigned long long)(2 * (long long)Y0 * (int)(F >> 32)) +
+                               (((unsigned long long)Y0 * (unsigned)F) >> 31);
+  unsigned long long o =
+      ((unsigned long long)(2045 - ex) << 52) + (((R >> 10) + 1) >> 1) - (1ull << 52);
+  if (m == (1ull << 52)) o = (unsigned long long)(2046 - ex) << 52;  // 1 / 2^k
+  return __longlong_as_double((long long)o);
+}
+// 1 / pivot; *bad when d is not positive (or NaN)
+JMG_DEV double pivot_rcp(double d, bool* bad) {
+  const int ex = (__double2hiint(d) >> 20);  // sign and exponent
+  if (ex >= 1 && ex <= 2044) return rcp_fixed(d);
+  *bad = !(d > 0.0);
+  return 1.0 / d;
+}
+
+// Diagonal block of kb <= 64 columns, in place, by one CTA of THREADS threads.  An
+// FP64 warp instruction holds its SM quarter's pipe for ~64 clocks, and the pivots
+// are a serial chain: warp 0 keeps column j in registers (two rows per lane) and in
+// step j updates column j+1, takes pivot j+1 (its reciprocal in integers) and hands
+// u_j = column j / a_jj to the trailing warps (named barrier 1); those apply
+// a_rc -= a_rj u_c to columns j+2 .. , column j+2 first, which they release
+// (named barrier 2: the chain's input of step j+1).  The trailing work sets the
+// time of the first columns and the chain that of the later ones, so the three
+// further warps of the chain's quarter help only for j < J0 (the barriers' counts
+// change there with them).  Each barrier is passed the same number of times on both
+// sides, and nothing leaves the loop early: the first pivot that is not positive is
+// recorded and the columns from it on are dropped.
+namespace diag64 {
+constexpr int TRAIL = 384, MORE = 96;  // threads of warps 1 .. 15 off / on the chain's quarter
+constexpr int J0 = 20;
+constexpr int LD = PW + 1;
+constexpr int NEL = PW * (PW + 1) / 2;
+constexpr int SMEM = (PW * LD + 2 * PW + 2 * PW) * 8 + NEL * 2;
+}  // namespace diag64
+
+JMG_DEV void bar_sync(int id, int count) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
+}
+JMG_DEV void bar_arrive(int id, int count) {
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(count) : "memory");
+}
+
+JMG_DEV void diag_body(double* sm_d64, double* __restrict__ A, int lda, int kb, int koff,
+                       int* __restrict__ info) {
+  using namespace diag64;
+  constexpr int TH = THREADS;
+  double* s64 = sm_d64;                 // s64[c * LD + r] = a_rc
+  double* s_u = s64 + PW * LD;          // [2][PW]
+  double* s_l = s_u + 2 * PW;           // [PW]
+  double* s_il = s_l + PW;              // [PW]
+  unsigned short* s_rc = reinterpret_cast<unsigned short*>(s_il + PW);  // packed -> (c, r)
+  __shared__ int fail;
+  const int t = threadIdx.x, warp = t / 32, lane = t % 32;
+  if (t == 0) fail = *(volatile int*)info;
+  __syncthreads();
+  if (fail != 0) return;  // an earlier block already failed
+  {
+    constexpr int Q = (PW * PW + TH - 1) / TH;
+    double v[Q];
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {  // all loads first
+      const int idx = t + TH * q, r = idx % PW, c = idx / PW;
+      v[q] = (idx < PW * PW && r < kb && c <= r) ? A[(size_t)c * lda + r] : 0.0;
+    }
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+      const int idx = t + TH * q;
+      if (idx < PW * PW) s64[(idx / PW) * LD + idx % PW] = v[q];
+    }
+  }
+  for (int c = warp; c < PW; c += TH / 32) {
+    const int base = c * PW - c * (c - 1) / 2;  // column c starts here in packed order
+    for (int r = c + lane; r < PW; r += 32) s_rc[base + r - c] = (unsigned short)((c << 8) | r);
+  }
+  __syncthreads();
+  if (warp == 0) {
+    double lo = s64[lane], hi = s64[lane + 32];  // column j, rows lane and lane + 32
+    bool bad = false;
+    double w = pivot_rcp(__shfl_sync(0xffffffffu, lo, 0), &bad);
+    int fj = bad ? 0 : -1;  // first failing column
+    for (int j = 0; j + 1 < kb; ++j) {
+      const int j1 = j + 1;
+      const double a1 = __shfl_sync(0xffffffffu, j1 < 32 ? lo : hi, j1 & 31);
+      const double v = a1 * w;  // u of row j+1
+      if (j > 0) bar_sync(2, j - 1 < J0 ? 32 + TRAIL + MORE : 32 + TRAIL);  // column j+1 done to j-1
+      double* cn = &s64[j1 * LD];
+      double nlo = cn[lane], nhi = cn[lane + 32];
+      double* u = &s_u[(j & 1) * PW];
+      bad = false;
+      if (j1 < 32) {
+        nlo = fma(-lo, v, nlo);
+        const double d = __shfl_sync(0xffffffffu, nlo, j1);
+        u[lane] = lo * w;
+        u[lane + 32] = hi * w;
+        nhi = fma(-hi, v, nhi);
+        cn[lane] = nlo;
+        cn[lane + 32] = nhi;
+        __syncwarp();
+        bar_arrive(1, j < J0 ? 32 + TRAIL + MORE : 32 + TRAIL);
+        w = pivot_rcp(d, &bad);
+      } else {
+        nhi = fma(-hi, v, nhi);
+        const double d = __shfl_sync(0xffffffffu, nhi, j1 - 32);
+        u[lane + 32] = hi * w;
+        cn[lane + 32] = nhi;
+        __syncwarp();
+        bar_arrive(1, j < J0 ? 32 + TRAIL + MORE : 32 + TRAIL);
+        w = pivot_rcp(d, &bad);
+      }
+      if (bad && fj < 0) fj = j1;
+      lo = nlo;
+      hi = nhi;
+    }
+    if (lane == 0 && fj >= 0) fail = fj + 1;
+  } else if (warp < 16) {
+    // index among the trailing warps, those of the chain's quarter last
+    const bool more = (warp & 3) == 0;
+    const int tq = (more ? 12 + warp / 4 - 1 : warp - 1 - warp / 4) * 32 + lane;
+    for (int j = 0; j + 1 < kb; ++j) {
+      if (more && j >= J0) break;
+      const int nt = j < J0 ? TRAIL + MORE : TRAIL;
+      __syncwarp();
+      bar_sync(1, 32 + nt);  // u_j and column j in place
+      const double* cj = &s64[j * LD];
+      const double* uj = &s_u[(j & 1) * PW];
+      if (j + 2 < kb) {
+        if (tq >= j + 2 && tq < kb) {
+          double* c2 = &s64[(j + 2) * LD];
+          c2[tq] = fma(-cj[tq], uj[j + 2], c2[tq]);
+        }
+        __syncwarp();
+        bar_arrive(2, 32 + nt);
+      }
+      const int c3 = j + 3;
+      const int e3 = c3 >= PW ? NEL : c3 * PW - c3 * (c3 - 1) / 2;
+      for (int e = e3 + tq; e < NEL; e += nt) {
+        const int rc = s_rc[e], c = rc >> 8, r = rc & 255;
+        if (r >= kb) continue;
+        s64[c * LD + r] = fma(-cj[r], uj[c], s64[c * LD + r]);
+      }
+    }
+  }
+  __syncthreads();
+  const int jdone = fail ? fail - 1 : kb;  // columns that are final
+  if (t < jdone) {  // l_cc = sqrt(a_cc), l_rc = a_rc / l_cc
+    const double l = sqrt(s64[t * LD + t]);
+    s_l[t] = l;
+    s_il[t] = 1.0 / l;
+  }
+  __syncthreads();
+  for (int c = warp; c < jdone; c += TH / 32)
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int r = lane + 32 * h;
+      if (r >= c && r < kb) A[(size_t)c * lda + r] = r == c ? s_l[c] : s64[c * LD + r] * s_il[c];
+    }
+  if (t == 0 && fail) atomicCAS(info, 0, koff + fail);
+}
+
+__global__ void __launch_bounds__(THREADS) k_oz_diag(double* __restrict__ A, int lda, int kb,
+                                                     int koff, int* __restrict__ info) {
+  extern __shared__ __align__(16) double sm_diag64[];
+  diag_body(sm_diag64, A, lda, kb, koff, info);
+}
+
+// ---------------------------------------------------------------------------
 // C (rows and columns from r0 on, columns below r0 + ncols, lower part) -=
-// P P^T, P given by its slices: row r of slice s is row s * n + r of the map.
+// P P^T, P given by its slices: row r of slice s is row s * n + r of the map.  CTA 0
+// takes tile 0 alone and then factors the diagonal block it has just updated (kb
+// columns), while the others work through the rest of the update.
 __global__ void __launch_bounds__(THREADS, 1)
     k_oz_syrk(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
               double* __restrict__ C, int ldc, int n, int r0, int ncols, int nkb,
-              const int* __restrict__ ex, int TI, int TJ, int ntiles, int* __restrict__ info,
-              unsigned long long wait_ns) {
+              const int* __restrict__ ex, int TI, int TJ, int ntiles, int kb_diag,
+              int* __restrict__ info, unsigned long long wait_ns) {
   using namespace tc;
   extern __shared__ __align__(1024) unsigned char sm_raw_ozf[];
   unsigned char* smem = reinterpret_cast<unsigned char*>(
@@ -153,6 +347,8 @@ __global__ void __launch_bounds__(THREADS, 1)
   __shared__ int s_fail, s_info;
 
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  // this CTA's tiles: first, first + step, ...
+  const int first = blockIdx.x, step = blockIdx.x == 0 ? ntiles : (int)gridDim.x - 1;
   if (threadIdx.x == 0) {
     s_fail = 0;
     s_info = *(volatile int*)info;
@@ -185,7 +381,7 @@ __global__ void __launch_bounds__(THREADS, 1)
   if (warp == 0) {
     if (lane == 0) {
       bool ok = true;
-      for (int b = blockIdx.x; b < ntiles && ok; b += gridDim.x) {
+      for (int b = first; b < ntiles && ok; b += step) {
         int ti, tj;
         if (!tile_of(b, TI, TJ, ti, tj)) continue;
         for (int kb = 0; kb < nkb && ok; ++kb) {
@@ -224,7 +420,7 @@ __global__ void __launch_bounds__(THREADS, 1)
       constexpr int GMAX = 256 / BN;  // B slices per MMA
       long long ga = 0, gb = 0, gw = 0;
       bool ok = true;
-      for (int b = blockIdx.x; b < ntiles && ok; b += gridDim.x) {
+      for (int b = first; b < ntiles && ok; b += step) {
         int ti, tj;
         if (!tile_of(b, TI, TJ, ti, tj)) continue;
         for (int kw = 0; kw < nkb && ok; kw += WIN, ++gw) {
@@ -284,7 +480,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     const long long half = 1ll << (47 - sh);
     long long gw = 0;
     bool ok = true;
-    for (int b = blockIdx.x; b < ntiles && ok; b += gridDim.x) {
+    for (int b = first; b < ntiles && ok; b += step) {
       int ti, tj;
       if (!tile_of(b, TI, TJ, ti, tj)) continue;
       const int row = r0 + ti * BM + q * 32 + lane;
@@ -341,7 +537,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         for (int c = 0; c < CW; ++c)
           if (c < jn) {
             const int ec = ex[c0 + c];
-            double r = sub_scaled(old[c], (long long)acc[c], er + ec - 14 - sh);
+            double r = old[c] - scaled_double((long long)acc[c], er + ec - 14 - sh);
             if (er == E_BAD || ec == E_BAD) r = __longlong_as_double(0x7FF8000000000000ll);
             cp[(size_t)c * ldc] = r;
           }
@@ -362,38 +558,44 @@ __global__ void __launch_bounds__(THREADS, 1)
   tc_fence_before();
   __syncthreads();
   if (warp == 1) tmem_dealloc(tmem, TCOLS);
+  if (blockIdx.x == 0 && !ld_shared_volatile(&s_fail)) {
+    __syncthreads();  // tile 0 is in global memory, the rings are idle
+    diag_body(reinterpret_cast<double*>(smem), C + (size_t)r0 * ldc + r0, ldc, kb_diag, r0, info);
+  }
 }
 
 // ---------------------------------------------------------------------------
 // Panel solve X L_kk^T = A21 (64 columns) and its slices.  G lanes share a row,
 // each holding the column pairs {2 (g + G i), 2 (g + G i) + 1}; the FP64 pipe
 // takes one warp instruction per ~64 clocks and SM quarter, so the row is spread
-// over just enough lanes to fill the chip.  The solve runs on unscaled columns
+// over just enough lanes to fill the chip with eight warps per SM (one warp per
+// quarter left half the issue slots to instruction-fetch and latency stalls).  The solve runs on unscaled columns
 // with Lh[j][l] = L_lj / L_jj (a_l -= a_j Lh[j][l]), the scaling by 1 / L_jj
 // comes last: one FP64 instruction per element and step, nothing else.
 template <int G>
-__global__ void __launch_bounds__(128) k_oz_panel(double* __restrict__ A, int lda, int n, int k,
+__global__ void __launch_bounds__(PT) k_oz_panel(double* __restrict__ A, int lda, int n, int k,
                                                   __nv_bfloat16* __restrict__ SP,
                                                   int* __restrict__ ex,
                                                   unsigned long long* __restrict__ rowmax,
                                                   int first, const int* __restrict__ info) {
   constexpr int NP = 32 / G;     // column pairs per lane
   constexpr int RW = 32 / G;     // rows per warp
-  constexpr int RB = 4 * RW;     // rows per CTA
+  constexpr int RB = PT / 32 * RW;  // rows per CTA
   __shared__ __align__(16) double Lh[PW * PW];
   __shared__ double rinv[PW];
   if (*(volatile const int*)info != 0) return;
   const int t = threadIdx.x, lane = t % 32, warp = t / 32;
   const double* Lkk = A + (size_t)k * lda + k;
   {
-    double v[32];
+    constexpr int Q = PW * PW / PT;
+    double v[Q];
 #pragma unroll
-    for (int i = 0; i < 32; ++i) {
-      const int idx = t + 128 * i, l = idx % PW, j = idx / PW;
+    for (int i = 0; i < Q; ++i) {
+      const int idx = t + PT * i, l = idx % PW, j = idx / PW;
       v[i] = l >= j ? Lkk[(size_t)j * lda + l] : 0.0;
     }
 #pragma unroll
-    for (int i = 0; i < 32; ++i) Lh[t + 128 * i] = v[i];
+    for (int i = 0; i < Q; ++i) Lh[t + PT * i] = v[i];
   }
   const int g = lane % G, rl = warp * RW + lane / G;
   const int row = k + PW + blockIdx.x * RB + rl;
@@ -407,8 +609,8 @@ __global__ void __launch_bounds__(128) k_oz_panel(double* __restrict__ A, int ld
   if (t < PW) rinv[t] = 1.0 / Lh[t * PW + t];
   __syncthreads();
 #pragma unroll 4
-  for (int i = 0; i < 32; ++i) {
-    const int idx = t + 128 * i, l = idx % PW, j = idx / PW;
+  for (int i = 0; i < PW * PW / PT; ++i) {
+    const int idx = t + PT * i, l = idx % PW, j = idx / PW;
     if (l > j) Lh[idx] *= rinv[j];
   }
   __syncthreads();
@@ -555,6 +757,7 @@ int potrf_split(int n, double* A, int lda, int* info, void* work, cudaStream_t s
   JMG_CUDA(cudaGetDevice(&dev));
   JMG_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
   JMG_TRY(ensure_smem(k_oz_syrk, SMEM));
+  JMG_TRY(ensure_smem(k_oz_diag, diag64::SMEM));
   CUtensorMap pa, pb, oa, ob;
   JMG_TRY(map_slices(&pa, panel, n, PW, BM));
   JMG_TRY(map_slices(&pb, panel, n, PW, BN));
@@ -567,23 +770,28 @@ int potrf_split(int n, double* A, int lda, int* info, void* work, cudaStream_t s
     const int TI = cdiv(n - r0, BM), TJ = cdiv(ncols, BN);
     const long long nt = tile_count(TI, TJ);
     k_oz_syrk<<<(int)std::min<long long>(nt, nsm), THREADS, SMEM, s>>>(
-        ma, mb, A, lda, n, r0, ncols, nkb, ex, TI, TJ, (int)nt, info, g_wait_ns);
+        ma, mb, A, lda, n, r0, ncols, nkb, ex, TI, TJ, (int)nt, std::min(PW, n - r0), info,
+        g_wait_ns);
     return launched();
   };
+  // the first diagonal block; every update leaves the next one factored
+  k_oz_diag<<<1, THREADS, diag64::SMEM, s>>>(A, lda, std::min(PW, n), 0, info);
+  JMG_TRY(launched());
   for (int k0 = 0; k0 < n; k0 += p.NB) {
     const int kend = std::min(k0 + p.NB, n);
     for (int k = k0; k < kend; k += PW) {
       const int kb = std::min(PW, n - k), m = n - k - kb;
-      JMG_TRY(launch_potf2(A + (size_t)k * lda + k, lda, kb, k, info, s));
       if (m <= 0) return JMG_OK;
       const int first = k == k0;
-      // lanes per row: enough rows per pass for the 4 quarters of every SM
-      if (m <= 32 * nsm)
-        k_oz_panel<4><<<cdiv(m, 32), 128, 0, s>>>(A, lda, n, k, panel, e_in, rowmax, first, info);
+      // lanes per row: enough rows per pass for the eight warps of every SM
+      if (m <= 16 * nsm)
+        k_oz_panel<16><<<cdiv(m, 16), PT, 0, s>>>(A, lda, n, k, panel, e_in, rowmax, first, info);
+      else if (m <= 32 * nsm)
+        k_oz_panel<8><<<cdiv(m, 32), PT, 0, s>>>(A, lda, n, k, panel, e_in, rowmax, first, info);
       else if (m <= 64 * nsm)
-        k_oz_panel<2><<<cdiv(m, 64), 128, 0, s>>>(A, lda, n, k, panel, e_in, rowmax, first, info);
+        k_oz_panel<4><<<cdiv(m, 64), PT, 0, s>>>(A, lda, n, k, panel, e_in, rowmax, first, info);
       else
-        k_oz_panel<1><<<cdiv(m, 128), 128, 0, s>>>(A, lda, n, k, panel, e_in, rowmax, first, info);
+        k_oz_panel<2><<<cdiv(m, 128), PT, 0, s>>>(A, lda, n, k, panel, e_in, rowmax, first, info);
       JMG_TRY(launched());
       if (k + PW < kend) JMG_TRY(update(pa, pb, k + PW, kend - (k + PW), 1, e_in));
     }
