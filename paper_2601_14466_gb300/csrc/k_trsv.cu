@@ -15,21 +15,22 @@
 // another SM's use of them, only for P_d, which the helpers finish LAG-1 blocks
 // ahead.
 //
-// The chain is bound by FP64 issue: a warp-wide FP64 instruction holds its SM
-// quarter's pipe for ~64 clocks, so a leader spreads its work over the quarters
-// and keeps only what must be serial on the chain.  Per right-hand side one chain
-// warp (lane = row) subtracts the product with block d-1 (32 FMAs) and substitutes
-// (32 FMAs: s_k -= (L_ki / L_ii) s_i on unscaled values, one scaling by 1 / L_kk at
-// the end, so a step is one shuffle and one FMA); aux warps on other quarters
+// The chain is bound by latency (FP64: 68 clocks for a dependent FMA, while the SM's
+// one FP64 pipe takes an independent warp instruction every 16), so a leader keeps
+// only what must be serial on it.  Per right-hand side one chain
+// warp (lane = row) subtracts the product with block d-1 and substitutes
+// (31 steps of s_k -= (L_ki / L_ii) s_i on unscaled values, one scaling by 1 / L_kk
+// at the end, so a step is one shuffle and one FMA); aux warps
 // form the products with blocks d-2 .. d-LAG+1 beforehand, prep warps scale the
 // diagonal blocks, loaders bring L through a four-step ring, and a fetching and
 // a publishing warp keep global round trips off the chain.  The roles meet
-// through counters in shared memory, no CTA-wide barrier.  A step takes 4.2 us in
-// FP64 and 1.9 us in FP32 up to 16 right-hand sides (28-32 us and 3.6 us with one
+// through counters in shared memory, no CTA-wide barrier.  A step takes 3.9 us in
+// FP64 and 1.8 us in FP32 up to 16 right-hand sides (28-32 us and 3.6 us with one
 // lane per right-hand side substituting and barriers between the phases): both
-// directions at n = 12288, 8 right-hand sides, FP64, 24.3 -> 3.8 ms; n = 8192, 16,
-// FP32, 1.85 -> 0.95 ms.  From 32 right-hand sides on FP64 is bound by the
-// helpers' products (n = 16384, 64: 35.7 ms, 0.96 TFLOP/s of 1.1).
+// directions at n = 12288, 8 right-hand sides, FP64, 24.3 -> 3.6 ms; n = 8192, 16,
+// FP32, 1.90 -> 0.92 ms.  From 32 right-hand sides on FP64 is bound by the
+// helpers' products (n = 16384, 64: 35.1 ms, 0.98 TFLOP/s of 1.1).  FP32 at
+// n = 16384, 64 right-hand sides is the one measured shape that lost: 4.35 -> 4.49 ms.
 //
 // Roles come from an atomic ticket in order (tickets below the number of leaders
 // NL lead; ticket t helps block LAG + t - NL), so the leaders are running before
@@ -39,6 +40,7 @@
 #include <algorithm>
 
 #include "kernels.h"
+#include "rcp64.cuh"
 
 namespace jmg {
 
@@ -49,13 +51,11 @@ constexpr int TH = 512;    // 16 warps
 constexpr int LDB = 33;    // row stride of a block of L in shared memory
 constexpr int RING = 4;    // leader: steps of L in flight or in use
 constexpr int SR = 8;      // leader: slots of the per-step rings (> LAG)
-constexpr int HRING = 8;   // helper: blocks of L in flight or in use
-constexpr int KCH = 4;     // finished blocks a helper multiplies per step (at most)
+constexpr int HRING = 16;  // helper: blocks of L in flight or in use
+constexpr int KCH = 8;     // finished blocks a helper multiplies per step (at most)
 
-// leader shapes: blocks the leader multiplies itself (d-1 .. d-LAG+1).  FP64
-// with one right-hand side: chain, three aux products and the scaling fill the
-// four SM quarters evenly; FP32 (no pipe limit) takes more blocks, so that the
-// helpers' round trip (~6 us) spans more steps.
+// leader shapes: blocks the leader multiplies itself (d-1 .. d-LAG+1), so many that
+// the helpers' round trip (~6 us) does not hold the chain up.
 template <typename T, int NR>
 struct Cfg;
 template <>
@@ -70,8 +70,8 @@ struct Cfg<float, 4> { static constexpr int LAG = 5, NAUX = 1; };
 template <typename T>
 struct Helper {
   T Ls[HRING][NBK][LDB];  // blocks of L: Ls[slot][k][i] = factor entry (row i, column k)
-  T Ys[KCH][NBK][GR + 1];  // finished rows of Y
-  T red[16][NBK];         // partial sums of the k parts
+  T Ys[KCH][NBK][GR + 4];  // finished rows of Y (padded; four columns load as one vector)
+  T red[16][4][NBK];       // partial sums of the k parts
 };
 template <typename T, int NR>
 struct Leader {
@@ -81,8 +81,8 @@ struct Leader {
   T rinv[RING][NBK];
   T Y[SR][NR][NBK];               // solved blocks
   T P[SR][NR][NBK];               // P_d
-  T Q[SR][NR][NAUX][NBK];         // aux products
-  int y_done[NR], q_done[NR][NAUX], p_done, prep_done[3], load_done[4];
+  T Q[SR][NR][NAUX][NBK];         // P_d minus the products of aux warps NAUX-1 .. a
+  int y_done[NR], q_done[NR][NAUX], p_done, prep_done, load_done[4];
 };
 template <typename T, int NR>
 struct Smem {
@@ -127,7 +127,11 @@ JMG_DEV void cp_async_wait(int n) {
     case 1: asm volatile("cp.async.wait_group 1;" ::: "memory"); break;
     case 2: asm volatile("cp.async.wait_group 2;" ::: "memory"); break;
     case 3: asm volatile("cp.async.wait_group 3;" ::: "memory"); break;
-    default: asm volatile("cp.async.wait_group 4;" ::: "memory"); break;
+    case 4: asm volatile("cp.async.wait_group 4;" ::: "memory"); break;
+    case 5: asm volatile("cp.async.wait_group 5;" ::: "memory"); break;
+    case 6: asm volatile("cp.async.wait_group 6;" ::: "memory"); break;
+    case 7: asm volatile("cp.async.wait_group 7;" ::: "memory"); break;
+    default: asm volatile("cp.async.wait_group 8;" ::: "memory"); break;
   }
 }
 
@@ -158,18 +162,18 @@ JMG_DEV int wait_gt(const int* p, int d, int* err, int* info, SM& S, uint64_t li
   return have;
 }
 
-// Bounded spin of a warp on a counter in shared memory until it is >= want;
-// false on abort or expiry.
+// Bounded spin of a warp on a counter in shared memory (each lane its own p, or all
+// the same) until every one is >= want; false, on every lane, on abort or expiry.
 template <typename SM>
 JMG_DEV bool wait_sm(const int* p, int want, int* err, int* info, SM& S, uint64_t limit_ns) {
-  if (ld_acquire_sm(p) >= want) return true;
+  if (__all_sync(0xffffffffu, ld_acquire_sm(p) >= want)) return true;
   const uint64_t t0 = globaltimer_ns();
   while (true) {
 #pragma unroll 1
     for (int i = 0; i < 64; ++i)
-      if (ld_acquire_sm(p) >= want) return true;
-    if (ld_shared_volatile(&S.abort)) return false;
-    if (globaltimer_ns() - t0 > limit_ns) {
+      if (__all_sync(0xffffffffu, ld_acquire_sm(p) >= want)) return true;
+    if (__any_sync(0xffffffffu, ld_shared_volatile(&S.abort))) return false;
+    if (__any_sync(0xffffffffu, globaltimer_ns() - t0 > limit_ns)) {
       give_up(err, info, S);
       return false;
     }
@@ -200,6 +204,18 @@ JMG_DEV void copy_block(T (*dst)[LDB], const T* L, int lda, int n, int bd, int b
     else
       q[u * qs] = T(0);
   }
+}
+
+// sum_k Lo[k][lane] y[k] over one block, in four sums (a dependent FP64 FMA waits
+// for 68 clocks, an independent one 16)
+template <typename T>
+JMG_DEV T block_dot(const T (*Lo)[LDB], const T* y, int lane) {
+  T a[4] = {T(0), T(0), T(0), T(0)};
+#pragma unroll
+  for (int k = 0; k < NBK; k += 4)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) a[q] = fma(Lo[k + q][lane], y[k + q], a[q]);
+  return (a[0] + a[1]) + (a[2] + a[3]);
 }
 }  // namespace trsv
 
@@ -240,9 +256,8 @@ __global__ void __launch_bounds__(trsv::TH, 1)
     int* my_cnt = cnt + S.ticket;
     if (t < NR) M.y_done[t] = 0;
     if (t < NR * NAUX) (&M.q_done[0][0])[t] = 0;
-    if (t < 3) M.prep_done[t] = 0;
+    if (t == 0) M.p_done = M.prep_done = 0;
     if (t < 4) M.load_done[t] = 0;
-    if (t == 0) M.p_done = 0;
     __syncthreads();
     auto wsm = [&](const int* p, int want) { return wait_sm(p, want, err, info, S, wait_ns); };
     auto signal = [&](int* p, int v) {
@@ -250,30 +265,27 @@ __global__ void __launch_bounds__(trsv::TH, 1)
       if (lane == 0) st_release_sm(p, v);
     };
     constexpr int AUX0 = NR == 1 ? 1 : 4;   // first aux warp: (column, part)
-    constexpr int PREP0 = NR == 1 ? 5 : 10;  // first prep warp
-    constexpr int NPREP = NR == 1 ? 3 : 2;
+    constexpr int PREP = 10, LOAD0 = 12;
+    // 1 / x: FP64 on the integer pipe, off the one the chain uses
+    auto inverse = [](T x) -> T {
+      if constexpr (sizeof(T) == 8) {
+        bool bad = false;
+        const T r = pivot_rcp(x < T(0) ? -x : x, &bad);
+        return x < T(0) ? -r : r;
+      } else {
+        return T(1) / x;
+      }
+    };
     if (warp < NR) {
       // ---- chain warp of right-hand side c0 + warp
       const int c = warp;
       if (c < ncol) {
         for (int d = 0; d < nblk; ++d) {
           const int b = blk(d), rows = min(NBK, n - b * NBK), slot = d % RING;
-          if (!wsm(&M.p_done, d + 1)) break;
-          T s = M.P[d % SR][c][lane];
-          bool ok = true;
-#pragma unroll
-          for (int a = 0; a < NAUX; ++a) {
-            if (d < 2 + a) continue;  // that part starts at block d - 2 - a
-            ok = ok && wsm(&M.q_done[c][a], d + 1);
-            s -= M.Q[d % SR][c][a][lane];
-          }
-          for (int w = 0; w < NPREP; ++w) ok = ok && wsm(&M.prep_done[w], d + 1);
-          if (!ok) break;
+          if (!wsm(&M.prep_done, d + 1) || !wsm(&M.q_done[c][0], d + 1)) break;
+          T s = M.Q[d % SR][c][0][lane];
           if (d >= 1) {
-            const T* y = M.Y[(d - 1) % SR][c];
-            const T(*Lo)[LDB] = M.Lo[slot][0];
-#pragma unroll
-            for (int k = 0; k < NBK; ++k) s = fma(-Lo[k][lane], y[k], s);
+            s -= block_dot<T>(M.Lo[slot][0], M.Y[(d - 1) % SR][c], lane);
           }
           const T(*Ld)[LDB] = M.Ld[slot];
 #pragma unroll
@@ -288,54 +300,52 @@ __global__ void __launch_bounds__(trsv::TH, 1)
         }
       }
     } else if (warp >= AUX0 && warp < AUX0 + NR * NAUX) {
-      // ---- aux warp: products with blocks d-2-a, d-2-a-NAUX, ... of column c
+      // ---- aux warp a of column c: products with blocks d-2-a, d-2-a-NAUX, ...; the
+      // warps pass P_d minus what has been multiplied so far from the last one (the
+      // oldest blocks) to the first, and that to the chain
       const int c = (warp - AUX0) % NR, a = (warp - AUX0) / NR;
       if (c < ncol) {
-        for (int d = 2 + a; d < nblk; ++d) {
+        for (int d = 0; d < nblk; ++d) {
+          if (!wsm(&M.load_done[lane & 3], d + 1)) break;  // every loader's part
           T s = T(0);
           bool ok = true;
-          // oldest block first; the newest (e = 2 + a) last
           constexpr int NE = (LAG - 2 + NAUX - 1) / NAUX;
-          for (int w = 0; w < 4; ++w) ok = ok && wsm(&M.load_done[w], d + 1);
-          if (!ok) break;
 #pragma unroll
-          for (int q = NE - 1; q >= 0; --q) {
+          for (int q = NE - 1; q >= 0; --q) {  // the newest block last
             const int e = 2 + a + q * NAUX;
             if (e >= LAG || d - e < 0) continue;
             if (!wsm(&M.y_done[c], d - e + 1)) {
               ok = false;
               break;
             }
-            const T* y = M.Y[(d - e) % SR][c];
-            const T(*Lo)[LDB] = M.Lo[d % RING][e - 1];
-#pragma unroll
-            for (int k = 0; k < NBK; ++k) s = fma(Lo[k][lane], y[k], s);
+            s -= block_dot<T>(M.Lo[d % RING][e - 1], M.Y[(d - e) % SR][c], lane);
           }
           if (!ok) break;
+          if (a == NAUX - 1) {
+            if (!wsm(&M.p_done, d + 1)) break;
+            s += M.P[d % SR][c][lane];
+          } else {
+            if (!wsm(&M.q_done[c][a + 1], d + 1)) break;
+            s += M.Q[d % SR][c][a + 1][lane];
+          }
           M.Q[d % SR][c][a][lane] = s;
           signal(&M.q_done[c][a], d + 1);
         }
       }
-    } else if (warp >= PREP0 && warp < PREP0 + NPREP) {
+    } else if (warp == PREP) {
       // ---- prep warp: 1 / L_ii and the scaled columns of the diagonal block
-      const int w0 = warp - PREP0;
       for (int d = 0; d < nblk; ++d) {
         const int slot = d % RING, rows = min(NBK, n - blk(d) * NBK);
-        bool ok = true;
-        for (int w = 0; w < 4; ++w) ok = ok && wsm(&M.load_done[w], d + 1);
-        if (!ok) break;
+        if (!wsm(&M.load_done[lane & 3], d + 1)) break;  // every loader's part
         T(*Ld)[LDB] = M.Ld[slot];
-        const T r = lane < rows ? T(1) / Ld[lane][lane] : T(0);
-        __syncwarp();
-        if (w0 == 0) M.rinv[slot][lane] = r;
-#pragma unroll
-        for (int q = 0; q < (NBK + NPREP - 1) / NPREP; ++q) {
-          const int i = w0 + q * NPREP;
-          if (i >= NBK) break;
+        const T r = lane < rows ? inverse(Ld[lane][lane]) : T(0);
+        M.rinv[slot][lane] = r;
+#pragma unroll 8
+        for (int i = 0; i < NBK - 1; ++i) {
           const T ri = __shfl_sync(0xffffffffu, r, i);
           if (lane > i) Ld[i][lane] *= ri;
         }
-        signal(&M.prep_done[w0], d + 1);
+        signal(&M.prep_done, d + 1);
       }
     } else if (warp == 8) {
       // ---- fetching warp: P_d (after its flag) into P[d % SR]
@@ -371,14 +381,14 @@ __global__ void __launch_bounds__(trsv::TH, 1)
         }
         __syncwarp();
       }
-    } else if (warp >= 12) {
+    } else if (warp >= LOAD0) {
       // ---- loaders: step d's blocks of L into slot d % RING, two steps in flight
       for (int d = 0; d <= nblk; ++d) {
         if (d < nblk) {
           bool ok = true;
           for (int c = 0; c < ncol; ++c) ok = ok && wsm(&M.y_done[c], d - RING + 1);
           if (!ok) break;
-          const int b = blk(d), slot = d % RING, w = warp - 12;
+          const int b = blk(d), slot = d % RING, w = warp - LOAD0;
           copy_block<4, true>(M.Ld[slot], L, lda, n, b, b, trans, w, lane);
 #pragma unroll 1
           for (int e = 1; e < LAG; ++e)
@@ -388,7 +398,7 @@ __global__ void __launch_bounds__(trsv::TH, 1)
         }
         if (d >= 1) {
           cp_async_wait(d < nblk ? 1 : 0);  // step d-1 has landed
-          signal(&M.load_done[warp - 12], d);
+          signal(&M.load_done[warp - LOAD0], d);
         }
       }
       cp_async_wait(0);  // nothing of ours may land after the CTA ends
@@ -399,9 +409,12 @@ __global__ void __launch_bounds__(trsv::TH, 1)
   // ================================================================ helpers
   Helper<T>& H = S.h;
   const int c0 = grp * GR;
-  int nrp = 1;  // right-hand sides, rounded up to a power of two
-  while (nrp < ncol_g) nrp *= 2;
-  const int hc = warp % nrp, part = warp / nrp, parts = 16 / nrp, kper = NBK / parts;
+  // a warp multiplies tq right-hand sides (4, or 2 or 1 of a narrow group) with its
+  // part of the 32 columns of a block: one value of L feeds tq products
+  const int tq = ncol_g > 2 ? 4 : ncol_g, nq = cdiv_dev(ncol_g, tq);
+  int nqp = 1;
+  while (nqp < nq) nqp *= 2;
+  const int hq = warp % nqp, part = warp / nqp, parts = 16 / nqp, kper = NBK / parts;
   while (true) {
     const int d = LAG + S.ticket - NL;  // block (in dependency order) of this ticket
     if (d >= nblk) break;
@@ -411,7 +424,7 @@ __global__ void __launch_bounds__(trsv::TH, 1)
       copy_block<16, false>(H.Ls[j % HRING], L, lda, n, b, blk(j), trans, warp, lane);
       cp_async_commit();
     };
-    T acc = T(0);
+    T acc[4] = {T(0), T(0), T(0), T(0)};
     int pfd = 0;  // blocks of L issued
     for (; pfd < min(ndep, HRING - KCH); ++pfd) issue_L(pfd);
     for (int j = 0; j < ndep;) {
@@ -441,10 +454,21 @@ __global__ void __launch_bounds__(trsv::TH, 1)
       __syncthreads();
       for (int q = 0; q < ready - j; ++q) {
         const T(*Lq)[LDB] = H.Ls[(j + q) % HRING];
-        const T(*Yq)[GR + 1] = H.Ys[q];
+        const T(*Yq)[GR + 4] = H.Ys[q];
+        if (tq == 4) {
 #pragma unroll 8
-        for (int k = part * kper; k < (part + 1) * kper; ++k)
-          acc = fma(Lq[k][lane], Yq[k][hc], acc);
+          for (int k = part * kper; k < (part + 1) * kper; ++k) {
+            const T l = Lq[k][lane];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) acc[c] = fma(l, Yq[k][4 * hq + c], acc[c]);
+          }
+        } else {
+          for (int k = part * kper; k < (part + 1) * kper; ++k) {
+            const T l = Lq[k][lane];
+            acc[0] = fma(l, Yq[k][0], acc[0]);
+            if (tq == 2) acc[1] = fma(l, Yq[k][1], acc[1]);
+          }
+        }
       }
       __syncthreads();  // the ring slots and Ys are free again
       j = ready;
@@ -452,11 +476,13 @@ __global__ void __launch_bounds__(trsv::TH, 1)
     cp_async_wait(0);  // no copy of ours may land after the CTA moves on
     if (S.abort) break;
     // P_d over B_d, then the flag
-    H.red[warp][lane] = acc;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) H.red[warp][c][lane] = acc[c];
     __syncthreads();
     if (warp < ncol_g && lane < rows) {
-      T sum = H.red[warp][lane];
-      for (int p = 1; p < parts; ++p) sum += H.red[warp + p * nrp][lane];
+      const int wq = warp / tq, wc = warp % tq;
+      T sum = H.red[wq][wc][lane];
+      for (int p = 1; p < parts; ++p) sum += H.red[wq + p * nqp][wc][lane];
       T* p = &B[(size_t)(c0 + warp) * ldb + row_of(b, rows, lane)];
       *p = __ldcg(p) - sum;
     }
