@@ -122,11 +122,10 @@ void jmg_default_options(jmg_options* opt);
 size_t jmg_workspace_size(int op, int n, int nrhs, int dtype, const jmg_options* opt);
 
 /* Bytes of `work` with which the same call takes its fastest route: never less
- * than jmg_workspace_size().  More than that only for the plain calls with a
- * factorisation (potrf, posv and posv_host, prec NATIVE, n > 64, FP32 n > 2560), whose trailing
- * updates then run on the tensor cores in error-free slices (about 8.1 KB per row of
- * A in FP64, 4.6 KB in FP32), with a 256-byte aligned `work`; with less, they run on
- * the CUDA cores. */
+ * than jmg_workspace_size().  More than that only for the plain FP64 calls with a
+ * factorisation (potrf, posv and posv_host, prec NATIVE), whose trailing updates
+ * then run on the tensor cores in error-free slices (about 7.2 KB per row of A),
+ * with a 256-byte aligned `work`; with less, they run on the FP64 CUDA cores. */
 size_t jmg_workspace_fast(int op, int n, int nrhs, int dtype, const jmg_options* opt);
 
 /*
@@ -135,12 +134,12 @@ size_t jmg_workspace_fast(int op, int n, int nrhs, int dtype, const jmg_options*
  *   n       order of A (n >= 0; n == 0 is a no-op)
  *   A       device, lower(A) in, lower(L) out; lda >= max(1, n)
  *   dtype   JMG_F64, or JMG_F32 (FP32 storage: FP32 panel solves and trailing
- *           updates; the diagonal blocks are factored in FP64
+ *           updates on the CUDA cores; the diagonal blocks are factored in FP64
  *           arithmetic and rounded to FP32)
  *   info    device int, written asynchronously (see above); may not be NULL
  *   opt     NULL or options (prec must be NATIVE)
  *   work    may be NULL when jmg_workspace_size(JMG_OP_POTRF, ...) is 0;
- *           jmg_workspace_fast(JMG_OP_POTRF, ...) bytes take the fastest route
+ *           jmg_workspace_fast(JMG_OP_POTRF, ...) bytes make FP64 fast
  * Asynchronous: returns once the kernels are queued on `stream`.
  */
 int jmg_potrf(int n, void* A, int lda, int dtype, int* info, const jmg_options* opt,

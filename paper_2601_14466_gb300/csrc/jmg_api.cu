@@ -249,18 +249,15 @@ static int factor_mixed(int n, float* W, int ldw, const jmg_options& o, const Pl
   return sv_prepare(n, W, ldw, at<float>(work, p.off_SV), s);
 }
 
-// Plain factorisation by the scratch at hand: with room for the slices the updates
-// run on the tensor cores, else on the CUDA cores.
+// Plain factorisation by the scratch at hand: FP64 with room for the slices runs
+// its updates on the tensor cores, everything else on the CUDA cores.
 static int potrf_native(int n, void* A, int lda, int dtype, int nb, int* info, void* work,
                         size_t lwork, cudaStream_t s) {
-  const size_t fast = ozf_workspace(n, dtype);
-  const bool split =
-      fast > 0 && work && lwork >= fast && !(reinterpret_cast<uintptr_t>(work) & 255);
-  if (dtype == JMG_F32)
-    return split ? potrf_split<float>(n, (float*)A, lda, info, work, s)
-                 : potrf_plain<float>(n, (float*)A, lda, nb, info, s);
-  return split ? potrf_split<double>(n, (double*)A, lda, info, work, s)
-               : potrf_plain<double>(n, (double*)A, lda, nb, info, s);
+  if (dtype == JMG_F32) return potrf_plain<float>(n, (float*)A, lda, nb, info, s);
+  const size_t fast = ozf_workspace(n);
+  if (fast > 0 && work && lwork >= fast && !(reinterpret_cast<uintptr_t>(work) & 255))
+    return potrf_split(n, (double*)A, lda, info, work, s);
+  return potrf_plain<double>(n, (double*)A, lda, nb, info, s);
 }
 
 // column max of |B| into colmax_r and R = B (start of refinement from X = 0)
@@ -731,9 +728,9 @@ size_t jmg_workspace_fast(int op, int n, int nrhs, int dtype, const jmg_options*
   jmg_options o;
   opts_or_default(opt, &o);
   const size_t base = jmg_workspace_size(op, n, nrhs, dtype, &o);
-  if (n <= 0 || (dtype != JMG_F64 && dtype != JMG_F32) || o.prec != JMG_PREC_NATIVE) return base;
+  if (n <= 0 || dtype != JMG_F64 || o.prec != JMG_PREC_NATIVE) return base;
   if (op == JMG_OP_POTRF || op == JMG_OP_POSV || op == JMG_OP_POSV_HOST)
-    return round_up(base, 256) + ozf_workspace(n, dtype);
+    return round_up(base, 256) + ozf_workspace(n);
   return base;
 }
 

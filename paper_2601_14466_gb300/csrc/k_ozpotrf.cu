@@ -1,5 +1,5 @@
-// k_ozpotrf.cu -- plain (FP64 and FP32) Cholesky factorisation with its trailing
-// updates on the BF16 tensor cores, by error-free splitting (Ozaki, Ogita, Oishi and Rump 2012,
+// k_ozpotrf.cu -- FP64 Cholesky factorisation with its trailing updates on the
+// BF16 tensor cores, by error-free splitting (Ozaki, Ogita, Oishi and Rump 2012,
 // "Error-free transformations of matrix multiplication by using fast routines of
 // matrix multiplication and its applications").
 //
@@ -22,9 +22,7 @@
 // one update of the block's remaining columns per panel (depth 64) and one of the
 // whole trailing matrix per block (depth 512, sliced again with one exponent per
 // row over the block); the CTA that updates the next diagonal block factors it in
-// the same launch, so a panel is two launches.  FP32 storage takes the same route
-// with S = 4 slices (31 bits of a row's scale, 10 products): its factor's error is
-// 0.63-0.8 of the FP32 CUDA-core route's.  Factor alone on one GB300, FP64
+// the same launch, so a panel is two launches.  Factor alone on one GB300, FP64
 // CUDA-core updates -> here: n = 1024 3.66 -> 1.10 ms, 3000 18.6 -> 3.6, 5000
 // 53 -> 7.1, 16384 1260 -> 66.6 ms (there the tensor cores do 28 products of slices
 // for one of FP64: 620 TFLOP/s over the whole factorisation).  Per panel, small
@@ -37,13 +35,7 @@
 
 namespace jmg {
 namespace ozf {
-// slices per operand: 8 S - 1 bits of the row's scale, past the 53 and 24 of the type
-template <typename T>
-struct Cut;
-template <>
-struct Cut<double> { static constexpr int S = 7; };
-template <>
-struct Cut<float> { static constexpr int S = 4; };
+constexpr int S = 7;           // slices per operand
 constexpr int BM = 128;        // rows of an output tile
 constexpr int BN = 64;         // columns of an output tile
 constexpr int BK = 64;         // K per block: 64 BF16 = one 128-byte swizzle row
@@ -52,48 +44,35 @@ constexpr int ASTAGES = 6;     // ring of row-slice tiles
 constexpr int THREADS = 576;   // warps 0-1 producer / MMA, 2-17 epilogue (16 columns each)
 constexpr int A_TILE = BM * BK * 2;  // 16 KiB
 constexpr int B_TILE = BN * BK * 2;  // 8 KiB
-template <typename T>
-constexpr int SMEM = 2 * Cut<T>::S * B_TILE + ASTAGES * A_TILE + 1024 + 256;
+constexpr int B_BUF = S * B_TILE;
+constexpr int SMEM = 2 * B_BUF + ASTAGES * A_TILE + 1024 + 256;
+constexpr uint32_t TCOLS = 512;      // 7 levels x 64 columns, rounded up
 constexpr int PW = 64;               // panel width
 constexpr int PT = 256;              // threads of the panel solve
 constexpr int GROUP = 8;             // row tiles per raster group
 constexpr int E_BAD = 1 << 20;       // exponent of a row that is not finite
 
-// |x| as an integer that orders like |x|
-JMG_DEV unsigned long long abs_bits(double x) {
-  return (unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull;
-}
-JMG_DEV unsigned long long abs_bits(float x) { return (unsigned)__float_as_int(x) & 0x7FFFFFFFu; }
-JMG_DEV bool sign_bit(double x) { return __double2hiint(x) < 0; }
-JMG_DEV bool sign_bit(float x) { return __float_as_int(x) < 0; }
-
-// exponent e with |x| 2^-e < 1 for every |x| <= m (m given by abs_bits); 0 for
-// m == 0, E_BAD for infinities and NaN.  (Subnormal: m = mb 2^-1074 or mb 2^-149.)
-template <typename T>
+// exponent e with |x| 2^-e < 1 for every |x| <= m (m as the bits of |x|);
+// 0 for m == 0, E_BAD for infinities and NaN
 JMG_DEV int scale_exp_bits(unsigned long long mb) {
-  constexpr bool f64 = sizeof(T) == 8;
   if (mb == 0) return 0;
-  const int ex = (int)(mb >> (f64 ? 52 : 23));
-  if (ex >= (f64 ? 0x7FF : 0xFF)) return E_BAD;
-  if (ex) return ex - (f64 ? 1022 : 126);
-  return (f64 ? -1010 : -85) - __clzll((long long)mb);
+  const int ex = (int)(mb >> 52);
+  if (ex >= 0x7FF) return E_BAD;
+  if (ex) return ex - 1022;
+  return -1010 - __clzll((long long)mb);  // subnormal: m = mb 2^-1074, mb < 2^(64-clz)
 }
 
-// The digits of x 2^-e (|x 2^-e| < 1): V = rint(x 2^(8S-1-e)), |V| <= 2^(8S-1), cut
-// into balanced base-256 digits from the bottom; integer operations only.
-template <typename T, int S = Cut<T>::S>
-JMG_DEV void digits(T x, int e, int (&d)[S]) {
-  constexpr bool f64 = sizeof(T) == 8;
-  constexpr int MB = f64 ? 52 : 23;  // stored significand bits
-  const unsigned long long b = abs_bits(x);
-  int ex = (int)(b >> MB);
-  unsigned long long M = b & ((1ull << MB) - 1);
+// The digits of x 2^-e (|x 2^-e| < 1): V = rint(x 2^(55-e)), |V| <= 2^55, cut into
+// balanced base-256 digits from the bottom; integer operations only.
+JMG_DEV void digits7(double x, int e, int (&d)[S]) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  int ex = (int)((b >> 52) & 0x7FF);
+  unsigned long long M = b & ((1ull << 52) - 1);
   if (ex)
-    M |= 1ull << MB;
+    M |= 1ull << 52;
   else
     ex = 1;
-  // x = M 2^(ex - bias - MB), V = M 2^sh
-  const int sh = ex - (f64 ? 1023 : 127) - MB + 8 * S - 1 - e;
+  const int sh = ex - 1020 - e;  // V = M 2^sh
   unsigned long long V = 0;
   if (sh >= 0) {
     V = sh <= 60 ? M << sh : 0ull;  // (below 2^55 for every finite row; subnormals shift far)
@@ -101,7 +80,7 @@ JMG_DEV void digits(T x, int e, int (&d)[S]) {
     const int k = -sh;
     V = (M >> k) + ((M >> (k - 1)) & 1ull);  // to nearest, ties away
   }
-  long long W = sign_bit(x) ? -(long long)V : (long long)V;
+  long long W = (b >> 63) ? -(long long)V : (long long)V;
 #pragma unroll
   for (int s = S - 1; s >= 1; --s) {
     const int k = (int)(signed char)(W & 255);
@@ -141,12 +120,9 @@ static long long tile_count(int TI, int TJ) {
   return (long long)GROUP * W * gt * (gt + 1) / 2 + (long long)(G - gt) * GROUP * TJ;
 }
 
-// v 2^ex rounded once to T (to nearest even), in integer operations: a conversion
-// holds the FP64 pipe as long as an FMA.
-template <typename T>
-JMG_DEV T scaled_value(long long v, int ex);
-template <>
-JMG_DEV double scaled_value<double>(long long v, int ex) {
+// v 2^ex rounded once to FP64 (to nearest even), in integer operations: a
+// conversion holds the FP64 pipe as long as an FMA.
+JMG_DEV double scaled_double(long long v, int ex) {
   if (v == 0) return 0.0;
   const unsigned long long u = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
   const int lz = __clzll((long long)u);
@@ -160,21 +136,8 @@ JMG_DEV double scaled_value<double>(long long v, int ex) {
   const unsigned long long bits = ((unsigned long long)(E - 1) << 52) + q;
   return __longlong_as_double((long long)(bits | ((unsigned long long)v & (1ull << 63))));
 }
-template <>
-JMG_DEV float scaled_value<float>(long long v, int ex) {
-  if (v == 0) return 0.0f;
-  const unsigned long long u = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
-  const int lz = __clzll((long long)u);
-  const unsigned long long m = u << lz;
-  const int E = 190 - lz + ex;
-  if (E < 1 || E > 253) return (float)ldexp((double)v, ex);
-  unsigned q = (unsigned)(m >> 40);
-  const unsigned long long rem = m & ((1ull << 40) - 1), half = 1ull << 39;
-  q += (rem > half || (rem == half && (q & 1))) ? 1 : 0;
-  const unsigned bits = ((unsigned)(E - 1) << 23) + q;
-  return __uint_as_float(bits | (v < 0 ? 0x80000000u : 0u));
-}
 
+// ---------------------------------------------------------------------------
 // Diagonal block of kb <= 64 columns, in place, by one CTA of THREADS threads.  An
 // FP64 warp instruction holds its SM quarter's pipe for ~64 clocks, and the pivots
 // are a serial chain: warp 0 keeps column j in registers (two rows per lane) and in
@@ -202,8 +165,7 @@ JMG_DEV void bar_arrive(int id, int count) {
   asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(count) : "memory");
 }
 
-template <typename T>
-JMG_DEV void diag_body(double* sm_d64, T* __restrict__ A, int lda, int kb, int koff,
+JMG_DEV void diag_body(double* sm_d64, double* __restrict__ A, int lda, int kb, int koff,
                        int* __restrict__ info) {
   using namespace diag64;
   constexpr int TH = THREADS;
@@ -219,16 +181,16 @@ JMG_DEV void diag_body(double* sm_d64, T* __restrict__ A, int lda, int kb, int k
   if (fail != 0) return;  // an earlier block already failed
   {
     constexpr int Q = (PW * PW + TH - 1) / TH;
-    T v[Q];
+    double v[Q];
 #pragma unroll
     for (int q = 0; q < Q; ++q) {  // all loads first
       const int idx = t + TH * q, r = idx % PW, c = idx / PW;
-      v[q] = (idx < PW * PW && r < kb && c <= r) ? A[(size_t)c * lda + r] : T(0);
+      v[q] = (idx < PW * PW && r < kb && c <= r) ? A[(size_t)c * lda + r] : 0.0;
     }
 #pragma unroll
     for (int q = 0; q < Q; ++q) {
       const int idx = t + TH * q;
-      if (idx < PW * PW) s64[(idx / PW) * LD + idx % PW] = (double)v[q];
+      if (idx < PW * PW) s64[(idx / PW) * LD + idx % PW] = v[q];
     }
   }
   for (int c = warp; c < PW; c += TH / 32) {
@@ -315,17 +277,15 @@ JMG_DEV void diag_body(double* sm_d64, T* __restrict__ A, int lda, int kb, int k
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int r = lane + 32 * h;
-      if (r >= c && r < kb)
-        A[(size_t)c * lda + r] = (T)(r == c ? s_l[c] : s64[c * LD + r] * s_il[c]);
+      if (r >= c && r < kb) A[(size_t)c * lda + r] = r == c ? s_l[c] : s64[c * LD + r] * s_il[c];
     }
   if (t == 0 && fail) atomicCAS(info, 0, koff + fail);
 }
 
-template <typename T>
-__global__ void __launch_bounds__(THREADS) k_oz_diag(T* __restrict__ A, int lda, int kb, int koff,
-                                                     int* __restrict__ info) {
+__global__ void __launch_bounds__(THREADS) k_oz_diag(double* __restrict__ A, int lda, int kb,
+                                                     int koff, int* __restrict__ info) {
   extern __shared__ __align__(16) double sm_diag64[];
-  diag_body<T>(sm_diag64, A, lda, kb, koff, info);
+  diag_body(sm_diag64, A, lda, kb, koff, info);
 }
 
 // ---------------------------------------------------------------------------
@@ -333,15 +293,12 @@ __global__ void __launch_bounds__(THREADS) k_oz_diag(T* __restrict__ A, int lda,
 // P P^T, P given by its slices: row r of slice s is row s * n + r of the map.  CTA 0
 // takes tile 0 alone and then factors the diagonal block it has just updated (kb
 // columns), while the others work through the rest of the update.
-template <typename T>
 __global__ void __launch_bounds__(THREADS, 1)
     k_oz_syrk(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-              T* __restrict__ C, int ldc, int n, int r0, int ncols, int nkb,
+              double* __restrict__ C, int ldc, int n, int r0, int ncols, int nkb,
               const int* __restrict__ ex, int TI, int TJ, int ntiles, int kb_diag,
               int* __restrict__ info, unsigned long long wait_ns) {
   using namespace tc;
-  constexpr int S = Cut<T>::S, B_BUF = S * B_TILE;
-  constexpr uint32_t TCOLS = S * BN <= 256 ? 256 : 512;
   extern __shared__ __align__(1024) unsigned char sm_raw_ozf[];
   unsigned char* smem = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(sm_raw_ozf) + 1023) & ~uintptr_t(1023));
@@ -483,13 +440,11 @@ __global__ void __launch_bounds__(THREADS, 1)
     }
   } else {
     // epilogue: warp w reads TMEM lane group q = w % 4 and 16 columns of every
-    // level.  acc holds sum_d level_d 2^(SH - 8 d): FP32, SH = 24, exactly; FP64, SH
-    // fractional bits chosen so that K products of at most 2^14 stay below 2^62, the
-    // last two levels rounded to them once per window.
+    // level.  acc holds sum_d level_d 2^(SH - 8 d), SH fractional bits chosen so
+    // that K products of at most 2^14 stay below 2^62.
     constexpr int CW = 16;
-    constexpr int DX = S == 7 ? 5 : S;  // levels added exactly
     const int q = warp & 3, ch = ((warp - 2) >> 2) * CW;
-    const int sh = S == 4 ? 24 : (nkb * BK <= 256 ? 40 : (nkb * BK <= 512 ? 39 : 38));
+    const int sh = nkb * BK <= 256 ? 40 : (nkb * BK <= 512 ? 39 : 38);
     const long long half = 1ll << (47 - sh);
     long long gw = 0;
     bool ok = true;
@@ -511,21 +466,16 @@ __global__ void __launch_bounds__(THREADS, 1)
         tc_fence_after();
         const uint32_t tacc = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)ch;
 #pragma unroll
-        for (int d = 0; d < DX; ++d) {
+        for (int d = 0; d < 5; ++d) {
           uint32_t v[16];
           tmem_ld16(tacc + (uint32_t)(d * BN), v);
           tmem_ld_wait();
-          if (d == S - 1) {
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(acce);
-          }
 #pragma unroll
           for (int c = 0; c < CW; ++c)
             acc[c] += (unsigned long long)((long long)__float2int_rn(__uint_as_float(v[c]))
                                            << (sh - 8 * d));
         }
-        if constexpr (DX < S) {
+        {
           uint32_t v[16], w[16];
           tmem_ld16(tacc + (uint32_t)(5 * BN), v);
           tmem_ld16(tacc + (uint32_t)(6 * BN), w);
@@ -546,17 +496,17 @@ __global__ void __launch_bounds__(THREADS, 1)
         break;
       }
       if (jn > 0) {
-        T* cp = C + (size_t)c0 * ldc + row;
+        double* cp = C + (size_t)c0 * ldc + row;
         const int er = ex[row];
-        T old[CW];
+        double old[CW];
 #pragma unroll
-        for (int c = 0; c < CW; ++c) old[c] = c < jn ? cp[(size_t)c * ldc] : T(0);
+        for (int c = 0; c < CW; ++c) old[c] = c < jn ? cp[(size_t)c * ldc] : 0.0;
 #pragma unroll
         for (int c = 0; c < CW; ++c)
           if (c < jn) {
             const int ec = ex[c0 + c];
-            T r = old[c] - scaled_value<T>((long long)acc[c], er + ec - 14 - sh);
-            if (er == E_BAD || ec == E_BAD) r = (T)__longlong_as_double(0x7FF8000000000000ll);
+            double r = old[c] - scaled_double((long long)acc[c], er + ec - 14 - sh);
+            if (er == E_BAD || ec == E_BAD) r = __longlong_as_double(0x7FF8000000000000ll);
             cp[(size_t)c * ldc] = r;
           }
       }
@@ -578,7 +528,7 @@ __global__ void __launch_bounds__(THREADS, 1)
   if (warp == 1) tmem_dealloc(tmem, TCOLS);
   if (blockIdx.x == 0 && !ld_shared_volatile(&s_fail)) {
     __syncthreads();  // tile 0 is in global memory, the rings are idle
-    diag_body<T>(reinterpret_cast<double*>(smem), C + (size_t)r0 * ldc + r0, ldc, kb_diag, r0, info);
+    diag_body(reinterpret_cast<double*>(smem), C + (size_t)r0 * ldc + r0, ldc, kb_diag, r0, info);
   }
 }
 
@@ -590,8 +540,8 @@ __global__ void __launch_bounds__(THREADS, 1)
 // quarter left half the issue slots to instruction-fetch and latency stalls).  The solve runs on unscaled columns
 // with Lh[j][l] = L_lj / L_jj (a_l -= a_j Lh[j][l]), the scaling by 1 / L_jj
 // comes last: one FP64 instruction per element and step, nothing else.
-template <typename T, int G>
-__global__ void __launch_bounds__(PT) k_oz_panel(T* __restrict__ A, int lda, int n, int k,
+template <int G>
+__global__ void __launch_bounds__(PT) k_oz_panel(double* __restrict__ A, int lda, int n, int k,
                                                   __nv_bfloat16* __restrict__ SP,
                                                   int* __restrict__ ex,
                                                   unsigned long long* __restrict__ rowmax,
@@ -599,36 +549,32 @@ __global__ void __launch_bounds__(PT) k_oz_panel(T* __restrict__ A, int lda, int
   constexpr int NP = 32 / G;     // column pairs per lane
   constexpr int RW = 32 / G;     // rows per warp
   constexpr int RB = PT / 32 * RW;  // rows per CTA
-  constexpr int S = Cut<T>::S;
-  struct alignas(2 * sizeof(T)) Pair {
-    T x, y;
-  };
-  __shared__ __align__(16) T Lh[PW * PW];
-  __shared__ T rinv[PW];
+  __shared__ __align__(16) double Lh[PW * PW];
+  __shared__ double rinv[PW];
   if (*(volatile const int*)info != 0) return;
   const int t = threadIdx.x, lane = t % 32, warp = t / 32;
-  const T* Lkk = A + (size_t)k * lda + k;
+  const double* Lkk = A + (size_t)k * lda + k;
   {
     constexpr int Q = PW * PW / PT;
-    T v[Q];
+    double v[Q];
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
       const int idx = t + PT * i, l = idx % PW, j = idx / PW;
-      v[i] = l >= j ? Lkk[(size_t)j * lda + l] : T(0);
+      v[i] = l >= j ? Lkk[(size_t)j * lda + l] : 0.0;
     }
 #pragma unroll
     for (int i = 0; i < Q; ++i) Lh[t + PT * i] = v[i];
   }
   const int g = lane % G, rl = warp * RW + lane / G;
   const int row = k + PW + blockIdx.x * RB + rl;
-  T x[2 * NP];
+  double x[2 * NP];
 #pragma unroll
   for (int i = 0; i < NP; ++i)
 #pragma unroll
     for (int h = 0; h < 2; ++h)
-      x[2 * i + h] = row < n ? A[(size_t)(k + 2 * (g + G * i) + h) * lda + row] : T(0);
+      x[2 * i + h] = row < n ? A[(size_t)(k + 2 * (g + G * i) + h) * lda + row] : 0.0;
   __syncthreads();
-  if (t < PW) rinv[t] = T(1) / Lh[t * PW + t];
+  if (t < PW) rinv[t] = 1.0 / Lh[t * PW + t];
   __syncthreads();
 #pragma unroll 4
   for (int i = 0; i < PW * PW / PT; ++i) {
@@ -639,11 +585,11 @@ __global__ void __launch_bounds__(PT) k_oz_panel(T* __restrict__ A, int lda, int
 #pragma unroll
   for (int j = 0; j < PW; ++j) {
     const int go = (j / 2) % G, io = (j / 2) / G;  // owner lane and register of column j
-    const T aj = __shfl_sync(0xffffffffu, x[2 * io + (j & 1)], go, G);
+    const double aj = G == 1 ? x[j] : __shfl_sync(0xffffffffu, x[2 * io + (j & 1)], go, G);
 #pragma unroll
     for (int i = 0; i < NP; ++i) {
       if (2 * (G - 1 + G * i) + 1 <= j) continue;  // every lane's pair is done
-      const Pair l2 = *reinterpret_cast<const Pair*>(&Lh[j * PW + 2 * (g + G * i)]);
+      const double2 l2 = *reinterpret_cast<const double2*>(&Lh[j * PW + 2 * (g + G * i)]);
       const int l = 2 * (g + G * i);
       if (l > j) x[2 * i] = fma(-aj, l2.x, x[2 * i]);
       if (l + 1 > j) x[2 * i + 1] = fma(-aj, l2.y, x[2 * i + 1]);
@@ -657,7 +603,8 @@ __global__ void __launch_bounds__(PT) k_oz_panel(T* __restrict__ A, int lda, int
       const int c = 2 * (g + G * i) + h;
       x[2 * i + h] *= rinv[c];
       if (row < n) A[(size_t)(k + c) * lda + row] = x[2 * i + h];
-      const unsigned long long b = abs_bits(x[2 * i + h]);
+      const unsigned long long b =
+          (unsigned long long)__double_as_longlong(x[2 * i + h]) & 0x7FFFFFFFFFFFFFFFull;
       mx = b > mx ? b : mx;
     }
 #pragma unroll
@@ -666,7 +613,7 @@ __global__ void __launch_bounds__(PT) k_oz_panel(T* __restrict__ A, int lda, int
     mx = b > mx ? b : mx;
   }
   if (row >= n) return;
-  const int e = scale_exp_bits<T>(mx);
+  const int e = scale_exp_bits(mx);
   if (g == 0) {
     ex[row] = e;
     rowmax[row] = first ? mx : (mx > rowmax[row] ? mx : rowmax[row]);
@@ -674,8 +621,8 @@ __global__ void __launch_bounds__(PT) k_oz_panel(T* __restrict__ A, int lda, int
 #pragma unroll
   for (int i = 0; i < NP; ++i) {
     int d0[S], d1[S];
-    digits<T>(x[2 * i], e, d0);
-    digits<T>(x[2 * i + 1], e, d1);
+    digits7(x[2 * i], e, d0);
+    digits7(x[2 * i + 1], e, d1);
 #pragma unroll
     for (int s = 0; s < S; ++s) {
       const __nv_bfloat162 p = __floats2bfloat162_rn((float)d0[s], (float)d1[s]);
@@ -686,39 +633,37 @@ __global__ void __launch_bounds__(PT) k_oz_panel(T* __restrict__ A, int lda, int
 
 // Slices of the finished block column k0 .. k0 + K - 1 (rows from r0 on) with one
 // exponent per row over the whole block.  grid = (32-row tiles, K / 64).
-template <typename T>
-__global__ void __launch_bounds__(256) k_oz_strip(const T* __restrict__ A, int lda, int n,
+__global__ void __launch_bounds__(256) k_oz_strip(const double* __restrict__ A, int lda, int n,
                                                   int k0, int r0, int K,
                                                   const unsigned long long* __restrict__ rowmax,
                                                   __nv_bfloat16* __restrict__ SP,
                                                   int* __restrict__ ex,
                                                   const int* __restrict__ info) {
-  constexpr int S = Cut<T>::S;
-  __shared__ T Ts[64][33];
+  __shared__ double T[64][33];
   if (*(volatile const int*)info != 0) return;
   const int t = threadIdx.x;
   const int rb = r0 + blockIdx.x * 32, kc = blockIdx.y * 64;
   {
-    T v[8];
+    double v[8];
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
       const int r = rb + t % 32, c = t / 32 + 8 * q;
-      v[q] = r < n ? A[(size_t)(k0 + kc + c) * lda + r] : T(0);
+      v[q] = r < n ? A[(size_t)(k0 + kc + c) * lda + r] : 0.0;
     }
 #pragma unroll
-    for (int q = 0; q < 8; ++q) Ts[t / 32 + 8 * q][t % 32] = v[q];
+    for (int q = 0; q < 8; ++q) T[t / 32 + 8 * q][t % 32] = v[q];
   }
   __syncthreads();
   const int rr = t / 8, cc = 8 * (t % 8), row = rb + rr;
   if (row >= n) return;
-  const int e = scale_exp_bits<T>(rowmax[row]);
+  const int e = scale_exp_bits(rowmax[row]);
   if (kc == 0 && cc == 0) ex[row] = e;
   uint32_t w[S][4];
 #pragma unroll
   for (int u = 0; u < 4; ++u) {
     int d0[S], d1[S];
-    digits<T>(Ts[cc + 2 * u][rr], e, d0);
-    digits<T>(Ts[cc + 2 * u + 1][rr], e, d1);
+    digits7(T[cc + 2 * u][rr], e, d0);
+    digits7(T[cc + 2 * u + 1][rr], e, d1);
 #pragma unroll
     for (int s = 0; s < S; ++s) {
       const __nv_bfloat162 p = __floats2bfloat162_rn((float)d0[s], (float)d1[s]);
@@ -731,7 +676,7 @@ __global__ void __launch_bounds__(256) k_oz_strip(const T* __restrict__ A, int l
         make_uint4(w[s][0], w[s][1], w[s][2], w[s][3]);
 }
 
-static int map_slices(CUtensorMap* map, const void* base, int S, int n, int K, int box_rows) {
+static int map_slices(CUtensorMap* map, const void* base, int n, int K, int box_rows) {
   return make_tmap_2d(map, base, (unsigned long long)K, (unsigned long long)S * n,
                       (unsigned long long)K * 2, BK, (unsigned)box_rows,
                       CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, CU_TENSOR_MAP_SWIZZLE_128B);
@@ -746,7 +691,7 @@ struct OzfPlan {
   int NB;
   size_t panel, strip, exp_in, exp_out, rowmax, total;
 };
-OzfPlan ozf_plan(int n, int S) {
+OzfPlan ozf_plan(int n) {
   OzfPlan p{};
   p.NB = (int)std::min<size_t>(512, round_up((size_t)n, ozf::PW));
   size_t off = 0;
@@ -755,8 +700,8 @@ OzfPlan ozf_plan(int n, int S) {
     off = round_up(off + b, 256);
     return at;
   };
-  p.panel = take((size_t)S * n * ozf::PW * 2);
-  p.strip = take(n > p.NB ? (size_t)S * n * p.NB * 2 : 0);
+  p.panel = take((size_t)ozf::S * n * ozf::PW * 2);
+  p.strip = take(n > p.NB ? (size_t)ozf::S * n * p.NB * 2 : 0);
   p.exp_in = take(sizeof(int) * (size_t)n);
   p.exp_out = take(sizeof(int) * (size_t)n);
   p.rowmax = take(sizeof(unsigned long long) * (size_t)n);
@@ -765,20 +710,11 @@ OzfPlan ozf_plan(int n, int S) {
 }
 }  // namespace
 
-size_t ozf_workspace(int n, int dtype) {
-  // FP64 gains at every size above one panel; FP32 has 64 times the FP64 rate on the
-  // CUDA cores and gains where the update outweighs the panels' chain (factor alone,
-  // CUDA cores / here: n = 2048 1.61 / 1.65 ms, 3000 2.56 / 2.47, 8192 12.5 / 8.8,
-  // 16384 63 / 30)
-  if (n <= (dtype == JMG_F32 ? 2560 : ozf::PW)) return 0;
-  return ozf_plan(n, dtype == JMG_F32 ? ozf::Cut<float>::S : ozf::Cut<double>::S).total;
-}
+size_t ozf_workspace(int n) { return n > ozf::PW ? ozf_plan(n).total : 0; }
 
-template <typename T>
-int potrf_split(int n, T* A, int lda, int* info, void* work, cudaStream_t s) {
+int potrf_split(int n, double* A, int lda, int* info, void* work, cudaStream_t s) {
   using namespace ozf;
-  constexpr int S = Cut<T>::S;
-  const OzfPlan p = ozf_plan(n, S);
+  const OzfPlan p = ozf_plan(n);
   char* w = static_cast<char*>(work);
   __nv_bfloat16* panel = reinterpret_cast<__nv_bfloat16*>(w + p.panel);
   __nv_bfloat16* strip = reinterpret_cast<__nv_bfloat16*>(w + p.strip);
@@ -788,26 +724,26 @@ int potrf_split(int n, T* A, int lda, int* info, void* work, cudaStream_t s) {
   int dev = 0, nsm = 152;
   JMG_CUDA(cudaGetDevice(&dev));
   JMG_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-  JMG_TRY(ensure_smem(k_oz_syrk<T>, SMEM<T>));
-  JMG_TRY(ensure_smem(k_oz_diag<T>, diag64::SMEM));
+  JMG_TRY(ensure_smem(k_oz_syrk, SMEM));
+  JMG_TRY(ensure_smem(k_oz_diag, diag64::SMEM));
   CUtensorMap pa, pb, oa, ob;
-  JMG_TRY(map_slices(&pa, panel, S, n, PW, BM));
-  JMG_TRY(map_slices(&pb, panel, S, n, PW, BN));
+  JMG_TRY(map_slices(&pa, panel, n, PW, BM));
+  JMG_TRY(map_slices(&pb, panel, n, PW, BN));
   if (n > p.NB) {
-    JMG_TRY(map_slices(&oa, strip, S, n, p.NB, BM));
-    JMG_TRY(map_slices(&ob, strip, S, n, p.NB, BN));
+    JMG_TRY(map_slices(&oa, strip, n, p.NB, BM));
+    JMG_TRY(map_slices(&ob, strip, n, p.NB, BN));
   }
   auto update = [&](const CUtensorMap& ma, const CUtensorMap& mb, int r0, int ncols, int nkb,
                     const int* ex) -> int {
     const int TI = cdiv(n - r0, BM), TJ = cdiv(ncols, BN);
     const long long nt = tile_count(TI, TJ);
-    k_oz_syrk<T><<<(int)std::min<long long>(nt, nsm), THREADS, SMEM<T>, s>>>(
+    k_oz_syrk<<<(int)std::min<long long>(nt, nsm), THREADS, SMEM, s>>>(
         ma, mb, A, lda, n, r0, ncols, nkb, ex, TI, TJ, (int)nt, std::min(PW, n - r0), info,
         g_wait_ns);
     return launched();
   };
   // the first diagonal block; every update leaves the next one factored
-  k_oz_diag<T><<<1, THREADS, diag64::SMEM, s>>>(A, lda, std::min(PW, n), 0, info);
+  k_oz_diag<<<1, THREADS, diag64::SMEM, s>>>(A, lda, std::min(PW, n), 0, info);
   JMG_TRY(launched());
   for (int k0 = 0; k0 < n; k0 += p.NB) {
     const int kend = std::min(k0 + p.NB, n);
@@ -815,32 +751,25 @@ int potrf_split(int n, T* A, int lda, int* info, void* work, cudaStream_t s) {
       const int kb = std::min(PW, n - k), m = n - k - kb;
       if (m <= 0) return JMG_OK;
       const int first = k == k0;
-      // lanes per row: FP64, enough rows per pass for the eight warps of every SM; FP32
-      // is not bound by its pipe and keeps more lanes per row longer
-      const int rows = m / (sizeof(T) == 8 ? 1 : 4);
-      auto panel_solve = [&](auto kern, int rb) {
-        kern<<<cdiv(m, rb), PT, 0, s>>>(A, lda, n, k, panel, e_in, rowmax, first, info);
-      };
-      if (rows <= 16 * nsm)
-        panel_solve(k_oz_panel<T, 16>, 16);
-      else if (rows <= 32 * nsm)
-        panel_solve(k_oz_panel<T, 8>, 32);
-      else if (rows <= 64 * nsm)
-        panel_solve(k_oz_panel<T, 4>, 64);
+      // lanes per row: enough rows per pass for the eight warps of every SM
+      if (m <= 16 * nsm)
+        k_oz_panel<16><<<cdiv(m, 16), PT, 0, s>>>(A, lda, n, k, panel, e_in, rowmax, first, info);
+      else if (m <= 32 * nsm)
+        k_oz_panel<8><<<cdiv(m, 32), PT, 0, s>>>(A, lda, n, k, panel, e_in, rowmax, first, info);
+      else if (m <= 64 * nsm)
+        k_oz_panel<4><<<cdiv(m, 64), PT, 0, s>>>(A, lda, n, k, panel, e_in, rowmax, first, info);
       else
-        panel_solve(k_oz_panel<T, 2>, 128);
+        k_oz_panel<2><<<cdiv(m, 128), PT, 0, s>>>(A, lda, n, k, panel, e_in, rowmax, first, info);
       JMG_TRY(launched());
       if (k + PW < kend) JMG_TRY(update(pa, pb, k + PW, kend - (k + PW), 1, e_in));
     }
     if (kend >= n) break;
-    k_oz_strip<T><<<dim3(cdiv(n - kend, 32), p.NB / 64), 256, 0, s>>>(A, lda, n, k0, kend, p.NB,
+    k_oz_strip<<<dim3(cdiv(n - kend, 32), p.NB / 64), 256, 0, s>>>(A, lda, n, k0, kend, p.NB,
                                                                   rowmax, strip, e_out, info);
     JMG_TRY(launched());
     JMG_TRY(update(oa, ob, kend, n - kend, p.NB / 64, e_out));
   }
   return JMG_OK;
 }
-template int potrf_split<double>(int, double*, int, int*, void*, cudaStream_t);
-template int potrf_split<float>(int, float*, int, int*, void*, cudaStream_t);
 
 }  // namespace jmg

@@ -74,12 +74,11 @@ int solve_llt(int n, int nrhs, const T* L, int lda, T* B, int ldb, int* sync, in
   return launch_trsv_persist<T>(n, nrhs, L, lda, B, ldb, 1, sync, info, s);
 }
 
-// ---- plain factorisation with split (Ozaki) updates on the tensor cores (k_ozpotrf.cu)
+// ---- FP64 factorisation with split (Ozaki) updates on the tensor cores (k_ozpotrf.cu)
 // Scratch of potrf_split for order n; 0 when that route does not take n.
-size_t ozf_workspace(int n, int dtype);
-// Cholesky factorisation in place; work: ozf_workspace bytes, 256-byte aligned.
-template <typename T>
-int potrf_split(int n, T* A, int lda, int* info, void* work, cudaStream_t s);
+size_t ozf_workspace(int n);
+// Cholesky factorisation in place; work: ozf_workspace(n) bytes, 256-byte aligned.
+int potrf_split(int n, double* A, int lda, int* info, void* work, cudaStream_t s);
 
 // ---- mixed-precision helpers
 // W (FP32, ldw) <- lower(A) (FP64), lower triangle only; plus shift on the diagonal.

@@ -1,9 +1,9 @@
-"""Plain factorisation with its updates in error-free slices on the tensor cores
+"""FP64 factorisation with its updates in error-free slices on the tensor cores
 (the route of jmg_potrf / jmg_posv when `work` holds jmg_workspace_fast bytes),
 against its input and against the general route, at the edges of its tiles
 (panels of 64 columns, tiles of 128 rows, blocks of 512 columns).
 
-Tolerance (u of the storage type): Cholesky gives |A - L L^T|_ij <= gamma_(n+1) (|L| |L^T|)_ij,
+Tolerance: Cholesky in FP64 gives |A - L L^T|_ij <= gamma_(n+1) (|L| |L^T|)_ij,
 and (|L| |L^T|)_ij <= sqrt(a_ii a_jj); the slices keep 2^-56 of each row's largest
 element of the block, below sqrt(a_ii), and the products left out stay below
 6 * 2^-56 of them, so n u sqrt(a_ii a_jj) covers both: (2 n + 2) u in all.
@@ -21,80 +21,62 @@ from helpers import DEV, U64, host, to_dev_colmajor
 from paper_2601_14466_gb300 import inputs, jmg
 
 
-U32 = 2.0 ** -24
-
-
 def _factor(A: torch.Tensor, route: str, lda=None):
+    view, _ = to_dev_colmajor(A, lda=lda)
     n = A.shape[0]
-    dt = jmg.JMG_F64 if A.dtype == torch.float64 else jmg.JMG_F32
-    buf = torch.full((n, lda or n), float("nan"), dtype=A.dtype, device=DEV)
-    buf[:, :n] = A.t().to(DEV)
-    view = buf.t()[:n]
     info = torch.full((1,), 77, dtype=torch.int32, device=DEV)
     o = jmg.default_options()
     lib = jmg.load()
-    nbytes = int(lib.jmg_workspace_fast(jmg.OP_POTRF, n, 1, dt, ctypes.byref(o)))
+    nbytes = int(lib.jmg_workspace_fast(jmg.OP_POTRF, n, 1, jmg.JMG_F64, ctypes.byref(o)))
     work = torch.empty(max(nbytes, 256), dtype=torch.uint8, device=DEV)
     wp, wl = (work.data_ptr(), nbytes) if route == "split" else (None, 0)
-    st = lib.jmg_potrf(n, view.data_ptr(), view.stride(1), dt, info.data_ptr(),
+    st = lib.jmg_potrf(n, view.data_ptr(), view.stride(1), jmg.JMG_F64, info.data_ptr(),
                        ctypes.byref(o), wp, wl, torch.cuda.current_stream().cuda_stream)
     assert st == 0
     torch.cuda.synchronize()
-    assert torch.isnan(buf[:, n:]).all()  # the padding is never written
     return host(view), int(info.item())
 
 
 def _backward(A: np.ndarray, L: np.ndarray) -> float:
-    L = np.tril(L).astype(np.float64)
+    L = np.tril(L)
     s = np.sqrt(np.diag(A))
-    wide = np.longdouble if A.shape[0] < 1000 else np.float64  # (FP64 suffices against FP32's u)
-    R = (A - (L.astype(wide) @ L.T.astype(wide))) / np.outer(s, s)
+    R = (A - (L.astype(np.longdouble) @ L.T.astype(np.longdouble))) / np.outer(s, s)
     return float(np.max(np.abs(R)))
 
 
-F64, F32 = torch.float64, torch.float32
-
-
 @pytest.mark.gpu
-@pytest.mark.parametrize("n,lda,dtype", [
-    (65, 65, F64), (127, 130, F64), (128, 128, F64), (192, 193, F64), (257, 257, F64),
-    (512, 512, F64), (513, 515, F64), (577, 577, F64), (641, 641, F64),
-    (2561, 2561, F32), (2689, 2691, F32), (3073, 3073, F32)])  # FP32 takes the route above 2560
+@pytest.mark.parametrize("n,lda", [(65, 65), (127, 130), (128, 128), (192, 193), (257, 257),
+                                   (512, 512), (513, 515), (577, 577), (641, 641)])
 @pytest.mark.parametrize("kind", ["gram", "graded", "ones"])
-def test_split_factor_reproduces_its_input(n, lda, kind, dtype):
+def test_split_factor_reproduces_its_input(n, lda, kind):
     A = inputs.gram_shift(n, 1.0, seed=inputs.seed_for("split", n))
     if kind == "graded":  # rows 16 decades apart
         d = torch.logspace(-8, 8, n, dtype=torch.float64)
         A = A * d[:, None] * d[None, :]
     elif kind == "ones":  # every digit of a row of L the same: the largest level sums
         A = torch.ones(n, n, dtype=torch.float64) + torch.eye(n, dtype=torch.float64)
-    A = A.to(dtype)
-    An = A.double().numpy()
+    An = A.numpy()
     Lower = torch.tril(A) + torch.triu(torch.full_like(A, float("nan")), 1)
     L, info = _factor(Lower, "split", lda)
     assert info == 0
     assert np.isnan(L[np.triu_indices(n, 1)]).all()  # the upper triangle is neither read nor written
-    assert _backward(An, L) <= (2 * n + 2) * (U64 if dtype == torch.float64 else U32)
+    assert _backward(An, L) <= (2 * n + 2) * U64
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("n,dtype", [(65, F64), (640, F64), (1100, F64), (2600, F32)])
-def test_split_factor_is_exact_on_integer_factors(n, dtype):
+@pytest.mark.parametrize("n", [65, 640, 1100])
+def test_split_factor_is_exact_on_integer_factors(n):
     Lt, A = inputs.integer_factor(n, seed=3)
-    assert A.abs().max() < 2 ** 24  # exact in either type
-    Lt, A = Lt.to(dtype), A.to(dtype)
     L, info = _factor(A, "split")
     assert info == 0
     np.testing.assert_array_equal(np.tril(L), Lt.numpy())
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("n,k,dtype", [(130, 0, F64), (130, 63, F64), (130, 64, F64), (700, 129, F64),
-                                       (700, 512, F64), (700, 699, F64), (2600, 1, F32),
-                                       (2600, 576, F32), (2600, 2599, F32)])
+@pytest.mark.parametrize("n,k", [(130, 0), (130, 63), (130, 64), (700, 129), (700, 512), (700, 699)])
 @pytest.mark.parametrize("bad", ["negative", "nan", "nan_below"])
-def test_split_factor_reports_the_first_bad_pivot(n, k, bad, dtype):
-    A = inputs.gram_shift(n, 1.0, seed=5).to(dtype)
+def test_split_factor_reports_the_first_bad_pivot(n, k, bad):
+    A = inputs.gram_shift(n, 1.0, seed=5)
     if bad == "negative":
         A[k, k] = -1.0
     elif bad == "nan":
@@ -133,10 +115,9 @@ def test_fast_scratch_is_never_less_and_only_more_where_it_helps():
                      ("fp32", jmg.JMG_F64)):
         o = jmg.default_options(prec=prec)
         for op in (jmg.OP_POTRF, jmg.OP_POTRS, jmg.OP_POSV, jmg.OP_POSV_HOST):
-            for n in (0, 1, 64, 65, 1000, 2560, 2561, 65536):
+            for n in (0, 1, 64, 65, 1000, 65536):
                 need = jmg.workspace_size(op, n, 3, o, dt)
                 fast = int(lib.jmg_workspace_fast(op, n, 3, dt, ctypes.byref(o)))
                 assert fast >= need
-                least = 64 if dt == jmg.JMG_F64 else 2560
-                more = prec == "fp64" and n > least and op != jmg.OP_POTRS
+                more = prec == "fp64" and dt == jmg.JMG_F64 and n > 64 and op != jmg.OP_POTRS
                 assert (fast > need + 255) == more
