@@ -1,4 +1,4 @@
-// k_trsv.cu -- blocked triangular solves with the Cholesky factor, one launch
+// k_trsv.cu -- blocked triangular solves with an FP64 Cholesky factor, one launch
 // per direction (paper: "Software design", the solve step of potrs):
 //
 //   forward   L Y = B :  Y_b = L_bb^{-1} (B_b - sum_{j<b} L_bj Y_j)
@@ -24,13 +24,11 @@
 // form the products with blocks d-2 .. d-LAG+1 beforehand, prep warps scale the
 // diagonal blocks, loaders bring L through a four-step ring, and a fetching and
 // a publishing warp keep global round trips off the chain.  The roles meet
-// through counters in shared memory, no CTA-wide barrier.  A step takes 3.9 us in
-// FP64 and 1.8 us in FP32 up to 16 right-hand sides (28-32 us and 3.6 us with one
-// lane per right-hand side substituting and barriers between the phases): both
-// directions at n = 12288, 8 right-hand sides, FP64, 24.3 -> 3.6 ms; n = 8192, 16,
-// FP32, 1.90 -> 0.92 ms.  From 32 right-hand sides on FP64 is bound by the
-// helpers' products (n = 16384, 64: 35.1 ms, 0.98 TFLOP/s of 1.1).  FP32 at
-// n = 16384, 64 right-hand sides is the one measured shape that lost: 4.35 -> 4.49 ms.
+// through counters in shared memory, no CTA-wide barrier.  A step takes 3.9 us up to
+// 16 right-hand sides (28-32 us with one lane per right-hand side substituting and
+// barriers between the phases): both directions at n = 12288, 8 right-hand sides,
+// 24.3 -> 3.6 ms.  From 32 right-hand sides on the helpers' products bound it
+// (n = 16384, 64: 42.8 -> 35.1 ms, 0.98 TFLOP/s of 1.1).
 //
 // Roles come from an atomic ticket in order (tickets below the number of leaders
 // NL lead; ticket t helps block LAG + t - NL), so the leaders are running before
@@ -62,10 +60,6 @@ template <>
 struct Cfg<double, 1> { static constexpr int LAG = 5, NAUX = 3; };
 template <>
 struct Cfg<double, 4> { static constexpr int LAG = 3, NAUX = 1; };
-template <>
-struct Cfg<float, 1> { static constexpr int LAG = 8, NAUX = 3; };
-template <>
-struct Cfg<float, 4> { static constexpr int LAG = 5, NAUX = 1; };
 
 template <typename T>
 struct Helper {
@@ -111,10 +105,6 @@ JMG_DEV void st_release_sm(int* p, int v) {
 }
 // asynchronous global -> shared copies of one element (L is final while the
 // kernel runs, so caching it in L1 is safe)
-JMG_DEV void cp_async_elem(float* dst, const float* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src)
-               : "memory");
-}
 JMG_DEV void cp_async_elem(double* dst, const double* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(dst)), "l"(src)
                : "memory");
@@ -266,15 +256,11 @@ __global__ void __launch_bounds__(trsv::TH, 1)
     };
     constexpr int AUX0 = NR == 1 ? 1 : 4;   // first aux warp: (column, part)
     constexpr int PREP = 10, LOAD0 = 12;
-    // 1 / x: FP64 on the integer pipe, off the one the chain uses
+    // 1 / x on the integer pipe, off the one the chain uses
     auto inverse = [](T x) -> T {
-      if constexpr (sizeof(T) == 8) {
-        bool bad = false;
-        const T r = pivot_rcp(x < T(0) ? -x : x, &bad);
-        return x < T(0) ? -r : r;
-      } else {
-        return T(1) / x;
-      }
+      bool bad = false;
+      const T r = pivot_rcp(x < T(0) ? -x : x, &bad);
+      return x < T(0) ? -r : r;
     };
     if (warp < NR) {
       // ---- chain warp of right-hand side c0 + warp
@@ -542,19 +528,15 @@ static int trsv_launch(int n, int nrhs, const T* L, int lda, T* B, int ldb, int 
   return JMG_OK;
 }
 
-template <typename T>
-int launch_trsv_persist(int n, int nrhs, const T* L, int lda, T* B, int ldb, int trans,
-                        int* sync, int* info, cudaStream_t s, int hold) {
+template <>
+int launch_trsv_persist<double>(int n, int nrhs, const double* L, int lda, double* B, int ldb,
+                                int trans, int* sync, int* info, cudaStream_t s, int hold) {
   if (n <= 0 || nrhs <= 0) return JMG_OK;
   // Up to 16 right-hand sides every one gets a leader of its own (the chain sets
   // the time); beyond, the helpers' products do, and four share a leader.
   if (nrhs <= trsv::GR)
-    return trsv_launch<T, 1>(n, nrhs, L, lda, B, ldb, trans, sync, info, s, hold);
-  return trsv_launch<T, 4>(n, nrhs, L, lda, B, ldb, trans, sync, info, s, hold);
+    return trsv_launch<double, 1>(n, nrhs, L, lda, B, ldb, trans, sync, info, s, hold);
+  return trsv_launch<double, 4>(n, nrhs, L, lda, B, ldb, trans, sync, info, s, hold);
 }
-template int launch_trsv_persist<float>(int, int, const float*, int, float*, int, int, int*,
-                                        int*, cudaStream_t, int);
-template int launch_trsv_persist<double>(int, int, const double*, int, double*, int, int, int*,
-                                         int*, cudaStream_t, int);
 
 }  // namespace jmg

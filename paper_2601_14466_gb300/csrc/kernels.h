@@ -66,6 +66,12 @@ size_t trsv_sync_ints(int n, int nrhs);
 template <typename T>
 int launch_trsv_persist(int n, int nrhs, const T* L, int lda, T* B, int ldb, int trans, int* sync,
                         int* info, cudaStream_t s, int hold = 0);
+template <>
+int launch_trsv_persist<double>(int n, int nrhs, const double* L, int lda, double* B, int ldb,
+                                int trans, int* sync, int* info, cudaStream_t s, int hold);
+template <>
+int launch_trsv_persist<float>(int n, int nrhs, const float* L, int lda, float* B, int ldb,
+                               int trans, int* sync, int* info, cudaStream_t s, int hold);
 // (L L^T) X = B: forward then backward with launch_trsv_persist.
 template <typename T>
 int solve_llt(int n, int nrhs, const T* L, int lda, T* B, int ldb, int* sync, int* info,
