@@ -226,14 +226,15 @@ static int factor_mixed(int n, float* W, int ldw, const jmg_options& o, const Pl
       if (m <= 0) break;
       float* Wkk = W + (size_t)k * ldw + k;
       float* L21 = Wkk + kb;
-      JMG_TRY(launch_trsm(L21, ldw, m, kb, Wkk, info_f, s));
       const size_t orow = (size_t)(k + kb - k0);  // operand row of L21's first row
-      if (fp8)
+      if (fp8) {
+        JMG_TRY(launch_trsm(L21, ldw, m, kb, Wkk, info_f, s));
         JMG_TRY(launch_quant_fp8(m, kb, L21, ldw, opA(orow, pp * kp), p.ldp,
                                  ex + (size_t)pp * lde + orow / 128, s));
-      else
-        JMG_TRY(launch_split_words(m, kb, L21, ldw, o.prec, o.words, opA(orow, pp * kp),
-                                   opB(orow, pp * kp), p.ldp, s));
+      } else {
+        JMG_TRY(launch_trsm_words(L21, ldw, m, kb, Wkk, info_f, o.prec, o.words,
+                                  opA(orow, pp * kp), opB(orow, pp * kp), p.ldp, s));
+      }
       const int ncb = k0 + NBk - (k + kb);  // columns of this block right of the panel
       if (ncb > 0) {
         // the block's remaining columns, with this panel's words only

@@ -427,127 +427,189 @@ int launch_trsm(double* A21, int lda, int m, int kb, const double* Lkk, const in
                 cudaStream_t s) {
   return trsm_impl<double, 32>(A21, lda, m, kb, Lkk, info, s);
 }
-// FP32 panel TRSM of the mixed path (kb == KB): row r of the panel solves
-// x Lkk^T = a by forward substitution, four threads per row (lanes 4r' .. 4r'+3
-// of a warp), each owning 8 of every 32 columns.  Columns go in 32-wide chunks:
-// chunk J first subtracts the finished chunks (x_k L_ck for k < 32J, an
-// independent FMA per column: the bulk of the work, spread over the four
-// threads), then solves its diagonal 32 x 32 block (x_k = a_k / L_kk by the
-// owner, broadcast to the row's other three lanes by a shuffle, a_c -= x_k L_ck).
-// The 64-row tile of the panel and L_kk (transposed, Lt[k][c] = L[c][k]) sit in
-// shared memory; global traffic is coalesced down the columns.
-namespace ptrsm {
-constexpr int RB = 64, TH = 256, LDX = RB + 1;
+// 16-bit words of the mixed path's tensor-core operands
+// word pairs (a, b) with a + b < words, ordered by significance
+__constant__ int c_pair_a[6] = {0, 0, 1, 0, 1, 2};
+__constant__ int c_pair_b[6] = {0, 1, 0, 2, 1, 0};
+int split_pairs(int words) { return words <= 1 ? 1 : (words == 2 ? 3 : 6); }
+template <typename H>
+JMG_DEV H to16(float v);
+template <>
+JMG_DEV __nv_bfloat16 to16<__nv_bfloat16>(float v) {
+  return __float2bfloat16_rn(v);
 }
+template <>
+JMG_DEV __half to16<__half>(float v) {
+  return __float2half_rn(v);
+}
+template <typename H>
+JMG_DEV float from16(H v);
+template <>
+JMG_DEV float from16<__nv_bfloat16>(__nv_bfloat16 v) {
+  return __bfloat162float(v);
+}
+template <>
+JMG_DEV float from16<__half>(__half v) {
+  return __half2float(v);
+}
+template <typename H>
+struct alignas(4) Two16 {
+  H x, y;
+};
 
+// FP32 panel TRSM (kb == KB): row r of the panel solves x Lkk^T = a, G lanes per row,
+// each holding the column pairs {2 (g + G i), 2 (g + G i) + 1}: step j shuffles a_j to
+// the row's lanes, x_j = a_j / L_jj (by the reciprocal), a_l -= x_j L_lj for l > j, in
+// this order whatever G is.  32-row tiles go through shared memory (coalesced down
+// the columns of L21), a resident grid keeps L_kk.  Bound by issue: about 20
+// instructions per step for 4 rows.
+//
+// With PA the same pass writes the rows' 16-bit words w0 = rn(x), w1 = rn(x - w0), ...
+// into the row-major extended operands of the update: pair p of the pair table takes
+// PA[:, p KB + c] = word a_p, PB[:, p KB + c] = word b_p (PB may be null).
+// Panel of 128 columns with FP16 words, n = 16384: 28 us a panel on average against
+// 25.4 + 8.6 us with the words in a pass of their own.
+namespace ptrsm {
+constexpr int RB = 32, TH = 256, G = 8, LDX = RB + 1;
 template <int KB>
-__global__ void __launch_bounds__(ptrsm::TH, 1) k_trsm_rows(float* __restrict__ A21, int lda, int m,
-                                                        const float* __restrict__ Lkk,
-                                                        const int* __restrict__ info) {
+constexpr size_t smem() {
+  return sizeof(float) * ((size_t)KB * KB + (size_t)KB * LDX + KB);
+}
+}  // namespace ptrsm
+
+template <int KB, typename H>
+__global__ void __launch_bounds__(ptrsm::TH, 2) k_trsm_rows(float* __restrict__ A21, int lda, int m,
+                                                            const float* __restrict__ Lkk,
+                                                            const int* __restrict__ info,
+                                                            int npairs, H* __restrict__ PA,
+                                                            H* __restrict__ PB, int ldp) {
   using namespace ptrsm;
+  constexpr int NP = KB / 2 / G;
   if (*(volatile const int*)info != 0) return;
   extern __shared__ __align__(16) float sm_trows[];
-  float(*Lt)[KB] = reinterpret_cast<float(*)[KB]>(sm_trows);            // KB x KB
-  float(*Xt)[LDX] = reinterpret_cast<float(*)[LDX]>(sm_trows + KB * KB);  // KB x RB (column-major tile)
-  float* rinv = sm_trows + KB * KB + KB * LDX;
-  const int t = threadIdx.x;
+  float* Lt = sm_trows;        // Lt[j * KB + l] = L_lj, l >= j
+  float* Xt = Lt + KB * KB;    // the tile: Xt[c * LDX + r]
+  float* rinv = Xt + KB * LDX;
+  const int t = threadIdx.x, lane = t % 32, warp = t / 32;
   for (int base = 0; base < KB * KB; base += TH * 16) {  // 16 independent loads per thread
     float v[16];
 #pragma unroll
     for (int q = 0; q < 16; ++q) {
-      const int idx = base + t + TH * q;
-      const int c = idx % KB, k = idx / KB;  // column k of L, row c
-      v[q] = (idx < KB * KB && c >= k) ? Lkk[(size_t)k * lda + c] : 0.0f;
+      const int idx = base + t + TH * q, l = idx % KB, j = idx / KB;
+      v[q] = l >= j ? Lkk[(size_t)j * lda + l] : 0.0f;
     }
 #pragma unroll
-    for (int q = 0; q < 16; ++q) {
-      const int idx = base + t + TH * q;
-      if (idx < KB * KB) Lt[idx / KB][idx % KB] = v[q];
-    }
+    for (int q = 0; q < 16; ++q) Lt[base + t + TH * q] = v[q];
   }
-  __syncthreads();  // Lt complete before its diagonal is read
-  if (t < KB) rinv[t] = 1.0f / Lt[t][t];
-  const int rl = t / 4, g = t % 4, lane = t % 32;
-  // L_kk stays in shared memory; the CTA takes 64-row tiles in turn
+  __syncthreads();
+  if (t < KB) rinv[t] = 1.0f / Lt[t * KB + t];
+  const int g = lane % G, rl = warp * (32 / G) + lane / G;
   for (int r0 = blockIdx.x * RB; r0 < m; r0 += gridDim.x * RB) {
-  __syncthreads();  // Lt, rinv ready; the previous tile's Xt is stored
-  for (int base = 0; base < KB * RB; base += TH * 16) {
-    float v[16];
+    __syncthreads();  // Lt, rinv are in place; the previous tile is stored
+    {
+      constexpr int Q = KB * RB / TH;
+      float v[Q];
 #pragma unroll
-    for (int q = 0; q < 16; ++q) {
-      const int idx = base + t + TH * q;
-      const int r = idx % RB, c = idx / RB;
-      v[q] = (idx < KB * RB && r0 + r < m) ? A21[(size_t)c * lda + r0 + r] : 0.0f;
+      for (int q = 0; q < Q; ++q)
+        v[q] = r0 + lane < m ? A21[(size_t)(warp + 8 * q) * lda + r0 + lane] : 0.0f;
+#pragma unroll
+      for (int q = 0; q < Q; ++q) Xt[(warp + 8 * q) * LDX + lane] = v[q];
+    }
+    __syncthreads();
+    float x[2 * NP];
+#pragma unroll
+    for (int i = 0; i < NP; ++i)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) x[2 * i + h] = Xt[(2 * (g + G * i) + h) * LDX + rl];
+#pragma unroll
+    for (int j = 0; j < KB; ++j) {
+      const int go = (j / 2) % G, io = (j / 2) / G;  // owner lane and register of column j
+      const float xj = __shfl_sync(0xffffffffu, x[2 * io + (j & 1)], go, G) * rinv[j];
+      if (g == go) x[2 * io + (j & 1)] = xj;
+#pragma unroll
+      for (int i = 0; i < NP; ++i) {
+        if (2 * (G - 1 + G * i) + 1 <= j) continue;  // every lane's pair is done
+        const int l = 2 * (g + G * i);
+        const float2 l2 = *reinterpret_cast<const float2*>(&Lt[j * KB + l]);
+        if (l > j) x[2 * i] = fmaf(-xj, l2.x, x[2 * i]);
+        if (l + 1 > j) x[2 * i + 1] = fmaf(-xj, l2.y, x[2 * i + 1]);
+      }
     }
 #pragma unroll
-    for (int q = 0; q < 16; ++q) {
-      const int idx = base + t + TH * q;
-      if (idx < KB * RB) Xt[idx / RB][idx % RB] = v[q];
+    for (int i = 0; i < NP; ++i)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int c = 2 * (g + G * i) + h;
+        Xt[c * LDX + rl] = x[2 * i + h];
+      }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < KB * RB / TH; ++q)
+      if (r0 + lane < m) A21[(size_t)(warp + 8 * q) * lda + r0 + lane] = Xt[(warp + 8 * q) * LDX + lane];
+    if (!PA) continue;
+#pragma unroll
+    for (int rr = 0; rr < RB / 8; ++rr) {  // a warp writes whole rows
+      const int rw = warp * (RB / 8) + rr, r = r0 + rw;
+      if (r >= m) break;
+#pragma unroll
+      for (int cb = 0; cb < KB; cb += 64) {
+        const int c = cb + 2 * lane;
+        float e0 = Xt[c * LDX + rw], e1 = Xt[(c + 1) * LDX + rw];
+        Two16<H> w[3];
+#pragma unroll
+        for (int u = 0; u < 3; ++u) {
+          w[u].x = to16<H>(e0);
+          w[u].y = to16<H>(e1);
+          e0 -= from16<H>(w[u].x);
+          e1 -= from16<H>(w[u].y);
+        }
+        for (int p = 0; p < npairs; ++p) {
+          const size_t at = (size_t)r * ldp + p * KB + c;
+          const int a = c_pair_a[p], b = c_pair_b[p];
+          *reinterpret_cast<Two16<H>*>(&PA[at]) = a == 0 ? w[0] : (a == 1 ? w[1] : w[2]);
+          if (PB) *reinterpret_cast<Two16<H>*>(&PB[at]) = b == 0 ? w[0] : (b == 1 ? w[1] : w[2]);
+        }
+      }
     }
   }
-  __syncthreads();
-#pragma unroll 1
-  for (int J = 0; J < KB / 32; ++J) {
-    const int j0 = J * 32, cb = j0 + 8 * g;  // this thread's 8 columns
-    float x[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) x[i] = Xt[cb + i][rl];
-    // the finished chunks
-#pragma unroll 4
-    for (int k = 0; k < j0; ++k) {
-      const float xk = Xt[k][rl];
-      const float4 l0 = *reinterpret_cast<const float4*>(&Lt[k][cb]);
-      const float4 l1 = *reinterpret_cast<const float4*>(&Lt[k][cb + 4]);
-      x[0] = fmaf(-xk, l0.x, x[0]);
-      x[1] = fmaf(-xk, l0.y, x[1]);
-      x[2] = fmaf(-xk, l0.z, x[2]);
-      x[3] = fmaf(-xk, l0.w, x[3]);
-      x[4] = fmaf(-xk, l1.x, x[4]);
-      x[5] = fmaf(-xk, l1.y, x[5]);
-      x[6] = fmaf(-xk, l1.z, x[6]);
-      x[7] = fmaf(-xk, l1.w, x[7]);
-    }
-    // the diagonal block of the chunk
-#pragma unroll
-    for (int kk = 0; kk < 32; ++kk) {
-      const int k = j0 + kk, go = kk / 8, io = kk % 8;
-      if (g == go) x[io] *= rinv[k];
-      const float xk = __shfl_sync(0xffffffffu, x[io], (lane & ~3) | go);
-      const float4 l0 = *reinterpret_cast<const float4*>(&Lt[k][cb]);
-      const float4 l1 = *reinterpret_cast<const float4*>(&Lt[k][cb + 4]);
-      const float l[8] = {l0.x, l0.y, l0.z, l0.w, l1.x, l1.y, l1.z, l1.w};
-#pragma unroll
-      for (int i = 0; i < 8; ++i)
-        if (8 * g + i > kk) x[i] = fmaf(-xk, l[i], x[i]);
-    }
-#pragma unroll
-    for (int i = 0; i < 8; ++i) Xt[cb + i][rl] = x[i];
-    __syncwarp();  // the row's four lanes read these in the next chunks
-  }
-  __syncthreads();
-  for (int idx = t; idx < KB * RB; idx += TH) {
-    const int r = idx % RB, c = idx / RB;
-    if (r0 + r < m) A21[(size_t)c * lda + r0 + r] = Xt[c][r];
-  }
-  }
+}
+
+template <int KB, typename H>
+static int trsm_rows_launch(float* A21, int lda, int m, const float* Lkk, const int* info, int np,
+                            void* PA, void* PB, int ldp, cudaStream_t s) {
+  auto k = k_trsm_rows<KB, H>;
+  JMG_TRY(ensure_smem(k, (int)ptrsm::smem<KB>()));
+  int dev = 0, nsm = 152;
+  JMG_CUDA(cudaGetDevice(&dev));
+  JMG_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+  const int grid = std::min(cdiv(m, ptrsm::RB), 2 * nsm);
+  k<<<grid, ptrsm::TH, ptrsm::smem<KB>(), s>>>(A21, lda, m, Lkk, info, np, (H*)PA, (H*)PB, ldp);
+  return launched();
 }
 
 int launch_trsm(float* A21, int lda, int m, int kb, const float* Lkk, const int* info,
                 cudaStream_t s) {
   if (m <= 0) return JMG_OK;
-  if (kb == 128 || kb == 64) {
-    auto k = (kb == 128) ? k_trsm_rows<128> : k_trsm_rows<64>;
-    const size_t smem = sizeof(float) * ((size_t)kb * kb + (size_t)kb * ptrsm::LDX + kb);
-    JMG_TRY(ensure_smem(k, (int)smem));
-    int dev = 0, nsm = 152, per_sm = 1;
-    JMG_CUDA(cudaGetDevice(&dev));
-    JMG_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    JMG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, ptrsm::TH, smem));
-    const int grid = std::max(1, std::min(cdiv(m, ptrsm::RB), std::max(per_sm, 1) * nsm));
-    k<<<grid, ptrsm::TH, smem, s>>>(A21, lda, m, Lkk, info);
-    return launched();
-  }
+  if (kb == 128)
+    return trsm_rows_launch<128, __half>(A21, lda, m, Lkk, info, 0, nullptr, nullptr, 0, s);
+  if (kb == 64)
+    return trsm_rows_launch<64, __half>(A21, lda, m, Lkk, info, 0, nullptr, nullptr, 0, s);
   return trsm_impl<float, 64>(A21, lda, m, kb, Lkk, info, s);
+}
+
+int launch_trsm_words(float* A21, int lda, int m, int kb, const float* Lkk, const int* info,
+                      int prec, int words, void* PA, void* PB, int ldp, cudaStream_t s) {
+  if (m <= 0) return JMG_OK;
+  const int np = split_pairs(words);
+  if (np == 1) PB = nullptr;
+  const bool half = prec == JMG_PREC_FP16;
+  if (kb == 128)
+    return half ? trsm_rows_launch<128, __half>(A21, lda, m, Lkk, info, np, PA, PB, ldp, s)
+                : trsm_rows_launch<128, __nv_bfloat16>(A21, lda, m, Lkk, info, np, PA, PB, ldp, s);
+  if (kb == 64)
+    return half ? trsm_rows_launch<64, __half>(A21, lda, m, Lkk, info, np, PA, PB, ldp, s)
+                : trsm_rows_launch<64, __nv_bfloat16>(A21, lda, m, Lkk, info, np, PA, PB, ldp, s);
+  return JMG_ERR_UNSUPPORTED;  // (a panel with rows below it is always full)
 }
 
 // ============================================================================
@@ -952,79 +1014,6 @@ int launch_lower_to_f32(int n, const double* A, int lda, float* W, int ldw, doub
                         cudaStream_t s) {
   if (n <= 0) return JMG_OK;
   k_lower_to_f32<<<n, 256, 0, s>>>(n, A, lda, W, ldw, shift);
-  return launched();
-}
-
-// word pairs (a, b) with a + b < words, ordered by significance
-__constant__ int c_pair_a[6] = {0, 0, 1, 0, 1, 2};
-__constant__ int c_pair_b[6] = {0, 1, 0, 2, 1, 0};
-int split_pairs(int words) { return words <= 1 ? 1 : (words == 2 ? 3 : 6); }
-
-template <typename H>
-JMG_DEV H to16(float v);
-template <>
-JMG_DEV __nv_bfloat16 to16<__nv_bfloat16>(float v) {
-  return __float2bfloat16_rn(v);
-}
-template <>
-JMG_DEV __half to16<__half>(float v) {
-  return __float2half_rn(v);
-}
-template <typename H>
-JMG_DEV float from16(H v);
-template <>
-JMG_DEV float from16<__nv_bfloat16>(__nv_bfloat16 v) {
-  return __bfloat162float(v);
-}
-template <>
-JMG_DEV float from16<__half>(__half v) {
-  return __half2float(v);
-}
-
-// 32 x 32 tiles through shared memory: read down the stored columns of L21,
-// write along the rows of the row-major extended operands.
-template <typename H>
-__global__ void k_split_words(int m, int kb, const float* __restrict__ L21, int ldw, int npairs,
-                              H* __restrict__ PA, H* __restrict__ PB, int ldp) {
-  __shared__ float tile[32][33];
-  const int r0 = blockIdx.x * 32, c0 = blockIdx.y * 32;
-  const int tx = threadIdx.x, ty = threadIdx.y;  // 32 x 8
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    int c = c0 + ty + 8 * q, r = r0 + tx;
-    tile[ty + 8 * q][tx] = (r < m && c < kb) ? L21[(size_t)c * ldw + r] : 0.0f;
-  }
-  __syncthreads();
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    int r = r0 + ty + 8 * q, c = c0 + tx;
-    if (r >= m || c >= kb) continue;
-    float rem = tile[tx][ty + 8 * q];
-    H w[3];
-#pragma unroll
-    for (int u = 0; u < 3; ++u) {
-      w[u] = to16<H>(rem);
-      rem = rem - from16<H>(w[u]);
-    }
-    for (int p = 0; p < npairs; ++p) {
-      PA[(size_t)r * ldp + p * kb + c] = w[c_pair_a[p]];
-      if (PB) PB[(size_t)r * ldp + p * kb + c] = w[c_pair_b[p]];
-    }
-  }
-}
-
-int launch_split_words(int m, int kb, const float* L21, int ldw, int prec, int words, void* PA,
-                       void* PB, int ldp, cudaStream_t s) {
-  if (m <= 0) return JMG_OK;
-  int np = split_pairs(words);
-  dim3 grid(cdiv(m, 32), cdiv(kb, 32)), block(32, 8);
-  if (prec == JMG_PREC_FP16)
-    k_split_words<__half><<<grid, block, 0, s>>>(m, kb, L21, ldw, np, (__half*)PA,
-                                                 np > 1 ? (__half*)PB : nullptr, ldp);
-  else
-    k_split_words<__nv_bfloat16><<<grid, block, 0, s>>>(m, kb, L21, ldw, np, (__nv_bfloat16*)PA,
-                                                        np > 1 ? (__nv_bfloat16*)PB : nullptr,
-                                                        ldp);
   return launched();
 }
 

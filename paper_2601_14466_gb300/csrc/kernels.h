@@ -90,11 +90,11 @@ int potrf_split(int n, double* A, int lda, int* info, void* work, cudaStream_t s
 // W (FP32, ldw) <- lower(A) (FP64), lower triangle only; plus shift on the diagonal.
 int launch_lower_to_f32(int n, const double* A, int lda, float* W, int ldw, double shift,
                         cudaStream_t s);
-// Split FP32 panel L21 (m x kb, ldw) into 16-bit words, written into the
-// extended operands PA / PB (row-major, m x kext, ldp) at K offset `koff`:
-// for each pair p of the pair table, PA[:, p*kb + c] = word a_p, PB = word b_p.
-int launch_split_words(int m, int kb, const float* L21, int ldw, int prec, int words, void* PA,
-                       void* PB, int ldp, cudaStream_t s);
+// The FP32 panel solve (kb 64 or 128) that also writes the solved rows' 16-bit words
+// into the extended operands PA / PB (row-major, m x kext, ldp) from their first
+// column on: for each pair p of the pair table, PA[:, p*kb + c] = word a_p, PB = b_p.
+int launch_trsm_words(float* A21, int lda, int m, int kb, const float* Lkk, const int* info,
+                      int prec, int words, void* PA, void* PB, int ldp, cudaStream_t s);
 int split_pairs(int words);  // number of (a, b) word pairs used for `words`
 
 // ---- refinement helpers
