@@ -16,7 +16,7 @@
 //
 // One launch per direction and per group of at most 64 right-hand sides.
 // Roles come from an atomic ticket in order: tickets 0 .. G-1 are LEADERS, one
-// per 16 right-hand sides, each running the chain above for its columns;
+// per CG right-hand sides, each running the chain above for its columns;
 // every later ticket is a HELPER of one block (in dependency order), forming
 // P_b for all columns of the launch from the finished blocks as the leaders
 // publish them, writing it in place over B_b and raising a flag.  A leader
@@ -46,7 +46,7 @@ namespace sv {
 
 constexpr int BS = 128;            // block rows
 constexpr int LAG = 3;             // blocks the leader multiplies itself: d-1, d-2
-constexpr int CG = 8;              // right-hand sides per leader
+constexpr int GMAX = 16;           // leaders per launch, at most
 constexpr int NMAX = 64;           // right-hand sides per launch
 constexpr int TH = 352;            // 8 compute warps, producer, publisher, fetcher
 constexpr int NCOMP = 256;
@@ -58,15 +58,19 @@ constexpr int HSLOTS = 2;          // helper: tile ring
 // The compute warps split the k range of every product (each warp reads only
 // its part of a block, so shared memory is read about once per product) and
 // the columns; partial sums meet once per step (leader) or per block (helper).
-// Leader: L_KG k-groups of L_KLEN k each x L_CQ column groups of L_CT.
-constexpr int L_CQ = CG >= 16 ? 2 : 1, L_CT = CG / L_CQ, L_KG = 8 / L_CQ, L_KLEN = BS / L_KG;
-constexpr int L_SLAB_READERS = (32 / L_KLEN) * L_CQ;  // warps that read each slab
+// Leader: L_KG k-groups of L_KLEN k each, all CG columns.  CG = 2 right-hand sides per
+// leader up to 16, 4 above: fewer make a step's products shorter, more leaders make
+// the helpers' waits longer (both directions, CG = 8 / 4 / 2: n = 32768, 16 right-hand
+// sides 2.99 / 2.46 / 2.25 ms; 16384, 64: 1.99 / 1.81 / 1.88; 65536, 32: 9.08 / 9.07 /
+// 9.39).
+constexpr int L_KG = 8, L_KLEN = BS / L_KG;
+constexpr int L_SLAB_READERS = 32 / L_KLEN;  // warps that read each slab
 // dynamic shared memory: helper = 2 x (64 KB tile + up to 32 KB of Y);
-// leader = 8 x 16 KB slabs + 2 P buffers + 3 Y buffers + 3 partial-sum
-// buffers (16 columns x 512 B each)
+// leader = 8 x 16 KB slabs + 2 P buffers + 3 Y buffers + 7 partial-sum
+// buffers (CG <= 4 columns x 512 B each)
 constexpr int YB = NMAX * BS * 4;  // bytes of one helper Y buffer (32 KB)
 constexpr int HELPER_BYTES = HSLOTS * (TILE_F * 4 + YB);
-constexpr int LEADER_BYTES = LSLOTS * SLAB_F * 4 + (5 + L_KG - 1) * CG * BS * 4;
+constexpr int LEADER_BYTES = LSLOTS * SLAB_F * 4 + (5 + L_KG - 1) * 4 * BS * 4;
 constexpr int DATA_BYTES = HELPER_BYTES > LEADER_BYTES ? HELPER_BYTES : LEADER_BYTES;
 constexpr int SMEM_BYTES = DATA_BYTES + 1024 /* alignment */ + 256 /* barriers */;
 
@@ -305,6 +309,23 @@ JMG_DEV bool wait_ge(const int* p, int G, int v, Ctl& C, int* err, int* info, ui
   return true;
 }
 
+// The same for all G <= 32 counters by a whole warp, one lane each: a counter costs an
+// L2 round trip, which one lane reading them in turn would pay G times.
+JMG_DEV bool wait_ge_warp(const int* p, int G, int v, Ctl& C, int* err, int* info,
+                          uint64_t limit, int lane) {
+  uint64_t t0 = 0;
+  while (!__all_sync(0xffffffffu, lane >= G || ld_acq(p + lane) >= v)) {
+    if (t0 == 0) t0 = globaltimer_ns();
+    if (__any_sync(0xffffffffu, ld_shared_volatile(&C.abort))) return false;
+    if (__any_sync(0xffffffffu, *(volatile const int*)err || globaltimer_ns() - t0 > limit)) {
+      raise(C, err, info);
+      return false;
+    }
+    __nanosleep(32);
+  }
+  return true;
+}
+
 // acc[r][c] += sign * sum over chunks ch0 .. ch1-1 (4 k each) of one 32-wide
 // k-slab of T(i, k) * V(k, c): T a swizzled tile slab (rows i = lane + 32 r),
 // V column-major with leading dimension BS (columns c0 + c).  Only rows r in
@@ -342,8 +363,9 @@ JMG_DEV void slab_product(const float* __restrict__ slab, const float* __restric
 
 }  // namespace sv
 
-// CT: helper columns per compute warp (N_pad = 8 CT right-hand sides per launch).
-template <int CT>
+// CT: helper columns per compute warp (N_pad = 8 CT right-hand sides per launch); CG:
+// right-hand sides per leader.
+template <int CT, int CG>
 __global__ void __launch_bounds__(sv::TH, 1)
     k_sv_solve(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmDh,
                const __grid_constant__ CUtensorMap tmDl, int n, int ncol, int cb,
@@ -396,7 +418,7 @@ __global__ void __launch_bounds__(sv::TH, 1)
         tc::mbar_init(&pfull[s], 1);
         tc::mbar_init(&pempty[s], 8);
       }
-      tc::mbar_init(ystored, L_CQ);       // the warps of k-group 0 store Y
+      tc::mbar_init(ystored, 1);  // the warp of k-group 0 stores Y
       tc::fence_mbar_init();
     }
     __syncthreads();
@@ -487,19 +509,19 @@ __global__ void __launch_bounds__(sv::TH, 1)
       }
     } else {
       // ------------------------------------------------------------ compute warps
-      const int kg = warp / L_CQ;           // k-group: k in [kg L_KLEN, (kg + 1) L_KLEN)
-      const int cw = (warp % L_CQ) * L_CT;  // this warp's columns (of the leader's CG)
+      const int kg = warp;  // k-group: k in [kg L_KLEN, (kg + 1) L_KLEN)
+      constexpr int cw = 0;
       const int ks = kg * L_KLEN;
       const int sl = ks >> 5, ch0 = (ks & 31) >> 2, ch1 = ch0 + L_KLEN / 4;
       long long gs = 0;
       for (int d = 0; d < nblk; ++d) {
         const int b = blk(d), buf = d & 1;
         bool ok = wait_bar(&pfull[buf], (uint32_t)(d >> 1) & 1, C, err, info, wait_ns);
-        float acc[4][L_CT];
+        float acc[4][CG];
 #pragma unroll
         for (int r = 0; r < 4; ++r)
 #pragma unroll
-          for (int c = 0; c < L_CT; ++c) acc[r][c] = 0.0f;
+          for (int c = 0; c < CG; ++c) acc[r][c] = 0.0f;
         int idx[3];
         const int m = tiles_of(d, idx);
         for (int q = 0; q < m; ++q, gs += 4) {
@@ -510,10 +532,10 @@ __global__ void __launch_bounds__(sv::TH, 1)
           if (ok) ok = wait_bar(&sfull[slot], (uint32_t)(gk / LSLOTS) & 1, C, err, info, wait_ns);
           // Li (lower): row groups sl..3 of slab sl; Li^T (upper): 0..sl
           if (ok && q == 0)
-            slab_product<L_CT, true>(slabs + slot * SLAB_F, V, 32 * sl, ch0, ch1, cw, lane,
+            slab_product<CG, true>(slabs + slot * SLAB_F, V, 32 * sl, ch0, ch1, cw, lane,
                                      trans ? 0 : sl, trans ? sl : 3, acc);
           else if (ok)
-            slab_product<L_CT, false>(slabs + slot * SLAB_F, V, 32 * sl, ch0, ch1, cw, lane, 0,
+            slab_product<CG, false>(slabs + slot * SLAB_F, V, 32 * sl, ch0, ch1, cw, lane, 0,
                                       3, acc);
           __syncwarp();
           if (lane == 0) {
@@ -527,7 +549,7 @@ __global__ void __launch_bounds__(sv::TH, 1)
 #pragma unroll
           for (int r = 0; r < 4; ++r)
 #pragma unroll
-            for (int c = 0; c < L_CT; ++c) R[(cw + c) * BS + lane + 32 * r] = acc[r][c];
+            for (int c = 0; c < CG; ++c) R[(cw + c) * BS + lane + 32 * r] = acc[r][c];
         }
         bar_sync_named(1, NCOMP);
         if (kg == 0) {
@@ -550,7 +572,7 @@ __global__ void __launch_bounds__(sv::TH, 1)
           for (int r = 0; r < 4; ++r) {
             const int i = lane + 32 * r;
 #pragma unroll
-            for (int c = 0; c < L_CT; ++c) {
+            for (int c = 0; c < CG; ++c) {
               float v = acc[r][c];
 #pragma unroll
               for (int q = 0; q < L_KG - 1; ++q) v += red[q * CG * BS + (cw + c) * BS + i];
@@ -605,30 +627,33 @@ __global__ void __launch_bounds__(sv::TH, 1)
     if (warp == 8) {
       // ------------------------------------------------------------ producer
       bool ok = true;
-      if (lane == 0) {
-        for (int q = 0; q < ndep; ++q) {
-          const int slot = (int)(gq % HSLOTS);
-          if (gq >= HSLOTS &&
-              !wait_bar(&empty[slot], (uint32_t)((gq / HSLOTS) - 1) & 1, C, err, info, wait_ns)) {
-            ok = false;
-            break;
-          }
-          const int j = blk(q);
-          // one phase per slot: both copies' bytes, then the arrival once the
-          // second copy is issued (the block of L does not wait for the chain)
+      for (int q = 0; q < ndep; ++q) {
+        const int slot = (int)(gq % HSLOTS);
+        if (lane == 0 && gq >= HSLOTS)
+          ok = wait_bar(&empty[slot], (uint32_t)((gq / HSLOTS) - 1) & 1, C, err, info, wait_ns);
+        ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0);
+        if (!ok) break;
+        const int j = blk(q);
+        // one phase per slot: both copies' bytes, then the arrival once the
+        // second copy is issued (the block of L does not wait for the chain)
+        if (lane == 0) {
           tc::mbar_expect_tx_only(&full[slot], TILE_F * 4 + NP * BS * 4);
           for (int s = 0; s < 4; ++s)
             tc::tma_load_2d(ringL + slot * TILE_F + s * SLAB_F, &tmW, j * BS + 32 * s, r0,
                             &full[slot]);
-          ok = wait_ge(cnt, G, q + 1, C, err, info, wait_ns);
+        }
+        ok = wait_ge_warp(cnt, G, q + 1, C, err, info, wait_ns, lane);
+        if (lane == 0) {
           if (ok) fence_proxy_async_global();
           // (on failure the block is still copied, so that the phase completes
           // and no copy is left in flight when the CTA ends)
           tc::tma_load_2d(ringY + slot * (NMAX * BS), &tmDh, j * BS, cb, &full[slot]);
           tc::mbar_arrive(&full[slot]);
-          ++gq;
-          if (!ok) break;
         }
+        ++gq;
+        if (!ok) break;
+      }
+      if (lane == 0) {
         // P_b is stored once the compute warps arrive: publish it, take the next ticket
         if (ok) ok = wait_bar(hdone, (uint32_t)round & 1, C, err, info, wait_ns);
         if (ok) {
@@ -640,7 +665,6 @@ __global__ void __launch_bounds__(sv::TH, 1)
         tc::mbar_arrive(tnext);  // release the compute warps either way
       }
       __syncwarp();
-      gq = __shfl_sync(0xffffffffu, gq, 0);
       if (!__shfl_sync(0xffffffffu, ok ? 1 : 0, 0)) break;
       my_ticket = C.ticket;
     } else {
@@ -723,7 +747,7 @@ size_t sv_image_bytes(int n) {
 
 size_t sv_sync_ints(int n, int nrhs) {
   (void)nrhs;  // one launch at a time reuses the same words
-  return 2 + sv::NMAX / sv::CG + (size_t)cdiv(std::max(n, 1), sv::BS);
+  return 2 + sv::GMAX + (size_t)cdiv(std::max(n, 1), sv::BS);
 }
 
 int sv_prepare(int n, float* W, int ldw, float* SV, cudaStream_t s) {
@@ -745,12 +769,12 @@ int sv_prepare(int n, float* W, int ldw, float* SV, cudaStream_t s) {
   return launched();
 }
 
-template <int CT>
+template <int CT, int CG>
 static int sv_launch(const CUtensorMap& mw, const CUtensorMap& mdh, const CUtensorMap& mdl, int n,
                      int ncol, int cb, const float* SV, float* D, int ldd, int trans, int* sync,
                      int* info, int grid, cudaStream_t s) {
-  JMG_TRY(ensure_smem(k_sv_solve<CT>, sv::SMEM_BYTES));
-  k_sv_solve<CT><<<grid, sv::TH, sv::SMEM_BYTES, s>>>(mw, mdh, mdl, n, ncol, cb, SV, D, ldd, trans,
+  JMG_TRY(ensure_smem(k_sv_solve<CT, CG>, sv::SMEM_BYTES));
+  k_sv_solve<CT, CG><<<grid, sv::TH, sv::SMEM_BYTES, s>>>(mw, mdh, mdl, n, ncol, cb, SV, D, ldd, trans,
                                                       sync, info, g_wait_ns);
   return launched();
 }
@@ -765,32 +789,33 @@ int sv_solve(int n, int nrhs, const float* W, int ldw, const float* SV, float* D
   int dev = 0, nsm = 152;
   JMG_CUDA(cudaGetDevice(&dev));
   JMG_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-  CUtensorMap mw, mdl;
+  CUtensorMap mw;
   JMG_TRY(make_tmap_2d(&mw, W, (unsigned long long)n, (unsigned long long)n,
                        (unsigned long long)ldw * 4, 32, sv::BS, CU_TENSOR_MAP_DATA_TYPE_FLOAT32,
                        CU_TENSOR_MAP_SWIZZLE_128B));
-  JMG_TRY(make_tmap_2d(&mdl, D, (unsigned long long)n, (unsigned long long)nrhs,
-                       (unsigned long long)ldd * 4, sv::BS, sv::CG,
-                       CU_TENSOR_MAP_DATA_TYPE_FLOAT32, CU_TENSOR_MAP_SWIZZLE_NONE));
   for (int cb = 0; cb < nrhs; cb += sv::NMAX) {
     const int ncol = std::min(sv::NMAX, nrhs - cb);
     const int ct = ncol > 32 ? 8 : ncol > 16 ? 4 : ncol > 8 ? 2 : 1;
-    CUtensorMap mdh;
+    const int cg = ncol > 16 ? 4 : 2;
+    CUtensorMap mdh, mdl;
+    JMG_TRY(make_tmap_2d(&mdl, D, (unsigned long long)n, (unsigned long long)nrhs,
+                         (unsigned long long)ldd * 4, sv::BS, cg, CU_TENSOR_MAP_DATA_TYPE_FLOAT32,
+                         CU_TENSOR_MAP_SWIZZLE_NONE));
     JMG_TRY(make_tmap_2d(&mdh, D, (unsigned long long)n, (unsigned long long)nrhs,
                          (unsigned long long)ldd * 4, sv::BS, 8 * ct,
                          CU_TENSOR_MAP_DATA_TYPE_FLOAT32, CU_TENSOR_MAP_SWIZZLE_NONE));
     // the error word survives every launch but the first forward one
     const int keep = (trans || cb > 0) ? 1 : 0;
     JMG_CUDA(cudaMemsetAsync(sync + keep, 0, sizeof(int) * (sv_sync_ints(n, nrhs) - keep), s));
-    const int G = cdiv(ncol, sv::CG);
+    const int G = cdiv(ncol, cg);
     const int helpers = std::max(0, nblk - sv::LAG);
     const int grid = std::max(G, std::min(nsm, G + helpers));
     int st;
     switch (ct) {
-      case 8: st = sv_launch<8>(mw, mdh, mdl, n, ncol, cb, SV, D, ldd, trans, sync, info, grid, s); break;
-      case 4: st = sv_launch<4>(mw, mdh, mdl, n, ncol, cb, SV, D, ldd, trans, sync, info, grid, s); break;
-      case 2: st = sv_launch<2>(mw, mdh, mdl, n, ncol, cb, SV, D, ldd, trans, sync, info, grid, s); break;
-      default: st = sv_launch<1>(mw, mdh, mdl, n, ncol, cb, SV, D, ldd, trans, sync, info, grid, s); break;
+      case 8: st = sv_launch<8, 4>(mw, mdh, mdl, n, ncol, cb, SV, D, ldd, trans, sync, info, grid, s); break;
+      case 4: st = sv_launch<4, 4>(mw, mdh, mdl, n, ncol, cb, SV, D, ldd, trans, sync, info, grid, s); break;
+      case 2: st = sv_launch<2, 2>(mw, mdh, mdl, n, ncol, cb, SV, D, ldd, trans, sync, info, grid, s); break;
+      default: st = sv_launch<1, 2>(mw, mdh, mdl, n, ncol, cb, SV, D, ldd, trans, sync, info, grid, s); break;
     }
     JMG_TRY(st);
   }
