@@ -140,16 +140,23 @@ static T* at(void* work, size_t off) {
 // in FP64 arithmetic).
 template <typename T>
 static int potrf_plain(int n, T* A, int lda, int nb, int* info, cudaStream_t s) {
-  for (int k = 0; k < n; k += nb) {
+  if (n <= 0) return JMG_OK;
+  JMG_TRY(launch_potf2(A, lda, std::min(nb, n), 0, info, s));
+  for (int k = 0; k < n; k += nb) {  // the diagonal block at k is factored
     const int kb = std::min(nb, n - k);
     T* Akk = A + (size_t)k * lda + k;
-    JMG_TRY(launch_potf2(Akk, lda, kb, k, info, s));
-    const int m = n - k - kb;
+    const int m = n - k - kb, kn = std::min(nb, m);
     if (m <= 0) break;
     T* L21 = Akk + kb;
+    T* A22 = A + (size_t)(k + kb) * lda + (k + kb);
     JMG_TRY(launch_trsm(L21, lda, m, kb, Akk, info, s));
-    JMG_TRY(launch_gemm<T>(m, m, kb, L21, lda, MODE_N, L21, lda, MODE_T,
-                           A + (size_t)(k + kb) * lda + (k + kb), lda, OUT_SUB_LOWER, 1, info, s));
+    if constexpr (sizeof(T) == 4) {
+      JMG_TRY(launch_syrk_f32(m, kb, kn, k + kb, L21, A22, lda, info, s));
+    } else {
+      JMG_TRY(launch_gemm<T>(m, m, kb, L21, lda, MODE_N, L21, lda, MODE_T, A22, lda,
+                             OUT_SUB_LOWER, 1, info, s));
+      JMG_TRY(launch_potf2(A22, lda, kn, k + kb, info, s));
+    }
   }
   return JMG_OK;
 }

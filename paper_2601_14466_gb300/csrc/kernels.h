@@ -32,6 +32,11 @@ int launch_trsm(double* A21, int lda, int m, int kb, const double* Lkk, const in
 int launch_trsm(float* A21, int lda, int m, int kb, const float* Lkk, const int* info,
                 cudaStream_t s);
 
+// FP32: C (m x m, lower) -= P P^T (m x kb, kb % 16 == 0), then the kn x kn block (kn <=
+// 128) at C's head is factored as by launch_potf2 with koff.
+int launch_syrk_f32(int m, int kb, int kn, int koff, const float* P, float* C, int lda, int* info,
+                    cudaStream_t s);
+
 // C (m x n) -= op(A) (m x k) * op(B) (k x n), T arithmetic.
 // For OUT_SUB_LOWER, m == n and the tile grid covers the lower triangle.
 // For OUT_PART, `C` is the partial buffer with `splits` slices of ldc*n.
