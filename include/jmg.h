@@ -122,10 +122,12 @@ void jmg_default_options(jmg_options* opt);
 size_t jmg_workspace_size(int op, int n, int nrhs, int dtype, const jmg_options* opt);
 
 /* Bytes of `work` with which the same call takes its fastest route: never less
- * than jmg_workspace_size().  More than that only for the plain FP64 calls with a
- * factorisation (potrf, posv and posv_host, prec NATIVE), whose trailing updates
- * then run on the tensor cores in error-free slices (about 7.2 KB per row of A),
- * with a 256-byte aligned `work`; with less, they run on the FP64 CUDA cores. */
+ * than jmg_workspace_size().  More than that only for plain FP64 calls (prec NATIVE):
+ * with a factorisation (potrf, posv, posv_host; n > 64), whose trailing updates
+ * then run on the tensor cores in error-free slices (about 8.1 KB per row of A), and
+ * with many right-hand sides in a large solve (potrs, posv, posv_host; nrhs > 16,
+ * n >= 4096 and n >= 8192 or n * nrhs >= 250000; about as much), whose products do.  `work` has to
+ * be 256-byte aligned for that; with less, they run on the FP64 CUDA cores. */
 size_t jmg_workspace_fast(int op, int n, int nrhs, int dtype, const jmg_options* opt);
 
 /*

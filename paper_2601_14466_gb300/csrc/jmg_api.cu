@@ -268,6 +268,15 @@ static int potrf_native(int n, void* A, int lda, int dtype, int nb, int* info, v
   return potrf_plain<double>(n, (double*)A, lda, nb, info, s);
 }
 
+// The plain FP64 solve by the scratch at hand (beyond sync's ints).
+static int solve_native(int n, int nrhs, const double* L, int lda, double* B, int ldb, int* sync,
+                        int* info, void* work, size_t lwork, cudaStream_t s) {
+  const size_t fast = ozs_workspace(n, nrhs);
+  if (fast > 0 && work && lwork >= fast && !(reinterpret_cast<uintptr_t>(work) & 255))
+    return solve_split(n, nrhs, L, lda, B, ldb, sync, info, work, s);
+  return solve_llt<double>(n, nrhs, L, lda, B, ldb, sync, info, s);
+}
+
 // column max of |B| into colmax_r and R = B (start of refinement from X = 0)
 __global__ void k_copy_colmax(int n, const double* __restrict__ B, int ldb, double* __restrict__ R,
                               double* __restrict__ colmax) {
@@ -737,9 +746,12 @@ size_t jmg_workspace_fast(int op, int n, int nrhs, int dtype, const jmg_options*
   opts_or_default(opt, &o);
   const size_t base = jmg_workspace_size(op, n, nrhs, dtype, &o);
   if (n <= 0 || dtype != JMG_F64 || o.prec != JMG_PREC_NATIVE) return base;
-  if (op == JMG_OP_POTRF || op == JMG_OP_POSV || op == JMG_OP_POSV_HOST)
-    return round_up(base, 256) + ozf_workspace(n);
-  return base;
+  const size_t factor = ozf_workspace(n), solve = ozs_workspace(n, nrhs);
+  size_t more = 0;
+  if (op == JMG_OP_POTRF) more = factor;
+  if (op == JMG_OP_POTRS) more = solve;
+  if (op == JMG_OP_POSV || op == JMG_OP_POSV_HOST) more = std::max(factor, solve);
+  return more ? round_up(base, 256) + more : base;
 }
 
 const char* jmg_status_string(int st) {
@@ -785,8 +797,9 @@ int jmg_potrs(int n, int nrhs, const void* L, int lda, void* B, int ldb, int dty
   if (dtype == JMG_F32)
     return solve_llt<float>(n, nrhs, (const float*)L, lda, (float*)B, ldb, (int*)work, nullptr,
                             (cudaStream_t)stream);
-  return solve_llt<double>(n, nrhs, (const double*)L, lda, (double*)B, ldb, (int*)work, nullptr,
-                           (cudaStream_t)stream);
+  const size_t sb = plain_solve_bytes(n, nrhs);
+  return solve_native(n, nrhs, (const double*)L, lda, (double*)B, ldb, (int*)work, nullptr,
+                      static_cast<char*>(work) + sb, lwork - sb, (cudaStream_t)stream);
 }
 
 int jmg_posv(int n, int nrhs, void* A, int lda, void* B, int ldb, int dtype, int* info,
@@ -814,8 +827,9 @@ int jmg_posv(int n, int nrhs, void* A, int lda, void* B, int ldb, int dtype, int
     JMG_CUDA(cudaMemsetAsync(info, 0, sizeof(int), s));
     // the solve's tickets and flags first, the factor's scratch behind them
     const size_t sb = plain_solve_bytes(n, nrhs);
-    JMG_TRY(potrf_native(n, A, lda, dtype, o.nb, info, work ? static_cast<char*>(work) + sb : nullptr,
-                         lwork > sb ? lwork - sb : 0, s));
+    char* more = work ? static_cast<char*>(work) + sb : nullptr;
+    const size_t lmore = lwork > sb ? lwork - sb : 0;
+    JMG_TRY(potrf_native(n, A, lda, dtype, o.nb, info, more, lmore, s));
     if (dtype == JMG_F32) {
       if (nrhs > 0)
         JMG_TRY(solve_llt<float>(n, nrhs, (const float*)A, lda, (float*)B, ldb, (int*)work, info,
@@ -823,8 +837,8 @@ int jmg_posv(int n, int nrhs, void* A, int lda, void* B, int ldb, int dtype, int
       return JMG_OK;
     }
     if (nrhs > 0)
-      JMG_TRY(solve_llt<double>(n, nrhs, (const double*)A, lda, (double*)B, ldb, (int*)work, info,
-                                s));
+      JMG_TRY(solve_native(n, nrhs, (const double*)A, lda, (double*)B, ldb, (int*)work, info, more,
+                           lmore, s));
     return JMG_OK;
   }
   if (dtype == JMG_F32) return JMG_ERR_UNSUPPORTED;  // mixed modes refine FP64 data

@@ -289,15 +289,20 @@ __global__ void __launch_bounds__(THREADS) k_oz_diag(double* __restrict__ A, int
 }
 
 // ---------------------------------------------------------------------------
-// C (rows and columns from r0 on, columns below r0 + ncols, lower part) -=
-// P P^T, P given by its slices: row r of slice s is row s * n + r of the map.  CTA 0
-// takes tile 0 alone and then factors the diagonal block it has just updated (kb
-// columns), while the others work through the rest of the update.
+// C (m x ncols) -= P Q^T, P and Q given by their slices and row exponents: row r of
+// slice s is row s * nA + rA + r of P's map (nB, rB: Q's).
+//  * RECT = false, the factorisation: Q is P's head, only the lower part is updated, and
+//    CTA 0 takes tile 0 alone and then factors the diagonal block it has just updated
+//    (kb_diag columns), while the others work through the rest of the update;
+//  * RECT = true, the blocked solves: the whole rectangle.
+// info may be null when RECT; err (RECT only) is the solve's error word.
+template <bool RECT>
 __global__ void __launch_bounds__(THREADS, 1)
-    k_oz_syrk(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-              double* __restrict__ C, int ldc, int n, int r0, int ncols, int nkb,
-              const int* __restrict__ ex, int TI, int TJ, int ntiles, int kb_diag,
-              int* __restrict__ info, unsigned long long wait_ns) {
+    k_oz_update(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+                double* __restrict__ C, int ldc, int nA, int rA, int nB, int rB, int m, int ncols,
+                int nkb, const int* __restrict__ exA, const int* __restrict__ exB, int TI, int TJ,
+                int ntiles, int kb_diag, int koff, int* __restrict__ info, int* __restrict__ err,
+                unsigned long long wait_ns) {
   using namespace tc;
   extern __shared__ __align__(1024) unsigned char sm_raw_ozf[];
   unsigned char* smem = reinterpret_cast<unsigned char*>(
@@ -316,10 +321,17 @@ __global__ void __launch_bounds__(THREADS, 1)
 
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   // this CTA's tiles: first, first + step, ...
-  const int first = blockIdx.x, step = blockIdx.x == 0 ? ntiles : (int)gridDim.x - 1;
+  const int first = blockIdx.x,
+            step = RECT ? (int)gridDim.x : (blockIdx.x == 0 ? ntiles : (int)gridDim.x - 1);
+  auto tile = [&](int b, int& ti, int& tj) -> bool {
+    if (!RECT) return tile_of(b, TI, TJ, ti, tj);
+    ti = b / TJ, tj = b % TJ;
+    return true;
+  };
   if (threadIdx.x == 0) {
     s_fail = 0;
-    s_info = *(volatile int*)info;
+    s_info = info ? *(volatile int*)info : 0;
+    if (RECT && *(volatile int*)err != 0) s_info = 1;  // an earlier launch gave up
     for (int i = 0; i < 2; ++i) {
       mbar_init(&bfull[i], 1);
       mbar_init(&bempty[i], 1);
@@ -351,7 +363,7 @@ __global__ void __launch_bounds__(THREADS, 1)
       bool ok = true;
       for (int b = first; b < ntiles && ok; b += step) {
         int ti, tj;
-        if (!tile_of(b, TI, TJ, ti, tj)) continue;
+        if (!tile(b, ti, tj)) continue;
         for (int kb = 0; kb < nkb && ok; ++kb) {
           const int bs = (int)(b_issued & 1);
           if (b_issued >= 2 &&
@@ -365,7 +377,7 @@ __global__ void __launch_bounds__(THREADS, 1)
           }
           mbar_expect_tx(&bfull[bs], B_BUF);
           for (int s = 0; s < S; ++s)
-            tma_load_2d(bbuf + bs * B_BUF + s * B_TILE, &tmB, kb * BK, s * n + r0 + tj * BN,
+            tma_load_2d(bbuf + bs * B_BUF + s * B_TILE, &tmB, kb * BK, s * nB + rB + tj * BN,
                         &bfull[bs]);
           ++b_issued;
           for (int s = 0; s < S; ++s) {
@@ -376,7 +388,7 @@ __global__ void __launch_bounds__(THREADS, 1)
               break;
             }
             mbar_expect_tx(&afull[st], A_TILE);
-            tma_load_2d(abuf + st * A_TILE, &tmA, kb * BK, s * n + r0 + ti * BM, &afull[st]);
+            tma_load_2d(abuf + st * A_TILE, &tmA, kb * BK, s * nA + rA + ti * BM, &afull[st]);
             ++a_issued;
           }
         }
@@ -390,7 +402,7 @@ __global__ void __launch_bounds__(THREADS, 1)
       bool ok = true;
       for (int b = first; b < ntiles && ok; b += step) {
         int ti, tj;
-        if (!tile_of(b, TI, TJ, ti, tj)) continue;
+        if (!tile(b, ti, tj)) continue;
         for (int kw = 0; kw < nkb && ok; kw += WIN, ++gw) {
           if (gw >= 1 && !mbar_wait(acce, (uint32_t)(gw - 1) & 1, wait_ns)) {
             ok = false;
@@ -450,11 +462,11 @@ __global__ void __launch_bounds__(THREADS, 1)
     bool ok = true;
     for (int b = first; b < ntiles && ok; b += step) {
       int ti, tj;
-      if (!tile_of(b, TI, TJ, ti, tj)) continue;
-      const int row = r0 + ti * BM + q * 32 + lane;
-      const int c0 = r0 + tj * BN + ch;
-      // columns c < jn of this thread are in range and on or below the diagonal
-      const int jn = row < n ? min(CW, min(r0 + ncols - c0, row - c0 + 1)) : 0;
+      if (!tile(b, ti, tj)) continue;
+      const int row = ti * BM + q * 32 + lane;
+      const int c0 = tj * BN + ch;
+      // columns c < jn of this thread are in range (and on or below the diagonal)
+      const int jn = row < m ? min(CW, min(ncols - c0, RECT ? CW : row - c0 + 1)) : 0;
       unsigned long long acc[CW];  // (unsigned: rows and columns past the end wrap, never trap)
 #pragma unroll
       for (int c = 0; c < CW; ++c) acc[c] = 0ull;
@@ -497,14 +509,14 @@ __global__ void __launch_bounds__(THREADS, 1)
       }
       if (jn > 0) {
         double* cp = C + (size_t)c0 * ldc + row;
-        const int er = ex[row];
+        const int er = exA[row];
         double old[CW];
 #pragma unroll
         for (int c = 0; c < CW; ++c) old[c] = c < jn ? cp[(size_t)c * ldc] : 0.0;
 #pragma unroll
         for (int c = 0; c < CW; ++c)
           if (c < jn) {
-            const int ec = ex[c0 + c];
+            const int ec = exB[c0 + c];
             double r = old[c] - scaled_double((long long)acc[c], er + ec - 14 - sh);
             if (er == E_BAD || ec == E_BAD) r = __longlong_as_double(0x7FF8000000000000ll);
             cp[(size_t)c * ldc] = r;
@@ -520,15 +532,16 @@ __global__ void __launch_bounds__(THREADS, 1)
         (void)mbar_wait(&bfull[u & 1], (uint32_t)(u >> 1) & 1, wait_ns);
       for (long long g = (a_issued > ASTAGES ? a_issued - ASTAGES : 0); g < a_issued; ++g)
         (void)mbar_wait(&afull[g % ASTAGES], (uint32_t)(g / ASTAGES) & 1, wait_ns);
-      atomicCAS(info, 0, -1);
+      if (info) atomicCAS(info, 0, -1);
+      if (RECT) atomicExch(err, JMG_ERR_TIMEOUT);
     }
   }
   tc_fence_before();
   __syncthreads();
   if (warp == 1) tmem_dealloc(tmem, TCOLS);
-  if (blockIdx.x == 0 && !ld_shared_volatile(&s_fail)) {
+  if (!RECT && blockIdx.x == 0 && !ld_shared_volatile(&s_fail)) {
     __syncthreads();  // tile 0 is in global memory, the rings are idle
-    diag_body(reinterpret_cast<double*>(smem), C + (size_t)r0 * ldc + r0, ldc, kb_diag, r0, info);
+    diag_body(reinterpret_cast<double*>(smem), C, ldc, kb_diag, koff, info);
   }
 }
 
@@ -640,7 +653,7 @@ __global__ void __launch_bounds__(256) k_oz_strip(const double* __restrict__ A, 
                                                   int* __restrict__ ex,
                                                   const int* __restrict__ info) {
   __shared__ double T[64][33];
-  if (*(volatile const int*)info != 0) return;
+  if (info && *(volatile const int*)info != 0) return;
   const int t = threadIdx.x;
   const int rb = r0 + blockIdx.x * 32, kc = blockIdx.y * 64;
   {
@@ -674,6 +687,95 @@ __global__ void __launch_bounds__(256) k_oz_strip(const double* __restrict__ A, 
   for (int s = 0; s < S; ++s)
     *reinterpret_cast<uint4*>(&SP[((size_t)s * n + row) * K + kc + cc]) =
         make_uint4(w[s][0], w[s][1], w[s][2], w[s][3]);
+}
+
+// ---------------------------------------------------------------------------
+// The blocked solves' operands.
+
+// Row maxima (abs_bits order) of every SK-wide block column of the lower L, diagonal
+// blocks included: out[b * n + i].  grid = (rows / 256, blocks); a thread walks its row,
+// coalesced across the threads.
+constexpr int SK = 512;
+__global__ void __launch_bounds__(256) k_oz_block_max(const double* __restrict__ L, int lda, int n,
+                                                      unsigned long long* __restrict__ out) {
+  const int i = blockIdx.x * 256 + threadIdx.x, k0 = blockIdx.y * SK;
+  if (i >= n) return;
+  unsigned long long mx = 0;
+  const int ke = min(k0 + SK, i + 1);
+#pragma unroll 8
+  for (int k = k0; k < ke; ++k) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(L[(size_t)k * lda + i]) &
+                                 0x7FFFFFFFFFFFFFFFull;
+    mx = b > mx ? b : mx;
+  }
+  out[(size_t)blockIdx.y * n + i] = mx;
+}
+// sc[i] = the exponent of row i of L over all its blocks
+__global__ void k_oz_row_scale(int n, int nb, const unsigned long long* __restrict__ bmax,
+                               int* __restrict__ sc) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  unsigned long long mx = 0;
+  for (int b = 0; b < nb; ++b) {
+    const unsigned long long v = bmax[(size_t)b * n + i];
+    mx = v > mx ? v : mx;
+  }
+  const int e = scale_exp_bits(mx);
+  sc[i] = e == E_BAD ? 0 : e;
+}
+
+// x 2^e by integer addition to the exponent field where it stays normal
+JMG_DEV double mul_pow2(double x, int e) {
+  const int E = (__double2hiint(x) >> 20) & 0x7FF;
+  if (E == 0 || E == 0x7FF || E + e < 1 || E + e > 0x7FE) return ldexp(x, e);
+  return __hiloint2double(__double2hiint(x) + (e << 20), __double2loint(x));
+}
+
+// Slices of the columns of a column-major P (kv <= SK rows, ncols columns), one
+// exponent per column: slice s, column c, row k at SP[(s * ncols + c) * SK + k] (zero
+// past kv).  Row k is scaled by 2^(sign sc[k]) first (sign 0: not).  One warp per
+// column.
+__global__ void __launch_bounds__(256) k_oz_cut_cols(const double* __restrict__ P, int ld, int kv,
+                                                     int ncols, const int* __restrict__ sc,
+                                                     int sign, __nv_bfloat16* __restrict__ SP,
+                                                     int* __restrict__ ex) {
+  const int c = blockIdx.x * 8 + threadIdx.x / 32, lane = threadIdx.x % 32;
+  if (c >= ncols) return;
+  constexpr int Q = SK / 64;
+  double x[2 * Q];
+#pragma unroll
+  for (int q = 0; q < Q; ++q)
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int k = 64 * q + 2 * lane + h;
+      x[2 * q + h] = k < kv ? P[(size_t)c * ld + k] : 0.0;
+    }
+  unsigned long long mx = 0;
+#pragma unroll
+  for (int i = 0; i < 2 * Q; ++i) {
+    const int k = 64 * (i / 2) + 2 * lane + (i & 1);
+    if (sign != 0 && k < kv) x[i] = mul_pow2(x[i], sign * sc[k]);
+    const unsigned long long b =
+        (unsigned long long)__double_as_longlong(x[i]) & 0x7FFFFFFFFFFFFFFFull;
+    mx = b > mx ? b : mx;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long b = __shfl_xor_sync(0xffffffffu, mx, o);
+    mx = b > mx ? b : mx;
+  }
+  const int e = scale_exp_bits(mx);
+  if (lane == 0) ex[c] = e;
+#pragma unroll
+  for (int q = 0; q < Q; ++q) {
+    int d0[S], d1[S];
+    digits7(x[2 * q], e, d0);
+    digits7(x[2 * q + 1], e, d1);
+#pragma unroll
+    for (int s = 0; s < S; ++s)
+      *reinterpret_cast<__nv_bfloat162*>(&SP[((size_t)s * ncols + c) * SK + 64 * q + 2 * lane]) =
+          __floats2bfloat162_rn((float)d0[s], (float)d1[s]);
+  }
 }
 
 static int map_slices(CUtensorMap* map, const void* base, int n, int K, int box_rows) {
@@ -724,7 +826,7 @@ int potrf_split(int n, double* A, int lda, int* info, void* work, cudaStream_t s
   int dev = 0, nsm = 152;
   JMG_CUDA(cudaGetDevice(&dev));
   JMG_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-  JMG_TRY(ensure_smem(k_oz_syrk, SMEM));
+  JMG_TRY(ensure_smem(k_oz_update<false>, SMEM));
   JMG_TRY(ensure_smem(k_oz_diag, diag64::SMEM));
   CUtensorMap pa, pb, oa, ob;
   JMG_TRY(map_slices(&pa, panel, n, PW, BM));
@@ -737,9 +839,9 @@ int potrf_split(int n, double* A, int lda, int* info, void* work, cudaStream_t s
                     const int* ex) -> int {
     const int TI = cdiv(n - r0, BM), TJ = cdiv(ncols, BN);
     const long long nt = tile_count(TI, TJ);
-    k_oz_syrk<<<(int)std::min<long long>(nt, nsm), THREADS, SMEM, s>>>(
-        ma, mb, A, lda, n, r0, ncols, nkb, ex, TI, TJ, (int)nt, std::min(PW, n - r0), info,
-        g_wait_ns);
+    k_oz_update<false><<<(int)std::min<long long>(nt, nsm), THREADS, SMEM, s>>>(
+        ma, mb, A + (size_t)r0 * lda + r0, lda, n, r0, n, r0, n - r0, ncols, nkb, ex + r0, ex + r0, TI,
+        TJ, (int)nt, std::min(PW, n - r0), r0, info, nullptr, g_wait_ns);
     return launched();
   };
   // the first diagonal block; every update leaves the next one factored
@@ -768,6 +870,109 @@ int potrf_split(int n, double* A, int lda, int* info, void* work, cudaStream_t s
                                                                   rowmax, strip, e_out, info);
     JMG_TRY(launched());
     JMG_TRY(update(oa, ob, kend, n - kend, p.NB / 64, e_out));
+  }
+  return JMG_OK;
+}
+
+// ---------------------------------------------------------------------------
+// Solves with many right-hand sides: (L L^T) X = B, FP64.  Blocks of SK rows: the
+// diagonal block by the one-launch substitution (k_trsv.cu), everything behind it by
+// one tensor-core update from exact slices,
+//   forward   B_rest -= L[rest, block] Y_block,
+//   backward  B_rest -= L[block, rest]^T X_block,
+// in place of FP64 products on the CUDA cores, which bound the one-launch solves from
+// about 16 right-hand sides on.  In the backward direction row k of the block is scaled
+// by 2^-sc[k] in L and 2^sc[k] in X (sc: the row's exponent), so that a badly scaled A =
+// D G D costs nothing (the forward one is scaled by rows already).
+namespace {
+struct SolvePlan {
+  int nb;
+  size_t strip, exr, cols, exc, bmax, sc, total;
+};
+SolvePlan solve_plan(int n, int nrhs) {
+  SolvePlan p{};
+  p.nb = cdiv(n, ozf::SK);
+  size_t off = 0;
+  auto take = [&](size_t b) {
+    const size_t at = off;
+    off = round_up(off + b, 256);
+    return at;
+  };
+  p.strip = take((size_t)ozf::S * n * ozf::SK * 2);
+  p.exr = take(sizeof(int) * (size_t)n);
+  p.cols = take((size_t)ozf::S * nrhs * ozf::SK * 2);
+  p.exc = take(sizeof(int) * round_up((size_t)nrhs, 64));
+  p.bmax = take(sizeof(unsigned long long) * (size_t)n * p.nb);
+  p.sc = take(sizeof(int) * (size_t)n);
+  p.total = off;
+  return p;
+}
+}  // namespace
+
+size_t ozs_workspace(int n, int nrhs) {
+  // Worth it where the one-launch solves are bound by their products.  Both directions,
+  // one launch each / blocked: n = 4100, 64 right-hand sides 2.74 / 2.59 ms; 8192, 33:
+  // 7.25 / 5.04; 16384, 16: 10.6 / 10.9; 16384, 20: 17.9 / 10.9; 16384, 64: 35.2 / 11.1;
+  // 12001, 100: 37.1 / 8.3.
+  if (nrhs <= 16 || n < 4096 || (n < 8192 && (long long)n * nrhs < 250000)) return 0;
+  return solve_plan(n, nrhs).total;
+}
+
+int solve_split(int n, int nrhs, const double* L, int lda, double* B, int ldb, int* sync,
+                int* info, void* work, cudaStream_t s) {
+  using namespace ozf;
+  const SolvePlan p = solve_plan(n, nrhs);
+  char* w = static_cast<char*>(work);
+  __nv_bfloat16* strip = reinterpret_cast<__nv_bfloat16*>(w + p.strip);
+  __nv_bfloat16* cols = reinterpret_cast<__nv_bfloat16*>(w + p.cols);
+  int* exr = reinterpret_cast<int*>(w + p.exr);
+  int* exc = reinterpret_cast<int*>(w + p.exc);
+  unsigned long long* bmax = reinterpret_cast<unsigned long long*>(w + p.bmax);
+  int* sc = reinterpret_cast<int*>(w + p.sc);
+  int dev = 0, nsm = 152;
+  JMG_CUDA(cudaGetDevice(&dev));
+  JMG_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+  JMG_TRY(ensure_smem(k_oz_update<true>, SMEM));
+  CUtensorMap mq;
+  JMG_TRY(map_slices(&mq, cols, nrhs, SK, BN));
+  k_oz_block_max<<<dim3(cdiv(n, 256), p.nb), 256, 0, s>>>(L, lda, n, bmax);
+  JMG_TRY(launched());
+  k_oz_row_scale<<<cdiv(n, 256), 256, 0, s>>>(n, p.nb, bmax, sc);
+  JMG_TRY(launched());
+  // C (m x nrhs, head of B + row0) -= strip cols^T; strip rows rA.. of nA per slice
+  auto update = [&](const CUtensorMap& mp, int nA, int rA, int row0, int m) -> int {
+    const int TI = cdiv(m, BM), TJ = cdiv(nrhs, BN), nt = TI * TJ;
+    k_oz_update<true><<<std::min(nt, nsm), THREADS, SMEM, s>>>(
+        mp, mq, B + row0, ldb, nA, rA, nrhs, 0, m, nrhs, SK / BK, exr + rA, exc, TI, TJ, nt, 0, 0,
+        info, sync, g_wait_ns);
+    return launched();
+  };
+  CUtensorMap mp;
+  JMG_TRY(map_slices(&mp, strip, n, SK, BM));
+  for (int b = 0; b < p.nb; ++b) {
+    const int k0 = b * SK, kb = std::min(SK, n - k0), k1 = k0 + kb;
+    JMG_TRY(trsv_block(kb, nrhs, L + (size_t)k0 * lda + k0, lda, B + k0, ldb, 0, b > 0, sync,
+                       info, s));
+    if (k1 >= n) break;
+    k_oz_strip<<<dim3(cdiv(n - k1, 32), SK / 64), 256, 0, s>>>(L, lda, n, k0, k1, SK,
+                                                              bmax + (size_t)b * n, strip, exr, info);
+    JMG_TRY(launched());
+    k_oz_cut_cols<<<cdiv(nrhs, 8), 256, 0, s>>>(B + k0, ldb, kb, nrhs, sc, 0, cols, exc);
+    JMG_TRY(launched());
+    JMG_TRY(update(mp, n, k1, k1, n - k1));
+  }
+  for (int b = p.nb - 1; b >= 0; --b) {
+    const int k0 = b * SK, kb = std::min(SK, n - k0);
+    JMG_TRY(trsv_block(kb, nrhs, L + (size_t)k0 * lda + k0, lda, B + k0, ldb, 1, 1, sync,
+                       info, s));
+    if (k0 == 0) break;
+    k_oz_cut_cols<<<cdiv(k0, 8), 256, 0, s>>>(L + k0, lda, kb, k0, sc + k0, -1, strip, exr);
+    JMG_TRY(launched());
+    k_oz_cut_cols<<<cdiv(nrhs, 8), 256, 0, s>>>(B + k0, ldb, kb, nrhs, sc + k0, 1, cols, exc);
+    JMG_TRY(launched());
+    CUtensorMap mt;
+    JMG_TRY(map_slices(&mt, strip, k0, SK, BM));
+    JMG_TRY(update(mt, k0, 0, 0, k0));
   }
   return JMG_OK;
 }

@@ -27,8 +27,9 @@
 // through counters in shared memory, no CTA-wide barrier.  A step takes 3.9 us up to
 // 16 right-hand sides (28-32 us with one lane per right-hand side substituting and
 // barriers between the phases): both directions at n = 12288, 8 right-hand sides,
-// 24.3 -> 3.6 ms.  From 32 right-hand sides on the helpers' products bound it
-// (n = 16384, 64: 42.8 -> 35.1 ms, 0.98 TFLOP/s of 1.1).
+// 24.3 -> 3.6 ms.  From 17 right-hand sides on the helpers' products bound it
+// (n = 16384, 64: 42.8 -> 35.1 ms, 0.98 TFLOP/s of 1.1); large solves then run blocked,
+// with their products on the tensor cores (solve_split in k_ozpotrf.cu).
 //
 // Roles come from an atomic ticket in order (tickets below the number of leaders
 // NL lead; ticket t helps block LAG + t - NL), so the leaders are running before
@@ -492,19 +493,18 @@ size_t trsv_sync_ints(int n, int nrhs) {
   return 1 + (size_t)groups * (1 + trsv_slots(nrhs) + cdiv(std::max(n, 1), trsv::NBK));
 }
 
+// keep_err: the error word stays as the launches before left it
 template <typename T, int NR>
-static int trsv_launch(int n, int nrhs, const T* L, int lda, T* B, int ldb, int trans, int* sync,
-                       int* info, cudaStream_t s, int hold) {
+static int trsv_launch(int n, int nrhs, const T* L, int lda, T* B, int ldb, int trans, int keep_err,
+                       int* sync, int* info, cudaStream_t s, int hold) {
   const int groups = cdiv(nrhs, trsv::GR), nblk = cdiv(n, trsv::NBK);
   int* err = sync;
   int* tickets = sync + 1;
   int* done = tickets + groups;
   const int slots = trsv_slots(nrhs);
   int* pflag = done + (size_t)groups * slots;
-  // the forward solve clears the error word with the rest; the backward solve
-  // keeps it, so that it returns at once after a forward solve that gave up
-  JMG_CUDA(cudaMemsetAsync(sync + (trans ? 1 : 0), 0,
-                           sizeof(int) * (trsv_sync_ints(n, nrhs) - (trans ? 1 : 0)), s));
+  JMG_CUDA(cudaMemsetAsync(sync + keep_err, 0,
+                           sizeof(int) * (trsv_sync_ints(n, nrhs) - keep_err), s));
   const size_t smem = sizeof(trsv::Smem<T, NR>);
   auto k = k_trsv_persist<T, NR>;
   JMG_TRY(ensure_smem(k, (int)smem));
@@ -528,15 +528,22 @@ static int trsv_launch(int n, int nrhs, const T* L, int lda, T* B, int ldb, int 
   return JMG_OK;
 }
 
-template <>
-int launch_trsv_persist<double>(int n, int nrhs, const double* L, int lda, double* B, int ldb,
-                                int trans, int* sync, int* info, cudaStream_t s, int hold) {
+int trsv_block(int n, int nrhs, const double* L, int lda, double* B, int ldb, int trans,
+               int keep_err, int* sync, int* info, cudaStream_t s, int hold) {
   if (n <= 0 || nrhs <= 0) return JMG_OK;
   // Up to 16 right-hand sides every one gets a leader of its own (the chain sets
   // the time); beyond, the helpers' products do, and four share a leader.
   if (nrhs <= trsv::GR)
-    return trsv_launch<double, 1>(n, nrhs, L, lda, B, ldb, trans, sync, info, s, hold);
-  return trsv_launch<double, 4>(n, nrhs, L, lda, B, ldb, trans, sync, info, s, hold);
+    return trsv_launch<double, 1>(n, nrhs, L, lda, B, ldb, trans, keep_err, sync, info, s, hold);
+  return trsv_launch<double, 4>(n, nrhs, L, lda, B, ldb, trans, keep_err, sync, info, s, hold);
+}
+
+// the forward solve clears the error word with the rest; the backward solve keeps
+// it, so that it returns at once after a forward solve that gave up
+template <>
+int launch_trsv_persist<double>(int n, int nrhs, const double* L, int lda, double* B, int ldb,
+                                int trans, int* sync, int* info, cudaStream_t s, int hold) {
+  return trsv_block(n, nrhs, L, lda, B, ldb, trans, trans ? 1 : 0, sync, info, s, hold);
 }
 
 }  // namespace jmg

@@ -77,6 +77,10 @@ int launch_trsv_persist<double>(int n, int nrhs, const double* L, int lda, doubl
 template <>
 int launch_trsv_persist<float>(int n, int nrhs, const float* L, int lda, float* B, int ldb,
                                int trans, int* sync, int* info, cudaStream_t s, int hold);
+// One direction on FP64 data; keep_err != 0 leaves the error word as earlier launches of
+// the same solve left it (launch_trsv_persist: kept by the backward direction).
+int trsv_block(int n, int nrhs, const double* L, int lda, double* B, int ldb, int trans,
+               int keep_err, int* sync, int* info, cudaStream_t s, int hold = 0);
 // (L L^T) X = B: forward then backward with launch_trsv_persist.
 template <typename T>
 int solve_llt(int n, int nrhs, const T* L, int lda, T* B, int ldb, int* sync, int* info,
@@ -90,6 +94,14 @@ int solve_llt(int n, int nrhs, const T* L, int lda, T* B, int ldb, int* sync, in
 size_t ozf_workspace(int n);
 // Cholesky factorisation in place; work: ozf_workspace(n) bytes, 256-byte aligned.
 int potrf_split(int n, double* A, int lda, int* info, void* work, cudaStream_t s);
+
+// Scratch of solve_split for this shape; 0 where the one-launch solves are the better
+// ones.
+size_t ozs_workspace(int n, int nrhs);
+// (L L^T) X = B on FP64 data, blocked, with split updates; sync and info as solve_llt,
+// work: ozs_workspace bytes, 256-byte aligned.
+int solve_split(int n, int nrhs, const double* L, int lda, double* B, int ldb, int* sync,
+                int* info, void* work, cudaStream_t s);
 
 // ---- mixed-precision helpers
 // W (FP32, ldw) <- lower(A) (FP64), lower triangle only; plus shift on the diagonal.

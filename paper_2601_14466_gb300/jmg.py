@@ -239,7 +239,7 @@ def potrs_(L: torch.Tensor, B: torch.Tensor) -> torch.Tensor:
         raise TypeError("potrs_: L and B must have the same dtype")
     pl, lda = _colmajor(L, "L")
     pb, ldb = _colmajor(B, "B")
-    work = workspace(OP_POTRS, L.shape[0], B.shape[1], None, L.device)
+    work = workspace(OP_POTRS, L.shape[0], B.shape[1], None, L.device, dt)
     st = load().jmg_potrs(L.shape[0], B.shape[1], pl, lda, pb, ldb, dt, work.data_ptr(),
                           work.numel(), _stream(L.device))
     _chk(st, "jmg_potrs")

@@ -120,4 +120,47 @@ def test_fast_scratch_is_never_less_and_only_more_where_it_helps():
                 fast = int(lib.jmg_workspace_fast(op, n, 3, dt, ctypes.byref(o)))
                 assert fast >= need
                 more = prec == "fp64" and dt == jmg.JMG_F64 and n > 64 and op != jmg.OP_POTRS
+                # (three right-hand sides: the solves never want more)
                 assert (fast > need + 255) == more
+
+
+def test_fast_scratch_of_the_solves_follows_their_shape():
+    lib = jmg.load()
+    for n, nrhs, more in ((4095, 100, False), (4096, 61, False), (4096, 62, True), (8192, 16, False),
+                          (8192, 17, True), (65536, 17, True), (100000, 1, False)):
+        need = jmg.workspace_size(jmg.OP_POTRS, n, nrhs)
+        fast = int(lib.jmg_workspace_fast(jmg.OP_POTRS, n, nrhs, jmg.JMG_F64, None))
+        assert (fast > need) == more and fast >= need
+        assert int(lib.jmg_workspace_fast(jmg.OP_POTRS, n, nrhs, jmg.JMG_F32, None)) == \
+            jmg.workspace_size(jmg.OP_POTRS, n, nrhs, None, jmg.JMG_F32)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n,nrhs,pad", [(4096, 62, 0), (4097, 64, 1), (4608, 65, 0), (5121, 49, 2)])
+@pytest.mark.parametrize("scaled", [False, True])
+def test_split_solve_matches_substitution(n, nrhs, pad, scaled):
+    # rows of L eight decades apart leave D X as it is for L -> D L, B -> D B: the same
+    # bound holds for it (substitution: 64 n u as in the other solve tests; the slices
+    # keep 2^-56 of a row's and a column's largest element in each block of 512)
+    L = inputs.lower_factor(n, seed=3)
+    B = inputs.uniform(n, nrhs, seed=4)
+    Xo = oracle.potrs(np.asfortranarray(L.numpy()), B.numpy())
+    d = torch.logspace(-4, 4, n, dtype=torch.float64)[torch.randperm(n, generator=torch.Generator().manual_seed(1))] \
+        if scaled else torch.ones(n, dtype=torch.float64)
+    lda, ldb = n + pad, n + 3
+    Lb = torch.full((n, lda), float("nan"), dtype=torch.float64, device=DEV)
+    Lb[:, :n] = (torch.tril(d[:, None] * L) + torch.triu(torch.full_like(L, float("nan")), 1)).t().to(DEV)
+    Bb = torch.full((nrhs, ldb), float("nan"), dtype=torch.float64, device=DEV)
+    Bb[:, :n] = (d[:, None] * B).t().to(DEV)
+    lib = jmg.load()
+    nbytes = int(lib.jmg_workspace_fast(jmg.OP_POTRS, n, nrhs, jmg.JMG_F64, None))
+    assert nbytes > jmg.workspace_size(jmg.OP_POTRS, n, nrhs)
+    work = torch.empty(nbytes, dtype=torch.uint8, device=DEV)
+    st = lib.jmg_potrs(n, nrhs, Lb.data_ptr(), lda, Bb.data_ptr(), ldb, jmg.JMG_F64, work.data_ptr(),
+                       nbytes, torch.cuda.current_stream().cuda_stream)
+    assert st == 0
+    torch.cuda.synchronize()
+    assert int(work[:4].view(torch.int32).item()) == 0
+    assert torch.isnan(Bb[:, n:]).all()
+    X = Bb[:, :n].t().cpu().numpy() * d.numpy()[:, None]
+    assert np.abs(X - Xo).max() <= 64 * n * U64 * max(1.0, np.abs(Xo).max())
