@@ -138,21 +138,26 @@ JMG_DEV double scaled_double(long long v, int ex) {
 }
 
 // ---------------------------------------------------------------------------
-// Diagonal block of kb <= 64 columns, in place, by one CTA of THREADS threads.  An
-// FP64 warp instruction holds its SM quarter's pipe for ~64 clocks, and the pivots
-// are a serial chain: warp 0 keeps column j in registers (two rows per lane) and in
+// Diagonal block of kb <= 64 columns, in place, by one CTA of THREADS threads.  A
+// dependent FP64 instruction waits 68 clocks and the pivots are a serial chain:
+// warp 0 keeps column j in registers (two rows per lane) and in
 // step j updates column j+1, takes pivot j+1 (its reciprocal in integers) and hands
 // u_j = column j / a_jj to the trailing warps (named barrier 1); those apply
 // a_rc -= a_rj u_c to columns j+2 .. , column j+2 first, which they release
-// (named barrier 2: the chain's input of step j+1).  The trailing work sets the
-// time of the first columns and the chain that of the later ones, so the three
-// further warps of the chain's quarter help only for j < J0 (the barriers' counts
-// change there with them).  Each barrier is passed the same number of times on both
-// sides, and nothing leaves the loop early: the first pivot that is not positive is
+// (named barrier 2: the chain's input of step j+1).  Each barrier is passed the same
+// number of times on both sides (their counts shrink with the trailing warps), and
+// nothing leaves the loop early: the first pivot that is not positive is
 // recorded and the columns from it on are dropped.
 namespace diag64 {
-constexpr int TRAIL = 384, MORE = 96;  // threads of warps 1 .. 15 off / on the chain's quarter
+// Trailing threads in step j: the trailing work sets the time of the first columns, the
+// chain that of the later ones, where every further warp in the queue of the SM's one
+// FP64 pipe (16 clocks a warp instruction) can hold it up.
 constexpr int J0 = 20;
+JMG_DEV int trail(int j) { return j < J0 ? 480 : 384; }
+// Participants of barrier 1 in step j: the chain warp and every thread that worked in
+// step j-1 (one that leaves arrives there once more, so that the others, who take its
+// elements over, see its last stores).
+JMG_DEV int count1(int j) { return 32 + trail(j > 0 ? j - 1 : 0); }
 constexpr int LD = PW + 1;
 constexpr int NEL = PW * (PW + 1) / 2;
 constexpr int SMEM = (PW * LD + 2 * PW + 2 * PW) * 8 + NEL * 2;
@@ -207,7 +212,7 @@ JMG_DEV void diag_body(double* sm_d64, double* __restrict__ A, int lda, int kb, 
       const int j1 = j + 1;
       const double a1 = __shfl_sync(0xffffffffu, j1 < 32 ? lo : hi, j1 & 31);
       const double v = a1 * w;  // u of row j+1
-      if (j > 0) bar_sync(2, j - 1 < J0 ? 32 + TRAIL + MORE : 32 + TRAIL);  // column j+1 done to j-1
+      if (j > 0) bar_sync(2, 32 + trail(j - 1));  // column j+1 done to j-1
       double* cn = &s64[j1 * LD];
       double nlo = cn[lane], nhi = cn[lane + 32];
       double* u = &s_u[(j & 1) * PW];
@@ -221,7 +226,7 @@ JMG_DEV void diag_body(double* sm_d64, double* __restrict__ A, int lda, int kb, 
         cn[lane] = nlo;
         cn[lane + 32] = nhi;
         __syncwarp();
-        bar_arrive(1, j < J0 ? 32 + TRAIL + MORE : 32 + TRAIL);
+        bar_arrive(1, count1(j));
         w = pivot_rcp(d, &bad);
       } else {
         nhi = fma(-hi, v, nhi);
@@ -229,7 +234,7 @@ JMG_DEV void diag_body(double* sm_d64, double* __restrict__ A, int lda, int kb, 
         u[lane + 32] = hi * w;
         cn[lane + 32] = nhi;
         __syncwarp();
-        bar_arrive(1, j < J0 ? 32 + TRAIL + MORE : 32 + TRAIL);
+        bar_arrive(1, count1(j));
         w = pivot_rcp(d, &bad);
       }
       if (bad && fj < 0) fj = j1;
@@ -238,14 +243,15 @@ JMG_DEV void diag_body(double* sm_d64, double* __restrict__ A, int lda, int kb, 
     }
     if (lane == 0 && fj >= 0) fail = fj + 1;
   } else if (warp < 16) {
-    // index among the trailing warps, those of the chain's quarter last
-    const bool more = (warp & 3) == 0;
-    const int tq = (more ? 12 + warp / 4 - 1 : warp - 1 - warp / 4) * 32 + lane;
+    const int tq = t - 32;  // index among the trailing threads
     for (int j = 0; j + 1 < kb; ++j) {
-      if (more && j >= J0) break;
-      const int nt = j < J0 ? TRAIL + MORE : TRAIL;
+      const int nt = trail(j);
       __syncwarp();
-      bar_sync(1, 32 + nt);  // u_j and column j in place
+      if (tq >= nt) {
+        bar_arrive(1, count1(j));
+        break;
+      }
+      bar_sync(1, count1(j));  // u_j and column j in place
       const double* cj = &s64[j * LD];
       const double* uj = &s_u[(j & 1) * PW];
       if (j + 2 < kb) {
