@@ -3,10 +3,12 @@
 // Paper: "Software design" -- the potrs workflow (Cholesky potrf followed by
 // potrs, optional log det) issued as one call on the framework's stream.
 //
-// Plain path (prec NATIVE, FP64): right-looking blocked Cholesky in place
-//   for each diagonal block k:  potf2 (FP64)  ->  panel TRSM (FP64)
-//                               ->  trailing SYRK update (FP64 CUDA cores)
-//   then blocked forward / back substitution.
+// Plain path (prec NATIVE): right-looking blocked Cholesky in place
+//   for each diagonal block k:  potf2  ->  panel TRSM  ->  trailing SYRK update
+//   then blocked forward / back substitution.  FP64 data with enough scratch
+//   (jmg_workspace_fast) take k_ozpotrf.cu's factorisation and, from a size on, its
+//   solves: the same steps with the products on the tensor cores from exact slices.
+//   With less, and for FP32 data, the products run on the CUDA cores.
 // Mixed path (prec BF16 / FP16): the same loop on an FP32 working copy W of
 //   lower(A) with FP64 diagonal blocks, an FP32 panel TRSM and tensor-core
 //   trailing updates on 16-bit split words; the FP32 factor then

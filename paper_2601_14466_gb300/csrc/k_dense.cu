@@ -967,18 +967,23 @@ int launch_residual(int n, int nrhs, const double* A, int lda, const double* X, 
 //   rowmax[i] = max_j |a_ij| truncated to its upper 32 bits (sign, exponent
 //               and 20 leading fraction bits): the same binary exponent as the
 //               maximum, which is all the row scales of the split residual use
-// over the full row j = 0..n-1.  One CTA per strip of 32 columns j reads them
+// over the full row j = 0..n-1.  One CTA per strip of 16 columns j reads them
 // down from the diagonal in 1024-row chunks (long contiguous runs of each
 // column, 16 loads in flight per thread).  Entry a_rj (r > j) adds to row r --
 // kept per thread for its four rows of the chunk and flushed with one atomic
 // per row and chunk -- and to row j (its mirror), kept per thread for the
-// strip's 32 columns and reduced across the CTA at the end; a_jj adds once.
+// strip's 16 columns and reduced across the CTA at the end; a_jj adds once.
 // The maxima are taken on the upper 32 bits of |a| as unsigned integers,
 // which order like the values (NaN above every finite value).
-__global__ void __launch_bounds__(256, 1) k_row_stats(int n, const double* __restrict__ A,
+// Bound by the FP64 pipe (one warp instruction per 16 clocks and SM), so an entry
+// costs its two additions and nothing else there (its sign is cleared in the upper
+// word), and strips of 16 columns let two CTAs share an SM: n = 16384 1326 -> 607 us
+// (strips of 32, one CTA, a third FP64 operation for the sign).
+constexpr int STATS_W = 16;
+__global__ void __launch_bounds__(256, 2) k_row_stats(int n, const double* __restrict__ A,
                                                       int lda, double* __restrict__ rowsum,
                                                       double* __restrict__ rowmax) {
-  constexpr int W = 32, U = 4, TH = 256, JB = 4;
+  constexpr int W = STATS_W, U = 4, TH = 256, JB = 4;
   __shared__ double red_s[TH / 32][W];
   __shared__ unsigned red_m[TH / 32][W];
   const int j0 = blockIdx.x * W;
@@ -993,27 +998,31 @@ __global__ void __launch_bounds__(256, 1) k_row_stats(int n, const double* __res
     unsigned rm[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) rs[u] = 0.0, rm[u] = 0u;
-    const double* base = A + (size_t)j0 * lda + rb + t;  // (column j0, row rb + t)
+    const double* col = A + (size_t)j0 * lda + rb + t;  // (column j0, row rb + t)
+    const bool inner = rb >= j0 + W && rb + TH * U <= n;  // all rows below the strip's diagonal
+    const int rt = rb + t - j0, rows = n - (rb + t);      // row in the strip, rows left
 #pragma unroll
     for (int jb = 0; jb < W; jb += JB) {
       double v[JB][U];
 #pragma unroll
-      for (int q = 0; q < JB; ++q)  // JB x U independent loads
+      for (int q = 0; q < JB; ++q) {  // JB x U independent loads
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-          const int j = j0 + jb + q, r = rb + t + TH * u;
-          v[q][u] = (jb + q < jn && r >= j && r < n) ? fabs(base[(jb + q) * lda + TH * u]) : 0.0;
+          const int i = TH * u;
+          v[q][u] = (inner && jn == W) || (jb + q < jn && rt + i >= jb + q && i < rows) ? col[i] : 0.0;
         }
+        col += lda;
+      }
 #pragma unroll
       for (int q = 0; q < JB; ++q)
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-          const int j = j0 + jb + q, r = rb + t + TH * u;
-          const unsigned hi = (unsigned)__double2hiint(v[q][u]);
-          rs[u] += v[q][u];
+          const unsigned hi = (unsigned)__double2hiint(v[q][u]) & 0x7fffffffu;
+          const double av = __hiloint2double((int)hi, __double2loint(v[q][u]));
+          rs[u] += av;
           rm[u] = max(rm[u], hi);
-          if (r > j) {
-            cs[jb + q] += v[q][u];
+          if (inner || rt + TH * u > jb + q) {
+            cs[jb + q] += av;
             cm[jb + q] = max(cm[jb + q], hi);
           }
         }
@@ -1027,7 +1036,7 @@ __global__ void __launch_bounds__(256, 1) k_row_stats(int n, const double* __res
       }
     }
   }
-  // the mirrored part of rows j0 .. j0+31: reduce the column sums over the CTA
+  // the mirrored part of the strip's rows: reduce the column sums over the CTA
 #pragma unroll
   for (int jj = 0; jj < W; ++jj) {
     double a = cs[jj];
@@ -1060,7 +1069,7 @@ int launch_row_stats(int n, const double* A, int lda, double* rowsum, double* ro
   if (n <= 0) return JMG_OK;
   if (rowsum) JMG_CUDA(cudaMemsetAsync(rowsum, 0, sizeof(double) * n, s));
   if (rowmax) JMG_CUDA(cudaMemsetAsync(rowmax, 0, sizeof(double) * n, s));
-  k_row_stats<<<cdiv(n, 32), 256, 0, s>>>(n, A, lda, rowsum, rowmax);
+  k_row_stats<<<cdiv(n, STATS_W), 256, 0, s>>>(n, A, lda, rowsum, rowmax);
   return launched();
 }
 

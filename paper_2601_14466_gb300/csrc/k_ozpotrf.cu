@@ -553,12 +553,12 @@ __global__ void __launch_bounds__(THREADS, 1)
 
 // ---------------------------------------------------------------------------
 // Panel solve X L_kk^T = A21 (64 columns) and its slices.  G lanes share a row,
-// each holding the column pairs {2 (g + G i), 2 (g + G i) + 1}; the FP64 pipe
-// takes one warp instruction per ~64 clocks and SM quarter, so the row is spread
-// over just enough lanes to fill the chip with eight warps per SM (one warp per
-// quarter left half the issue slots to instruction-fetch and latency stalls).  The solve runs on unscaled columns
-// with Lh[j][l] = L_lj / L_jj (a_l -= a_j Lh[j][l]), the scaling by 1 / L_jj
-// comes last: one FP64 instruction per element and step, nothing else.
+// each holding the column pairs {2 (g + G i), 2 (g + G i) + 1}; an SM's FP64 pipe
+// takes one warp instruction per 16 clocks and a dependent one waits 68, so the row
+// is spread over just enough lanes to fill the chip with eight warps per SM (four left
+// half the pipe idle).  The solve runs on unscaled columns with Lh[j][l] = L_lj / L_jj
+// (a_l -= a_j Lh[j][l]), the scaling by 1 / L_jj comes last: one FP64 instruction per
+// element and step, nothing else.
 template <int G>
 __global__ void __launch_bounds__(PT) k_oz_panel(double* __restrict__ A, int lda, int n, int k,
                                                   __nv_bfloat16* __restrict__ SP,
