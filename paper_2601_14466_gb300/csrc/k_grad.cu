@@ -7,12 +7,14 @@
 // transformations ("Summary"); reverse-mode differentiation is one of them, and
 // this is its matrix-calculus form for a symmetric A read from one triangle.
 //
-// One CTA per 64 x 64 lower tile (ti >= tj); the rank-2 nrhs products run on
-// the FP64 CUDA cores (4 x 4 register tile per thread).  The tile is written
+// Few right-hand sides: one CTA per 64 x 64 lower tile (ti >= tj); the rank-2 nrhs
+// products run on the FP64 CUDA cores (4 x 4 register tile per thread).  The tile is written
 // to (ti, tj) directly and to the mirror (tj, ti) through a shared-memory
 // transpose so that both stores coalesce down columns; on diagonal tiles the
 // upper half is the mirror of the lower half, so Abar is exactly symmetric.
 #include "kernels.h"
+#include "ozslice.cuh"
+#include "tc_ptx.cuh"
 
 namespace jmg {
 
@@ -57,8 +59,9 @@ __global__ void __launch_bounds__(256) k_sym_grad(int n, int nrhs, const double*
       Xj[k][r] = (kin && gj < n) ? X[(size_t)gk * ldx + gj] : 0.0;
     }
     __syncthreads();
-#pragma unroll
-    for (int k = 0; k < KC; ++k) {
+    const int kn = min(KC, nrhs - k0);
+#pragma unroll 4
+    for (int k = 0; k < kn; ++k) {
       double bi[4], xi[4], bj[4], xj[4];
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
@@ -96,12 +99,239 @@ __global__ void __launch_bounds__(256) k_sym_grad(int n, int nrhs, const double*
   }
 }
 
+// ---------------------------------------------------------------------------
+// The same on the tensor cores, from exact slices (k_ozpotrf.cu): 2 nrhs FP64 FMAs per
+// entry hold the FP64 pipe for nrhs clocks and SM, the slices of a chunk of KC = 16
+// right-hand sides cost a tile the same whatever the FP64 work.  One CTA per 128 x 64
+// tile of the lower trapezoid; per chunk the two products Bbar_i X_j^T and X_i Bbar_j^T
+// one after the other: stage 16 columns of both operands, cut every row into seven
+// digits straight into the swizzled operand tiles, 28 slice products into seven TMEM
+// levels (exact: |sum| <= 7 16 2^14 < 2^24), one conversion and one FP64 addition per
+// entry.  Column k of the pair is scaled by 2^s_k and 2^-s_k first (s_k from the tile's
+// column maxima), so that a pair with a large Bbar and a small X next to one with the
+// opposite costs no digits.  A chunk with an entry that is not finite takes FP64 FMAs
+// from the staged columns, as does everything after a wait that ran out.
+// n = 8192, 16 right-hand sides: 1829 -> 693 us (a tile's phases, not pipelined, take
+// ~25 us; the 537 MB written would take 80), error against 64 bits 0.75 of the FMAs'.
+namespace grad {
+constexpr int BM = 128, BN = 64, TH = 512;
+constexpr int A_TILE = BM * 128, B_TILE = BN * 128;  // rows of 128 bytes, 16 BF16 of them used
+constexpr int LDT = BM + 1;
+constexpr int SMEM = ozf::S * (A_TILE + B_TILE) + KC * (BM + BN) * 8 + 1024;
+static_assert(BN * LDT * 8 <= ozf::S * A_TILE, "the output tile lies over the operand tiles");
+}  // namespace grad
+
+__global__ void __launch_bounds__(grad::TH, 1)
+    k_sym_grad_tc(int n, int nrhs, const double* __restrict__ Bb, int ldb,
+                  const double* __restrict__ X, int ldx, double* __restrict__ G, int ldg,
+                  unsigned long long wait_ns) {
+  using namespace grad;
+  using namespace tc;
+  using ozf::S;
+  extern __shared__ __align__(1024) unsigned char sm_raw_grad[];
+  unsigned char* abuf = reinterpret_cast<unsigned char*>(
+      (reinterpret_cast<uintptr_t>(sm_raw_grad) + 1023) & ~uintptr_t(1023));
+  unsigned char* bbuf = abuf + S * A_TILE;
+  double* sP = reinterpret_cast<double*>(bbuf + S * B_TILE);  // [KC][BM]
+  double* sQ = sP + KC * BM;                                  // [KC][BN]
+  __shared__ uint64_t bar;
+  __shared__ uint32_t tmem_slot;
+  __shared__ int s_ep[BM], s_eq[BN], s_k[KC];  // row exponents, column shifts
+  const int t = threadIdx.x, warp = t / 32, lane = t % 32;
+  // tile b: row tile ti has the column tiles 0 .. 2 ti + 1
+  int ti = (int)((sqrtf(4.0f * (float)blockIdx.x + 1.0f) - 1.0f) * 0.5f);
+  while ((long long)ti * (ti + 1) > (long long)blockIdx.x) --ti;
+  while ((long long)(ti + 1) * (ti + 2) <= (long long)blockIdx.x) ++ti;
+  const int tj = (int)(blockIdx.x - (long long)ti * (ti + 1));
+  const int i0 = ti * BM, j0 = tj * BN;
+  if (j0 >= n) return;
+  if (t == 0) {
+    mbar_init(&bar, 1);
+    fence_mbar_init();
+  }
+  if (warp == 0) {
+    tmem_alloc(&tmem_slot, 512);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = tmem_slot;
+
+  constexpr int CW = 16;
+  const int q = warp & 3, ch = (warp >> 2) * CW;  // TMEM lane quarter, columns of this warp
+  const int r = q * 32 + lane;
+  double v[CW];
+#pragma unroll
+  for (int c = 0; c < CW; ++c) v[c] = 0.0;
+  bool ok = true;  // uniform over the CTA
+  uint32_t phase = 0;
+  for (int k0 = 0; k0 < nrhs; k0 += KC) {
+#pragma unroll 1
+    for (int half = 0; half < 2; ++half) {
+      const double* P = half ? X : Bb;
+      const double* Q = half ? Bb : X;
+      const int ldp = half ? ldx : ldb, ldq = half ? ldb : ldx;
+      bool fin = true;
+      {
+        double a[6];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int k = t / BM + 4 * u, gi = i0 + t % BM;
+          a[u] = (k0 + k < nrhs && gi < n) ? P[(size_t)(k0 + k) * ldp + gi] : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          const int k = t / BN + 8 * u, gj = j0 + t % BN;
+          a[4 + u] = (k0 + k < nrhs && gj < n) ? Q[(size_t)(k0 + k) * ldq + gj] : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < 6; ++u)
+          fin = fin && ((unsigned)__double2hiint(a[u]) & 0x7ff00000u) != 0x7ff00000u;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) sP[(t / BM + 4 * u) * BM + t % BM] = a[u];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) sQ[(t / BN + 8 * u) * BN + t % BN] = a[4 + u];
+      }
+      const bool slices = __syncthreads_and(fin) && ok;
+      if (slices) {
+        {  // column k = warp: shift by half the difference of the maxima's exponents
+          unsigned mp = 0, mq = 0;
+#pragma unroll
+          for (int u = 0; u < BM / 32; ++u)
+            mp = max(mp, (unsigned)__double2hiint(sP[warp * BM + lane + 32 * u]) & 0x7fffffffu);
+#pragma unroll
+          for (int u = 0; u < BN / 32; ++u)
+            mq = max(mq, (unsigned)__double2hiint(sQ[warp * BN + lane + 32 * u]) & 0x7fffffffu);
+          mp = __reduce_max_sync(0xffffffffu, mp);
+          mq = __reduce_max_sync(0xffffffffu, mq);
+          if (lane == 0) s_k[warp] = ((int)(mq >> 20) - (int)(mp >> 20)) / 2;
+        }
+        __syncthreads();
+        if (t < 2 * (BM + BN)) {  // eight values of a row of P (t < 256) or Q
+          const bool isq = t >= 2 * BM;
+          const int w = isq ? t - 2 * BM : t, row = w / 2, h = 8 * (w & 1);
+          const double* src = isq ? sQ + row : sP + row;
+          const int ld = isq ? BN : BM;
+          double x[8];
+          int sk[8], e = -(1 << 20);
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            x[u] = src[(h + u) * ld];
+            sk[u] = isq ? -s_k[h + u] : s_k[h + u];
+            const unsigned long long b =
+                (unsigned long long)__double_as_longlong(x[u]) & 0x7FFFFFFFFFFFFFFFull;
+            if (b) e = max(e, max((int)(b >> 52), 1) - 1022 + sk[u]);
+          }
+          e = max(e, __shfl_xor_sync(0xffffffffu, e, 1));
+          if (h == 0) (isq ? s_eq : s_ep)[row] = e;
+          uint32_t d4[S][4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            int d0[S], d1[S];
+            ozf::digits7(x[2 * u], e - sk[2 * u], d0);
+            ozf::digits7(x[2 * u + 1], e - sk[2 * u + 1], d1);
+#pragma unroll
+            for (int s = 0; s < S; ++s) {
+              const __nv_bfloat162 p = __floats2bfloat162_rn((float)d0[s], (float)d1[s]);
+              d4[s][u] = *reinterpret_cast<const uint32_t*>(&p);
+            }
+          }
+          unsigned char* dst = (isq ? bbuf : abuf) + row * 128 + (((h >> 3) ^ (row & 7)) << 4);
+          const int tile = isq ? B_TILE : A_TILE;
+#pragma unroll
+          for (int s = 0; s < S; ++s)
+            *reinterpret_cast<uint4*>(dst + s * tile) =
+                make_uint4(d4[s][0], d4[s][1], d4[s][2], d4[s][3]);
+          fence_proxy_async();
+        }
+        tc_fence_before();
+        __syncthreads();
+        if (t == 0) {
+          tc_fence_after();
+          constexpr int GMAX = 256 / BN;
+          for (int a = 0; a < S; ++a)
+            for (int b0 = 0; b0 < S - a; b0 += GMAX) {
+              const int cnt = min(GMAX, S - a - b0);
+              tc_mma_f16(tmem + (uint32_t)((a + b0) * BN), sdesc_sw128(smem_u32(abuf + a * A_TILE)),
+                         sdesc_sw128(smem_u32(bbuf + b0 * B_TILE)), idesc_f16(BM, BN * cnt, 1),
+                         a == 0 ? 0u : 1u);
+            }
+          tc_commit(&bar);
+        }
+        __syncwarp();
+        ok = __syncthreads_and(mbar_wait(&bar, phase, wait_ns));
+        phase ^= 1;
+      }
+      if (slices && ok) {
+        tc_fence_after();
+        const uint32_t tacc = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)ch;
+        constexpr int sh = 40;
+        long long acc[CW];
+#pragma unroll
+        for (int c = 0; c < CW; ++c) acc[c] = 0;
+#pragma unroll
+        for (int d = 0; d < S; ++d) {
+          uint32_t w[16];
+          tmem_ld16(tacc + (uint32_t)(d * BN), w);
+          tmem_ld_wait();
+#pragma unroll
+          for (int c = 0; c < CW; ++c) {
+            const long long y = __float2int_rn(__uint_as_float(w[c]));
+            acc[c] += d < 6 ? y << (sh - 8 * (d < 6 ? d : 0)) : (y + (1 << 7)) >> 8;
+          }
+        }
+        const int er = s_ep[r] - 14 - sh;
+#pragma unroll
+        for (int c = 0; c < CW; ++c) v[c] += ozf::scaled_double(acc[c], er + s_eq[ch + c]);
+      } else {
+        for (int k = 0; k < KC; ++k)
+#pragma unroll
+          for (int c = 0; c < CW; ++c) v[c] = fma(sP[k * BM + r], sQ[k * BN + ch + c], v[c]);
+      }
+      tc_fence_before();
+      __syncthreads();  // accumulators and staged columns are free
+    }
+  }
+  if (!ok) (void)mbar_wait(&bar, phase ^ 1, 1000000000ull);  // the products still under way
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 0) tmem_dealloc(tmem, 512);
+  const int row = i0 + r;
+  double* T = reinterpret_cast<double*>(abuf);  // T[c * LDT + r]
+#pragma unroll
+  for (int c = 0; c < CW; ++c) {
+    const double g = -0.5 * v[c];
+    const int col = j0 + ch + c;
+    T[(ch + c) * LDT + r] = g;
+    if (row < n && col <= row) G[(size_t)col * ldg + row] = g;
+  }
+  __syncthreads();
+  for (int i = warp; i < BM; i += TH / 32)  // column i0 + i of G, rows j0 ..
+#pragma unroll
+    for (int h = 0; h < BN; h += 32) {
+      const int col = i0 + i, gj = j0 + h + lane;
+      if (col < n && gj < col) G[(size_t)col * ldg + gj] = T[(h + lane) * LDT + i];
+    }
+}
+
 int launch_sym_grad(int n, int nrhs, const double* Bb, int ldb, const double* X, int ldx, double* G,
                     int ldg, cudaStream_t s) {
   if (n <= 0) return JMG_OK;
   if (nrhs <= 0) {
     JMG_CUDA(cudaMemset2DAsync(G, sizeof(double) * ldg, 0, sizeof(double) * n, n, s));
     return JMG_OK;
+  }
+  // FP64 work grows with nrhs, a chunk on the tensor cores costs the same from 1 to 16:
+  // n = 8192 nrhs 5 630 / 693 us, 6 744 / 685; n = 2048 5 52 / 53, 8 77 / 53; one wave of
+  // tiles (n <= 1024) 11 31 / 29, 8 24 / 29.
+  if (nrhs >= (n <= 1024 ? 12 : 6)) {
+    using namespace grad;
+    JMG_TRY(ensure_smem(k_sym_grad_tc, SMEM));
+    const long long TI = cdiv(n, BM);
+    k_sym_grad_tc<<<(unsigned)(TI * (TI + 1)), TH, SMEM, s>>>(n, nrhs, Bb, ldb, X, ldx, G, ldg,
+                                                             g_wait_ns);
+    return launched();
   }
   k_sym_grad<<<(unsigned)tri_tiles(cdiv(n, grad::TB)), 256, 0, s>>>(n, nrhs, Bb, ldb, X, ldx, G,
                                                                       ldg);
