@@ -105,12 +105,12 @@ static size_t plain_solve_bytes(int n, int nrhs) {
   return round_up(sizeof(int) * trsv_sync_ints(n, nrhs), 256);
 }
 
-// Side streams and events of the mixed path, created once per device on first
+// Side stream and events of the mixed path, created once per device on first
 // use and kept for the life of the process (a call made on another thread
 // shares them: events are re-recorded, which can only add dependencies).
 struct DevAux {
-  cudaStream_t hi = nullptr, lo = nullptr;  // high / low priority, non-blocking
-  cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
+  cudaStream_t lo = nullptr;  // low priority, non-blocking
+  cudaEvent_t ev[2] = {nullptr, nullptr};
 };
 static int dev_aux(DevAux** out) {
   static std::mutex mu;
@@ -120,12 +120,12 @@ static int dev_aux(DevAux** out) {
   if (dev < 0 || dev >= 64) return JMG_ERR_UNSUPPORTED;
   std::lock_guard<std::mutex> lock(mu);
   DevAux& a = aux[dev];
-  if (!a.hi) {
+  if (!a.lo) {
     int prio_lo = 0, prio_hi = 0;
     JMG_CUDA(cudaDeviceGetStreamPriorityRange(&prio_lo, &prio_hi));
+    for (auto& e : a.ev)
+      if (!e) JMG_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
     JMG_CUDA(cudaStreamCreateWithPriority(&a.lo, cudaStreamNonBlocking, prio_lo));
-    for (auto& e : a.ev) JMG_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-    JMG_CUDA(cudaStreamCreateWithPriority(&a.hi, cudaStreamNonBlocking, prio_hi));
   }
   *out = &a;
   return JMG_OK;
@@ -174,9 +174,8 @@ static int potrf_plain(int n, T* A, int lda, int nb, int* info, cudaStream_t s) 
 //  * after the block's last panel, ONE update of the whole trailing matrix with
 //    the block's operand (depth NB words per pair): the read-modify-write of the
 //    trailing matrix happens once per NB columns instead of once per panel.
-// Every update is split in two: the next panel's columns first, then the rest
-// on one SM fewer, while the next diagonal block (one CTA, bound by its serial
-// chain) is factored on a second stream on the free SM.
+// CTA 0 of every update factors the next diagonal block (bound by its serial chain)
+// behind its one tile, while the others do the rest.
 static int factor_mixed(int n, float* W, int ldw, const jmg_options& o, const Plan& p,
                         void* work, int* info_f, int* err, cudaStream_t s) {
   const int nb = o.nb, NB = p.NB;
@@ -190,40 +189,19 @@ static int factor_mixed(int n, float* W, int ldw, const jmg_options& o, const Pl
   // operand row r of the current block <-> row k0 + r of W
   auto opA = [&](size_t row, int col) { return PA + (row * p.ldp + col) * esz; };
   auto opB = [&](size_t row, int col) { return PB + (row * p.ldp + col) * esz; };
-  // the high-priority side stream and its events (made once per device)
-  DevAux* aux = nullptr;
-  JMG_TRY(dev_aux(&aux));
-  struct {
-    cudaStream_t s2;
-    cudaEvent_t panel, diag;
-  } side{aux->hi, aux->ev[0], aux->ev[1]};
-  int dev = 0, nsm = 152;
-  JMG_CUDA(cudaGetDevice(&dev));
-  JMG_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
 
   // C (rows x cols trapezoid at W[r0, r0]) -= operand rows [orow, orow + rows) x K columns
-  // [kc, kc + kext); FP8 exponents from panel kc / nb on (one chunk per panel)
-  auto update = [&](int r0, int rows, int cols, size_t orow, int kc, int kext, int ctas) -> int {
+  // [kc, kc + kext), its diagonal block at the head factored; FP8 exponents from panel
+  // kc / nb on (one chunk per panel)
+  auto update = [&](int r0, int rows, int cols, size_t orow, int kc, int kext) -> int {
     float* Cp = W + (size_t)r0 * ldw + r0;
+    const int kd = std::min(nb, rows);
     if (fp8)
       return launch_syrk_fp8(rows, cols, kext, opA(orow, kc), p.ldp,
-                             ex + (size_t)(kc / nb) * lde + orow / 128, lde, Cp, ldw, err, s, ctas);
+                             ex + (size_t)(kc / nb) * lde + orow / 128, lde, Cp, ldw, err, s, kd,
+                             r0, info_f);
     return launch_syrk_tc(rows, cols, kext, opA(orow, kc), opB(orow, kc), p.ldp, o.prec, Cp, ldw,
-                          err, s, ctas, 0, kp);
-  };
-  // the update of a trapezoid whose first nb columns hold the next diagonal
-  // block: those columns first, the block on the side stream, then the rest
-  auto update_lookahead = [&](int r0, int rows, int cols, size_t orow, int kc, int kext) -> int {
-    const int pc = std::min(nb, cols);
-    JMG_TRY(update(r0, rows, pc, orow, kc, kext, 0));
-    JMG_CUDA(cudaEventRecord(side.panel, s));
-    JMG_CUDA(cudaStreamWaitEvent(side.s2, side.panel, 0));
-    JMG_TRY(launch_potf2(W + (size_t)r0 * ldw + r0, ldw, std::min(nb, rows), r0, info_f, side.s2));
-    JMG_CUDA(cudaEventRecord(side.diag, side.s2));
-    if (cols > pc && rows > pc)
-      JMG_TRY(update(r0 + pc, rows - pc, cols - pc, orow + pc, kc, kext, nsm - 1));
-    JMG_CUDA(cudaStreamWaitEvent(s, side.diag, 0));
-    return JMG_OK;
+                          err, s, 0, kp, kd, r0, info_f);
   };
 
   JMG_TRY(launch_potf2(W, ldw, std::min(nb, n), 0, info_f, s));
@@ -247,10 +225,10 @@ static int factor_mixed(int n, float* W, int ldw, const jmg_options& o, const Pl
       const int ncb = k0 + NBk - (k + kb);  // columns of this block right of the panel
       if (ncb > 0) {
         // the block's remaining columns, with this panel's words only
-        JMG_TRY(update_lookahead(k + kb, m, ncb, orow, pp * kp, kp));
+        JMG_TRY(update(k + kb, m, ncb, orow, pp * kp, kp));
       } else {
         // the block is factored: the whole trailing matrix, with every panel of it
-        JMG_TRY(update_lookahead(k + kb, m, m, orow, 0, q * kp));
+        JMG_TRY(update(k + kb, m, m, orow, 0, q * kp));
       }
     }
   }
@@ -506,8 +484,8 @@ static int posv_mixed(int n, int nrhs, const double* A, int lda, double* B, int 
     DevAux* aux = nullptr;
     JMG_TRY(dev_aux(&aux));
     pro.s3 = aux->lo;  // the low-priority side stream and its events (made once per device)
-    pro.start = aux->ev[2];
-    pro.done = aux->ev[3];
+    pro.start = aux->ev[0];
+    pro.done = aux->ev[1];
     JMG_CUDA(cudaEventRecord(pro.start, s));  // A and the workspace are ready here
     JMG_CUDA(cudaStreamWaitEvent(pro.s3, pro.start, 0));
     if (p.split) {  // one pass for the row sums (||A||_inf) and row maxima (slice scales)
@@ -1164,7 +1142,7 @@ int jmg_dev_syrk_tc_idle_producer(int m, int ncols, int kext, const void* PA, co
   if (ncols <= 0 || ncols > m) return -2;
   if (ldc < m) return -9;
   if (!err) return -10;
-  return launch_syrk_tc(m, ncols, kext, PA, PB, ldp, prec, C, ldc, err, (cudaStream_t)stream, 0,
+  return launch_syrk_tc(m, ncols, kext, PA, PB, ldp, prec, C, ldc, err, (cudaStream_t)stream,
                         1);
 }
 

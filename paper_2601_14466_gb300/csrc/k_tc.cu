@@ -33,6 +33,7 @@
 #include <algorithm>
 
 #include "kernels.h"
+#include "potrf_diag.cuh"
 #include "tc_ptx.cuh"
 
 namespace jmg {
@@ -75,12 +76,20 @@ constexpr uint32_t PTMEM_COLS = 256;
 //         per instruction); the accumulator of tile (ti, tj) is scaled by
 //         2^-(exps[ti] + exps[tj]) in the epilogue (power-of-two tile scales).
 // Both step 32 bytes along the swizzled row per instruction.
+//
+// kb_diag > 0: CTA 0 takes tile 0 alone and then factors the diagonal block at its head
+// (kb_diag columns, koff and info as in launch_potf2) while the others do the rest: the
+// chain of panels waits for one tile and the block, with no launch and no event between
+// them.  (With the first columns' update, the block on a second stream and the rest as
+// three launches: whole solves at n = 16384 FP16x2 29.0 -> 27.7 ms, 32768 BF16 86.0 ->
+// 83.0, 65536 FP8 703 -> 701, where the block hides behind the update either way.)
 template <int KIND>
 __global__ void __launch_bounds__(PTHREADS, 1)
     k_syrk_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
               float* __restrict__ C, int ldc, int m, int ncols, int kext, int ab_fmt,
               int ntiles, int TJ, const signed char* __restrict__ exps, int lde, int cstages,
-              int* __restrict__ err, unsigned long long wait_ns, int hold_producer) {
+              int* __restrict__ err, unsigned long long wait_ns, int hold_producer, int kb_diag,
+              int koff, int* __restrict__ info) {
   extern __shared__ __align__(1024) unsigned char sm_raw[];
   unsigned char* smem =
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(sm_raw) + 1023) & ~uintptr_t(1023));
@@ -93,6 +102,9 @@ __global__ void __launch_bounds__(PTHREADS, 1)
 
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const int nk = kext / (KIND == 0 ? BK : 2 * BK);  // stage = 128 bytes of K per row
+  // this CTA's tiles: blockIdx.x, + step, ...
+  const int step = kb_diag == 0 ? (int)gridDim.x
+                                : (blockIdx.x == 0 ? ntiles : (int)gridDim.x - 1);
 
   if (threadIdx.x == 0) {
     s_fail = 0;
@@ -124,7 +136,7 @@ __global__ void __launch_bounds__(PTHREADS, 1)
     // takes its abort path
     if (lane == 0 && !hold_producer) {
       long long g = 0;
-      for (int b = blockIdx.x; b < ntiles; b += gridDim.x) {
+      for (int b = blockIdx.x; b < ntiles; b += step) {
         int ti, tj;
         trap_index(b, TJ, ti, tj);
         for (int kb = 0; kb < nk; ++kb, ++g) {
@@ -154,7 +166,7 @@ __global__ void __launch_bounds__(PTHREADS, 1)
       const int nch = nk / cstages;
       long long g = 0, ci = 0;
       bool ok = true;
-      for (int b = blockIdx.x; b < ntiles && ok; b += gridDim.x) {
+      for (int b = blockIdx.x; b < ntiles && ok; b += step) {
         for (int c = 0; c < nch && ok; ++c, ++ci) {
           const int a = (int)(ci & 1);
           if (ci >= 2 && !mbar_wait(&acc_empty[a], (uint32_t)((ci / 2) - 1) & 1, wait_ns)) {
@@ -215,10 +227,10 @@ __global__ void __launch_bounds__(PTHREADS, 1)
     const int nch = nk / cstages;
     long long ci = 0;
     bool ok = true;
-    for (int b = blockIdx.x; b < ntiles && ok; b += gridDim.x) {
+    for (int b = blockIdx.x; b < ntiles && ok; b += step) {
       int ti, tj;
       trap_index(b, TJ, ti, tj);
-      prefetch_c(b + gridDim.x);
+      prefetch_c(b + step);
       float acc[2][32];
 #pragma unroll
       for (int h = 0; h < 2; ++h)
@@ -288,6 +300,11 @@ __global__ void __launch_bounds__(PTHREADS, 1)
   tc_fence_before();
   __syncthreads();
   if (warp == 1) tmem_dealloc(tmem, PTMEM_COLS);
+  if (kb_diag > 0 && blockIdx.x == 0 && !ld_shared_volatile(&s_fail)) {
+    __syncthreads();  // tile 0 is in global memory, the stages are idle
+    if (threadIdx.x >= pdiag::TH) return;
+    potrf_diag_body<float>(C, ldc, kb_diag, koff, info);
+  }
 }
 
 }  // namespace tc
@@ -346,8 +363,8 @@ static int make_map(CUtensorMap* map, const void* base, int rows, int cols, int 
 template <int KIND>
 static int syrk_persistent(int m, int ncols, int kext, int kchunk, const CUtensorMap& ma,
                            const CUtensorMap& mb, int ab_fmt, const signed char* exps, int lde,
-                           float* C, int ldc, int* err, cudaStream_t s, int max_ctas,
-                           int hold = 0) {
+                           float* C, int ldc, int* err, cudaStream_t s, int hold, int kb_diag,
+                           int koff, int* info) {
   const int stage_k = KIND == 0 ? tc::BK : 2 * tc::BK;  // K elements per stage
   if (kchunk <= 0 || kchunk > kext) kchunk = kext;
   if (kchunk % stage_k || kext % kchunk) return JMG_ERR_ALIGN;
@@ -358,16 +375,16 @@ static int syrk_persistent(int m, int ncols, int kext, int kchunk, const CUtenso
   JMG_TRY(ensure_smem(tc::k_syrk_tc<KIND>, tc::PSMEM_BYTES));
   const int TI = cdiv(m, tc::BM), TJ = cdiv(ncols, tc::BN);
   const long long ntiles = (long long)TJ * (TJ + 1) / 2 + (long long)(TI - TJ) * TJ;
-  const int grid = (int)std::min<long long>(ntiles, max_ctas > 0 ? std::min(max_ctas, nsm) : nsm);
+  const int grid = (int)std::min<long long>(ntiles, nsm);
   tc::k_syrk_tc<KIND><<<grid, tc::PTHREADS, tc::PSMEM_BYTES, s>>>(
       ma, mb, C, ldc, m, ncols, kext, ab_fmt, (int)ntiles, TJ, exps, lde, cstages, err, g_wait_ns,
-      hold);
+      hold, kb_diag, koff, info);
   return launched();
 }
 
 int launch_syrk_tc(int m, int ncols, int kext, const void* PA, const void* PB, int ldp, int prec,
-                   float* C, int ldc, int* err, cudaStream_t s, int max_ctas, int hold,
-                   int kchunk) {
+                   float* C, int ldc, int* err, cudaStream_t s, int hold, int kchunk, int kb_diag,
+                   int koff, int* info) {
   if (m <= 0 || ncols <= 0 || kext <= 0) return JMG_OK;
   if (ncols > m) return JMG_ERR_UNSUPPORTED;
   if (kext % tc::BK || ldp % 64 || ldp < kext) return JMG_ERR_ALIGN;
@@ -379,11 +396,12 @@ int launch_syrk_tc(int m, int ncols, int kext, const void* PA, const void* PB, i
   JMG_TRY(make_map(&ma, PA, m, kext, ldp, 2, dt));
   JMG_TRY(make_map(&mb, PB, m, kext, ldp, 2, dt));
   return syrk_persistent<0>(m, ncols, kext, kchunk, ma, mb, prec == JMG_PREC_BF16 ? 1 : 0, nullptr,
-                            0, C, ldc, err, s, max_ctas, hold);
+                            0, C, ldc, err, s, hold, kb_diag, koff, info);
 }
 
 int launch_syrk_fp8(int m, int ncols, int kext, const void* Q, int ldq, const signed char* e,
-                    int lde, float* C, int ldc, int* err, cudaStream_t s, int max_ctas) {
+                    int lde, float* C, int ldc, int* err, cudaStream_t s, int kb_diag, int koff,
+                    int* info) {
   if (m <= 0 || ncols <= 0 || kext <= 0) return JMG_OK;
   if (ncols > m) return JMG_ERR_UNSUPPORTED;
   if (kext % 128 || ldq % 128 || ldq < kext) return JMG_ERR_ALIGN;
@@ -391,7 +409,8 @@ int launch_syrk_fp8(int m, int ncols, int kext, const void* Q, int ldq, const si
   if (!e) return JMG_ERR_UNSUPPORTED;
   CUtensorMap mq;
   JMG_TRY(make_map(&mq, Q, m, kext, ldq, 1, CU_TENSOR_MAP_DATA_TYPE_UINT8));
-  return syrk_persistent<1>(m, ncols, kext, 128, mq, mq, 0, e, lde, C, ldc, err, s, max_ctas);
+  return syrk_persistent<1>(m, ncols, kext, 128, mq, mq, 0, e, lde, C, ldc, err, s, 0, kb_diag,
+                            koff, info);
 }
 
 }  // namespace jmg
