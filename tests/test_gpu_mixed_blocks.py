@@ -22,7 +22,7 @@ def test_diagonal_blocks_edges(n, prec, nb):
     u, b = rng.uniform(-1, 1, n), rng.standard_normal(n)
     A = np.eye(n) + np.outer(u, u) / n
     x = b - u * ((u @ b) / n) / (1 + (u @ u) / n)
-    Ad = torch.from_numpy(A).cuda()
+    Ad = torch.from_numpy(A).cuda().mT  # (symmetric)
     X, si = jmg.posv(Ad, torch.from_numpy(b[:, None]).cuda(), prec=prec, nb=nb)
     assert np.abs(X.cpu().numpy()[:, 0] - x).max() <= 1e-12 * np.abs(x).max()
 
@@ -32,6 +32,6 @@ def test_failing_pivot_position(k):
     n = 1152
     A = torch.eye(n, dtype=torch.float64, device="cuda")
     A[k, k] = -1.0
-    _, si = jmg.posv(A, torch.ones(n, 1, dtype=torch.float64, device="cuda"), prec="bf16",
+    _, si = jmg.posv(A.mT, torch.ones(n, 1, dtype=torch.float64, device="cuda"), prec="bf16",
                      shift_retry=False, check=False)
     assert si.info == k + 1
