@@ -222,6 +222,10 @@ __global__ void __launch_bounds__(PTHREADS, 1)
       }
     };
     prefetch_c(blockIdx.x);
+    // 16-bit words: CTA 0's diagonal block goes to its factorisation through shared
+    // memory, where the stages are idle by the epilogue of its only tile (n = 16384 27.7
+    // -> 27.4 ms, 8192 gradient 13.1 -> 12.9; with FP8 the block hides behind the rest)
+    const int keep = blockIdx.x == 0 ? kb_diag : 0;
     // the chunks of a tile add up in registers (this warp's 32 rows x 64
     // columns), then one read-modify-write of C per tile
     const int nch = nk / cstages;
@@ -279,8 +283,17 @@ __global__ void __launch_bounds__(PTHREADS, 1)
 #pragma unroll
           for (int j = 0; j < 32; ++j) old[j] = j < jn ? cp[j * ldc] : 0.0f;
 #pragma unroll
-          for (int j = 0; j < 32; ++j)
-            if (j < jn) cp[j * ldc] = old[j] - acc[h][j];
+          for (int j = 0; j < 32; ++j) acc[h][j] = old[j] - acc[h][j];
+          if (KIND == 0 && r < keep && cb < keep) {  // (64 columns of the tile at a time: all or none)
+            float* sa = reinterpret_cast<float*>(sm_raw) + cb * pdiag::LD + r;
+#pragma unroll
+            for (int j = 0; j < 32; ++j)
+              if (j < jn) sa[j * pdiag::LD] = acc[h][j];
+          } else {
+#pragma unroll
+            for (int j = 0; j < 32; ++j)
+              if (j < jn) cp[j * ldc] = acc[h][j];
+          }
         }
       }
     }
@@ -301,9 +314,9 @@ __global__ void __launch_bounds__(PTHREADS, 1)
   __syncthreads();
   if (warp == 1) tmem_dealloc(tmem, PTMEM_COLS);
   if (kb_diag > 0 && blockIdx.x == 0 && !ld_shared_volatile(&s_fail)) {
-    __syncthreads();  // tile 0 is in global memory, the stages are idle
+    __syncthreads();  // the block is in place, the stages are idle
     if (threadIdx.x >= pdiag::TH) return;
-    potrf_diag_body<float>(C, ldc, kb_diag, koff, info);
+    potrf_diag_body<float, KIND == 0>(C, ldc, kb_diag, koff, info);
   }
 }
 

@@ -84,7 +84,9 @@ JMG_DEV void load4<double>(const double* p, double (&v)[4]) {
 }
 }  // namespace pdiag
 
-template <typename T>
+// LOADED: the block's lower part is in shared memory already (in the layout below; the
+// caller's barrier lies between), A is only written.
+template <typename T, bool LOADED = false>
 JMG_DEV void potrf_diag_body(T* __restrict__ A, int lda, int kb, int koff,
                              int* __restrict__ info) {
   using namespace pdiag;
@@ -98,7 +100,7 @@ JMG_DEV void potrf_diag_body(T* __restrict__ A, int lda, int kb, int koff,
   if (t == 0) fail = *(volatile int*)info;  // one read, so every thread takes the same exit
   __syncthreads();
   if (fail != 0) return;  // an earlier block already failed
-  for (int base = 0; base < kb * kb; base += TH * 16) {  // 16 independent loads per thread
+  for (int base = 0; !LOADED && base < kb * kb; base += TH * 16) {  // 16 independent loads per thread
     T v[16];
 #pragma unroll
     for (int q = 0; q < 16; ++q) {
