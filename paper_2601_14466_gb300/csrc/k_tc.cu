@@ -282,17 +282,15 @@ __global__ void __launch_bounds__(PTHREADS, 1)
           float old[32];
 #pragma unroll
           for (int j = 0; j < 32; ++j) old[j] = j < jn ? cp[j * ldc] : 0.0f;
-#pragma unroll
-          for (int j = 0; j < 32; ++j) acc[h][j] = old[j] - acc[h][j];
-          if (KIND == 0 && r < keep && cb < keep) {  // (64 columns of the tile at a time: all or none)
+          if (KIND == 0 && r < keep && cb < keep) {  // (columns past keep lie above the diagonal)
             float* sa = reinterpret_cast<float*>(sm_raw) + cb * pdiag::LD + r;
 #pragma unroll
             for (int j = 0; j < 32; ++j)
-              if (j < jn) sa[j * pdiag::LD] = acc[h][j];
+              if (j < jn) sa[j * pdiag::LD] = old[j] - acc[h][j];
           } else {
 #pragma unroll
             for (int j = 0; j < 32; ++j)
-              if (j < jn) cp[j * ldc] = acc[h][j];
+              if (j < jn) cp[j * ldc] = old[j] - acc[h][j];
           }
         }
       }
