@@ -310,7 +310,10 @@ JMG_DEV bool wait_ge(const int* p, int G, int v, Ctl& C, int* err, int* info, ui
 }
 
 // The same for all G <= 32 counters by a whole warp, one lane each: a counter costs an
-// L2 round trip, which one lane reading them in turn would pay G times.
+// L2 round trip, which one lane reading them in turn would pay G times.  The vote says
+// that every lane has acquired its counter but orders no memory between the lanes: the
+// __syncwarp does, so that what follows on lane 0 (proxy fence, copy of every leader's
+// columns) comes after all of the acquires.
 JMG_DEV bool wait_ge_warp(const int* p, int G, int v, Ctl& C, int* err, int* info,
                           uint64_t limit, int lane) {
   uint64_t t0 = 0;
@@ -323,6 +326,7 @@ JMG_DEV bool wait_ge_warp(const int* p, int G, int v, Ctl& C, int* err, int* inf
     }
     __nanosleep(32);
   }
+  __syncwarp();
   return true;
 }
 
