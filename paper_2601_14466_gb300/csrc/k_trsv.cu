@@ -154,15 +154,23 @@ JMG_DEV int wait_gt(const int* p, int d, int* err, int* info, SM& S, uint64_t li
 }
 
 // Bounded spin of a warp on a counter in shared memory (each lane its own p, or all
-// the same) until every one is >= want; false, on every lane, on abort or expiry.
+// the same) until every one is >= want; false, on every lane, on abort or expiry.  The
+// vote orders no memory between the lanes; the __syncwarp puts what any lane reads next
+// after the acquires of all of them.
 template <typename SM>
 JMG_DEV bool wait_sm(const int* p, int want, int* err, int* info, SM& S, uint64_t limit_ns) {
-  if (__all_sync(0xffffffffu, ld_acquire_sm(p) >= want)) return true;
+  if (__all_sync(0xffffffffu, ld_acquire_sm(p) >= want)) {
+    __syncwarp();
+    return true;
+  }
   const uint64_t t0 = globaltimer_ns();
   while (true) {
 #pragma unroll 1
     for (int i = 0; i < 64; ++i)
-      if (__all_sync(0xffffffffu, ld_acquire_sm(p) >= want)) return true;
+      if (__all_sync(0xffffffffu, ld_acquire_sm(p) >= want)) {
+        __syncwarp();
+        return true;
+      }
     if (__any_sync(0xffffffffu, ld_shared_volatile(&S.abort))) return false;
     if (__any_sync(0xffffffffu, globaltimer_ns() - t0 > limit_ns)) {
       give_up(err, info, S);

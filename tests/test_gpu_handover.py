@@ -33,3 +33,9 @@ def _repeat(solve, n, nrhs, dtype, tol):
 def test_block_inverse_solves_repeat(n, nrhs):
     # 5, 8 and 16 leaders; the bound of the other tests of these solves
     _repeat(jmg.sv_potrs_, n, nrhs, torch.float32, 2048 * 2.0 ** -24)
+
+
+@pytest.mark.parametrize("n,nrhs", [(1500, 3), (3000, 16), (1000, 40)])
+def test_fp64_solves_repeat(n, nrhs):
+    # 3 and 16 leaders of one right-hand side, groups of 4 leaders of four
+    _repeat(jmg.potrs_, n, nrhs, torch.float64, 64 * n * U64)
