@@ -118,11 +118,22 @@ unsigned long long jmg_dev_set_wait_limit_ns(unsigned long long ns);
  * syrk_tc_idle_producer: the tensor-core trailing update (arguments as
  *   jmg_dev_syrk_tc) with its copy producer idle: the MMA issuer's wait for the
  *   first stage runs out; afterwards *err != 0 and C is untouched.
+ *
+ * oz_factor_idle_producer, oz_solve_idle_producer: the FP64 factorisation and the
+ *   blocked FP64 solve with their products in slices (arguments as jmg_potrf and
+ *   jmg_potrs; work: jmg_workspace_fast bytes of that call; n > 64, and a shape that
+ *   the blocked solve takes) with the updates' copy producers idle.  Afterwards
+ *   *info == -1 and the columns right of the first panel are untouched; the first int
+ *   of work == JMG_ERR_TIMEOUT and the rows of B below the first 512 are untouched.
  */
 int jmg_dev_trsv_leaderless(int n, int nrhs, const void* L, int lda, void* B, int ldb, int dtype,
                             int* sync, int* info, void* stream);
 int jmg_dev_syrk_tc_idle_producer(int m, int ncols, int kext, const void* PA, const void* PB,
                                   int ldp, int prec, float* C, int ldc, int* err, void* stream);
+int jmg_dev_oz_factor_idle_producer(int n, double* A, int lda, int* info, void* work, size_t lwork,
+                                    void* stream);
+int jmg_dev_oz_solve_idle_producer(int n, int nrhs, const double* L, int lda, double* B, int ldb,
+                                   void* work, size_t lwork, void* stream);
 
 /*
  * The block-inverse triangular solves of the mixed path on a caller's FP32

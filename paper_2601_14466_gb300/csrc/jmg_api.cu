@@ -1146,6 +1146,35 @@ int jmg_dev_syrk_tc_idle_producer(int m, int ncols, int kext, const void* PA, co
                         1);
 }
 
+int jmg_dev_oz_factor_idle_producer(int n, double* A, int lda, int* info, void* work, size_t lwork,
+                                    void* stream) {
+  if (n <= 64) return -1;
+  if (!A) return -2;
+  if (lda < n) return -3;
+  if (!info) return -4;
+  if (!work || lwork < ozf_workspace(n)) return JMG_ERR_WORKSPACE;
+  if (reinterpret_cast<uintptr_t>(work) & 255) return JMG_ERR_ALIGN;
+  cudaStream_t s = (cudaStream_t)stream;
+  JMG_CUDA(cudaMemsetAsync(info, 0, sizeof(int), s));
+  return potrf_split(n, A, lda, info, work, s, 1);
+}
+
+int jmg_dev_oz_solve_idle_producer(int n, int nrhs, const double* L, int lda, double* B, int ldb,
+                                   void* work, size_t lwork, void* stream) {
+  if (n <= 0) return -1;
+  if (nrhs <= 0) return -2;
+  if (!L) return -3;
+  if (lda < n) return -4;
+  if (!B) return -5;
+  if (ldb < n) return -6;
+  const size_t sb = plain_solve_bytes(n, nrhs), fast = ozs_workspace(n, nrhs);
+  if (!fast) return JMG_ERR_UNSUPPORTED;
+  if (!work || lwork < sb + fast) return JMG_ERR_WORKSPACE;
+  if (reinterpret_cast<uintptr_t>(work) & 255) return JMG_ERR_ALIGN;
+  return solve_split(n, nrhs, L, lda, B, ldb, (int*)work, nullptr, static_cast<char*>(work) + sb,
+                     (cudaStream_t)stream, 1);
+}
+
 int jmg_dev_quant_fp8(int m, int kb, const float* L21, int ldw, void* Q, int ldq, signed char* e,
                       void* stream) {
   if (m < 0) return -1;

@@ -252,7 +252,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                 double* __restrict__ C, int ldc, int nA, int rA, int nB, int rB, int m, int ncols,
                 int nkb, const int* __restrict__ exA, const int* __restrict__ exB, int TI, int TJ,
                 int ntiles, int kb_diag, int koff, int* __restrict__ info, int* __restrict__ err,
-                unsigned long long wait_ns) {
+                unsigned long long wait_ns, int hold) {
   using namespace tc;
   extern __shared__ __align__(1024) unsigned char sm_raw_ozf[];
   unsigned char* smem = reinterpret_cast<unsigned char*>(
@@ -266,7 +266,8 @@ __global__ void __launch_bounds__(THREADS, 1)
   uint64_t* aempty = afull + ASTAGES;
   uint64_t* accf = aempty + ASTAGES;
   uint64_t* acce = accf + 1;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acce + 1);
+  uint64_t* drain = acce + 1;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
   __shared__ int s_fail, s_info;
 
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
@@ -292,6 +293,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     }
     mbar_init(accf, 1);
     mbar_init(acce, 16);
+    mbar_init(drain, 1);
     fence_mbar_init();
     prefetch_tmap(&tmA);
     prefetch_tmap(&tmB);
@@ -309,7 +311,8 @@ __global__ void __launch_bounds__(THREADS, 1)
 
   long long b_issued = 0, a_issued = 0;
   if (warp == 0) {
-    if (lane == 0) {
+    // hold (a test hook) keeps the producer idle: the MMA warp's first wait runs out
+    if (lane == 0 && !hold) {
       bool ok = true;
       for (int b = first; b < ntiles && ok; b += step) {
         int ti, tj;
@@ -485,7 +488,9 @@ __global__ void __launch_bounds__(THREADS, 1)
       if (info) atomicCAS(info, 0, -1);
       if (RECT) atomicExch(err, JMG_ERR_TIMEOUT);
     }
+    if (warp == 1 && lane == 0) mma_drain(drain, wait_ns);
   }
+  __syncwarp();
   tc_fence_before();
   __syncthreads();
   if (warp == 1) tmem_dealloc(tmem, TCOLS);
@@ -764,7 +769,7 @@ OzfPlan ozf_plan(int n) {
 
 size_t ozf_workspace(int n) { return n > ozf::PW ? ozf_plan(n).total : 0; }
 
-int potrf_split(int n, double* A, int lda, int* info, void* work, cudaStream_t s) {
+int potrf_split(int n, double* A, int lda, int* info, void* work, cudaStream_t s, int hold) {
   using namespace ozf;
   const OzfPlan p = ozf_plan(n);
   char* w = static_cast<char*>(work);
@@ -791,7 +796,7 @@ int potrf_split(int n, double* A, int lda, int* info, void* work, cudaStream_t s
     const long long nt = tile_count(TI, TJ);
     k_oz_update<false><<<(int)std::min<long long>(nt, nsm), THREADS, SMEM, s>>>(
         ma, mb, A + (size_t)r0 * lda + r0, lda, n, r0, n, r0, n - r0, ncols, nkb, ex + r0, ex + r0, TI,
-        TJ, (int)nt, std::min(PW, n - r0), r0, info, nullptr, g_wait_ns);
+        TJ, (int)nt, std::min(PW, n - r0), r0, info, nullptr, g_wait_ns, hold);
     return launched();
   };
   // the first diagonal block; every update leaves the next one factored
@@ -869,7 +874,7 @@ size_t ozs_workspace(int n, int nrhs) {
 }
 
 int solve_split(int n, int nrhs, const double* L, int lda, double* B, int ldb, int* sync,
-                int* info, void* work, cudaStream_t s) {
+                int* info, void* work, cudaStream_t s, int hold) {
   using namespace ozf;
   const SolvePlan p = solve_plan(n, nrhs);
   char* w = static_cast<char*>(work);
@@ -894,7 +899,7 @@ int solve_split(int n, int nrhs, const double* L, int lda, double* B, int ldb, i
     const int TI = cdiv(m, BM), TJ = cdiv(nrhs, BN), nt = TI * TJ;
     k_oz_update<true><<<std::min(nt, nsm), THREADS, SMEM, s>>>(
         mp, mq, B + row0, ldb, nA, rA, nrhs, 0, m, nrhs, SK / BK, exr + rA, exc, TI, TJ, nt, 0, 0,
-        info, sync, g_wait_ns);
+        info, sync, g_wait_ns, hold);
     return launched();
   };
   CUtensorMap mp;

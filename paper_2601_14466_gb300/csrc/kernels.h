@@ -93,7 +93,9 @@ int solve_llt(int n, int nrhs, const T* L, int lda, T* B, int ldb, int* sync, in
 // Scratch of potrf_split for order n; 0 when that route does not take n.
 size_t ozf_workspace(int n);
 // Cholesky factorisation in place; work: ozf_workspace(n) bytes, 256-byte aligned.
-int potrf_split(int n, double* A, int lda, int* info, void* work, cudaStream_t s);
+// hold != 0 (here and below) is a test hook: the updates' TMA producers stay idle, so
+// their first bounded wait runs out (g_wait_ns) and they leave through their abort path.
+int potrf_split(int n, double* A, int lda, int* info, void* work, cudaStream_t s, int hold = 0);
 
 // Scratch of solve_split for this shape; 0 where the one-launch solves are the better
 // ones.
@@ -101,7 +103,7 @@ size_t ozs_workspace(int n, int nrhs);
 // (L L^T) X = B on FP64 data, blocked, with split updates; sync and info as solve_llt,
 // work: ozs_workspace bytes, 256-byte aligned.
 int solve_split(int n, int nrhs, const double* L, int lda, double* B, int ldb, int* sync,
-                int* info, void* work, cudaStream_t s);
+                int* info, void* work, cudaStream_t s, int hold = 0);
 
 // ---- mixed-precision helpers
 // W (FP32, ldw) <- lower(A) (FP64), lower triangle only; plus shift on the diagonal.

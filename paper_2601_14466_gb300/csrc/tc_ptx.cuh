@@ -97,6 +97,13 @@ JMG_DEV void tc_commit(uint64_t* bar) {
           smem_u32(bar))
       : "memory");
 }
+// Abort path, on the thread that issued this CTA's MMAs: wait (bounded) until every one of
+// them has ended, so that none writes TMEM or reads shared memory given back by then.
+// `bar`: one arrival, not used for anything else.
+JMG_DEV void mma_drain(uint64_t* bar, uint64_t limit_ns) {
+  tc_commit(bar);
+  (void)mbar_wait(bar, 0, limit_ns);
+}
 JMG_DEV void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
