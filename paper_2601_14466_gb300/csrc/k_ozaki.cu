@@ -247,7 +247,8 @@ __global__ void __launch_bounds__(oz::THREADS, 1)
   uint64_t* aempty = afull + ASTAGES;
   uint64_t* accf = aempty + ASTAGES;  // NBUF
   uint64_t* acce = accf + NBUF;       // NBUF
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acce + NBUF);
+  uint64_t* drain = acce + NBUF;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
   __shared__ int s_fail;
 
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
@@ -272,6 +273,7 @@ __global__ void __launch_bounds__(oz::THREADS, 1)
       mbar_init(&accf[i], 1);
       mbar_init(&acce[i], N * 4 / 16);
     }
+    mbar_init(drain, 1);
     fence_mbar_init();
     prefetch_tmap(&tmA);
     prefetch_tmap(&tmX);
@@ -450,7 +452,9 @@ __global__ void __launch_bounds__(oz::THREADS, 1)
         (void)mbar_wait(&afull[g % ASTAGES], (uint32_t)(g / ASTAGES) & 1, wait_ns);
       atomicExch(err, 1);
     }
+    if (warp == 1 && lane == 0) mma_drain(drain, wait_ns);
   }
+  __syncwarp();
   tc_fence_before();
   __syncthreads();
   if (warp == 1) tmem_dealloc(tmem, TCOLS);

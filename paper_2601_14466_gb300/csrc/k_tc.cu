@@ -97,7 +97,8 @@ __global__ void __launch_bounds__(PTHREADS, 1)
   uint64_t* empty = full + PSTAGES;
   uint64_t* acc_full = empty + PSTAGES;
   uint64_t* acc_empty = acc_full + 2;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
+  uint64_t* drain = acc_empty + 2;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
   __shared__ int s_fail;
 
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
@@ -116,6 +117,7 @@ __global__ void __launch_bounds__(PTHREADS, 1)
       mbar_init(&acc_full[a], 1);
       mbar_init(&acc_empty[a], EPI_WARPS);
     }
+    mbar_init(drain, 1);
     fence_mbar_init();
     prefetch_tmap(&tmA);
     prefetch_tmap(&tmB);
@@ -307,7 +309,9 @@ __global__ void __launch_bounds__(PTHREADS, 1)
         (void)mbar_wait(&full[g % PSTAGES], (uint32_t)(g / PSTAGES) & 1, wait_ns);
       atomicExch(err, 1);
     }
+    if (warp == 1 && lane == 0) mma_drain(drain, wait_ns);
   }
+  __syncwarp();
   tc_fence_before();
   __syncthreads();
   if (warp == 1) tmem_dealloc(tmem, PTMEM_COLS);
