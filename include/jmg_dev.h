@@ -125,6 +125,10 @@ unsigned long long jmg_dev_set_wait_limit_ns(unsigned long long ns);
  *   the blocked solve takes) with the updates' copy producers idle.  Afterwards
  *   *info == -1 and the columns right of the first panel are untouched; the first int
  *   of work == JMG_ERR_TIMEOUT and the rows of B below the first 512 are untouched.
+ *
+ * sym_grad_no_products: jmg_sym_grad (nrhs >= 12, so that it takes the tensor-core
+ *   kernel) with no product issued: the wait for the first one runs out and the FP64
+ *   units do all of them; the result is jmg_sym_grad's.
  */
 int jmg_dev_trsv_leaderless(int n, int nrhs, const void* L, int lda, void* B, int ldb, int dtype,
                             int* sync, int* info, void* stream);
@@ -134,6 +138,8 @@ int jmg_dev_oz_factor_idle_producer(int n, double* A, int lda, int* info, void* 
                                     void* stream);
 int jmg_dev_oz_solve_idle_producer(int n, int nrhs, const double* L, int lda, double* B, int ldb,
                                    void* work, size_t lwork, void* stream);
+int jmg_dev_sym_grad_no_products(int n, int nrhs, const double* Bbar, int ldb, const double* X,
+                                 int ldx, double* Abar, int ldab, void* stream);
 
 /*
  * The block-inverse triangular solves of the mixed path on a caller's FP32

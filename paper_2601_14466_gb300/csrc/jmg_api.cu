@@ -1175,6 +1175,19 @@ int jmg_dev_oz_solve_idle_producer(int n, int nrhs, const double* L, int lda, do
                      (cudaStream_t)stream, 1);
 }
 
+int jmg_dev_sym_grad_no_products(int n, int nrhs, const double* Bbar, int ldb, const double* X,
+                                 int ldx, double* Abar, int ldab, void* stream) {
+  if (n <= 0) return -1;
+  if (nrhs <= 0) return -2;
+  if (!Bbar) return -3;
+  if (ldb < n) return -4;
+  if (!X) return -5;
+  if (ldx < n) return -6;
+  if (!Abar) return -7;
+  if (ldab < n) return -8;
+  return launch_sym_grad(n, nrhs, Bbar, ldb, X, ldx, Abar, ldab, (cudaStream_t)stream, 1);
+}
+
 int jmg_dev_quant_fp8(int m, int kb, const float* L21, int ldw, void* Q, int ldq, signed char* e,
                       void* stream) {
   if (m < 0) return -1;

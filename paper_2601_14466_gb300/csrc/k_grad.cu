@@ -124,7 +124,7 @@ static_assert(BN * LDT * 8 <= ozf::S * A_TILE, "the output tile lies over the op
 __global__ void __launch_bounds__(grad::TH, 1)
     k_sym_grad_tc(int n, int nrhs, const double* __restrict__ Bb, int ldb,
                   const double* __restrict__ X, int ldx, double* __restrict__ G, int ldg,
-                  unsigned long long wait_ns) {
+                  unsigned long long wait_ns, int hold) {
   using namespace grad;
   using namespace tc;
   using ozf::S;
@@ -134,7 +134,7 @@ __global__ void __launch_bounds__(grad::TH, 1)
   unsigned char* bbuf = abuf + S * A_TILE;
   double* sP = reinterpret_cast<double*>(bbuf + S * B_TILE);  // [KC][BM]
   double* sQ = sP + KC * BM;                                  // [KC][BN]
-  __shared__ uint64_t bar;
+  __shared__ uint64_t bar, drain;
   __shared__ uint32_t tmem_slot;
   __shared__ int s_ep[BM], s_eq[BN], s_k[KC];  // row exponents, column shifts
   const int t = threadIdx.x, warp = t / 32, lane = t % 32;
@@ -147,6 +147,7 @@ __global__ void __launch_bounds__(grad::TH, 1)
   if (j0 >= n) return;
   if (t == 0) {
     mbar_init(&bar, 1);
+    mbar_init(&drain, 1);
     fence_mbar_init();
   }
   if (warp == 0) {
@@ -247,7 +248,7 @@ __global__ void __launch_bounds__(grad::TH, 1)
         }
         tc_fence_before();
         __syncthreads();
-        if (t == 0) {
+        if (t == 0 && !hold) {  // (hold, a test hook: no products, the wait below runs out)
           tc_fence_after();
           constexpr int GMAX = 256 / BN;
           for (int a = 0; a < S; ++a)
@@ -293,7 +294,8 @@ __global__ void __launch_bounds__(grad::TH, 1)
       __syncthreads();  // accumulators and staged columns are free
     }
   }
-  if (!ok) (void)mbar_wait(&bar, phase ^ 1, 1000000000ull);  // the products still under way
+  if (!ok && t == 0) mma_drain(&drain, wait_ns);  // the products still under way
+  __syncwarp();
   tc_fence_before();
   __syncthreads();
   if (warp == 0) tmem_dealloc(tmem, 512);
@@ -316,7 +318,7 @@ __global__ void __launch_bounds__(grad::TH, 1)
 }
 
 int launch_sym_grad(int n, int nrhs, const double* Bb, int ldb, const double* X, int ldx, double* G,
-                    int ldg, cudaStream_t s) {
+                    int ldg, cudaStream_t s, int hold) {
   if (n <= 0) return JMG_OK;
   if (nrhs <= 0) {
     JMG_CUDA(cudaMemset2DAsync(G, sizeof(double) * ldg, 0, sizeof(double) * n, n, s));
@@ -330,7 +332,7 @@ int launch_sym_grad(int n, int nrhs, const double* Bb, int ldb, const double* X,
     JMG_TRY(ensure_smem(k_sym_grad_tc, SMEM));
     const long long TI = cdiv(n, BM);
     k_sym_grad_tc<<<(unsigned)(TI * (TI + 1)), TH, SMEM, s>>>(n, nrhs, Bb, ldb, X, ldx, G, ldg,
-                                                             g_wait_ns);
+                                                             g_wait_ns, hold);
     return launched();
   }
   k_sym_grad<<<(unsigned)tri_tiles(cdiv(n, grad::TB)), 256, 0, s>>>(n, nrhs, Bb, ldb, X, ldx, G,

@@ -179,8 +179,9 @@ int launch_scale_from_f32(int n, int nrhs, const float* D, int ldd, const double
 int launch_diag_max(int n, const double* A, int lda, double* out, cudaStream_t s);
 
 // ---- adjoint (k_grad.cu): G = -(Bb X^T + X Bb^T)/2, full symmetric n x n
+// hold != 0 is a test hook: the tensor-core kernel issues no products, so its waits run out.
 int launch_sym_grad(int n, int nrhs, const double* Bb, int ldb, const double* X, int ldx, double* G,
-                    int ldg, cudaStream_t s);
+                    int ldg, cudaStream_t s, int hold = 0);
 
 // ---- block-inverse solves with the FP32 factor of the mixed path (k_solve.cu)
 // Bytes of the per-factorisation images (inverses of the diagonal blocks and the

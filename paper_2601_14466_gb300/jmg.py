@@ -99,6 +99,7 @@ _SIGS = {
     "jmg_dev_syrk_tc_idle_producer": (_I, [_I, _I, _I, _P, _P, _I, _I, _P, _I, _P, _P]),
     "jmg_dev_oz_factor_idle_producer": (_I, [_I, _P, _I, _P, _P, _SZ, _P]),
     "jmg_dev_oz_solve_idle_producer": (_I, [_I, _I, _P, _I, _P, _I, _P, _SZ, _P]),
+    "jmg_dev_sym_grad_no_products": (_I, [_I, _I, _P, _I, _P, _I, _P, _I, _P]),
     "jmg_dev_quant_fp8": (_I, [_I, _I, _P, _I, _P, _I, _P, _P]),
     "jmg_dev_sv_workspace": (_SZ, [_I, _I]),
     "jmg_dev_sv_potrs": (_I, [_I, _I, _P, _I, _P, _I, _P, _SZ, _P]),

@@ -75,3 +75,19 @@ def test_solve_update_wait_runs_out(short_waits):
     X = torch.linalg.solve_triangular(Ld.mT, Y, upper=True)
     assert int(work[:4].view(torch.int32).item()) == 0
     assert float((Bd - X).abs().max()) <= 64 * n * U64 * max(1.0, float(X.abs().max()))
+
+
+@pytest.mark.parametrize("n,nrhs", [(65, 12), (300, 35)])
+def test_adjoint_wait_runs_out(short_waits, n, nrhs):
+    Y, X = inputs.uniform(n, nrhs, seed=5).to(DEV), inputs.uniform(n, nrhs, seed=6).to(DEV)
+    Yc, Xc = jmg.colmajor_copy(Y), jmg.colmajor_copy(X)
+    G = torch.full((n, n), float("nan"), dtype=torch.float64, device=DEV)
+    st = jmg.load().jmg_dev_sym_grad_no_products(n, nrhs, Yc.data_ptr(), n, Xc.data_ptr(), n,
+                                                 G.data_ptr(), n, _stream())
+    assert st == 0
+    torch.cuda.synchronize()
+    jmg.set_wait_limit_ns(2_000_000_000)
+    want = -0.5 * (Y @ X.t() + X @ Y.t())
+    tol = (2 * nrhs + 2) * U64 * (Y.abs() @ X.abs().t() + X.abs() @ Y.abs().t())
+    assert bool(((G - want).abs() <= tol).all())
+    assert bool(((jmg.sym_grad(Yc, Xc) - want).abs() <= tol).all())
