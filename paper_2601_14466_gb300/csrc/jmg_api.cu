@@ -106,11 +106,23 @@ static size_t plain_solve_bytes(int n, int nrhs) {
 }
 
 // Side stream and events of the mixed path, created once per device on first
-// use and kept for the life of the process (a call made on another thread
-// shares them: events are re-recorded, which can only add dependencies).
+// use and kept for the life of the process.  Calls on several threads share them.
+// `start` carries a dependency from a caller's stream to the side stream, so another
+// thread's record between its record and its wait would replace the caller's stream by
+// that thread's: both happen under `mu`.  `done` is recorded on the side stream, in
+// order: a later record can only add work to what a caller waits for.
 struct DevAux {
+  std::mutex mu;
   cudaStream_t lo = nullptr;  // low priority, non-blocking
-  cudaEvent_t ev[2] = {nullptr, nullptr};
+  cudaEvent_t start = nullptr, done = nullptr;
+
+  // the side stream waits for what is queued on s
+  int follow(cudaStream_t s) {
+    std::lock_guard<std::mutex> lock(mu);
+    JMG_CUDA(cudaEventRecord(start, s));
+    JMG_CUDA(cudaStreamWaitEvent(lo, start, 0));
+    return JMG_OK;
+  }
 };
 static int dev_aux(DevAux** out) {
   static std::mutex mu;
@@ -123,8 +135,8 @@ static int dev_aux(DevAux** out) {
   if (!a.lo) {
     int prio_lo = 0, prio_hi = 0;
     JMG_CUDA(cudaDeviceGetStreamPriorityRange(&prio_lo, &prio_hi));
-    for (auto& e : a.ev)
-      if (!e) JMG_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+    for (cudaEvent_t* e : {&a.start, &a.done})
+      if (!*e) JMG_CUDA(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
     JMG_CUDA(cudaStreamCreateWithPriority(&a.lo, cudaStreamNonBlocking, prio_lo));
   }
   *out = &a;
@@ -470,7 +482,7 @@ static int posv_mixed(int n, int nrhs, const double* A, int lda, double* B, int 
   // workspace alive for it).
   struct Prologue {
     cudaStream_t main = nullptr, s3 = nullptr;
-    cudaEvent_t start = nullptr, done = nullptr;
+    cudaEvent_t done = nullptr;
     bool pending = false;
     int wait() {
       if (pending) JMG_CUDA(cudaStreamWaitEvent(main, done, 0));
@@ -484,10 +496,8 @@ static int posv_mixed(int n, int nrhs, const double* A, int lda, double* B, int 
     DevAux* aux = nullptr;
     JMG_TRY(dev_aux(&aux));
     pro.s3 = aux->lo;  // the low-priority side stream and its events (made once per device)
-    pro.start = aux->ev[0];
-    pro.done = aux->ev[1];
-    JMG_CUDA(cudaEventRecord(pro.start, s));  // A and the workspace are ready here
-    JMG_CUDA(cudaStreamWaitEvent(pro.s3, pro.start, 0));
+    pro.done = aux->done;
+    JMG_TRY(aux->follow(s));  // A and the workspace are ready here
     if (p.split) {  // one pass for the row sums (||A||_inf) and row maxima (slice scales)
       double* rowmax = at<double>(work, p.off_ozrow);
       JMG_TRY(launch_row_stats(n, A, lda, c.rowsum, rowmax, pro.s3));
