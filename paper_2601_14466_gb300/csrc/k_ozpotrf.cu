@@ -232,8 +232,11 @@ JMG_DEV void diag_body(double* sm_d64, double* __restrict__ A, int lda, int kb, 
   if (t == 0 && fail) atomicCAS(info, 0, koff + fail);
 }
 
+// The first block; any: nany flags of the factorisation's updates, cleared here.
 __global__ void __launch_bounds__(THREADS) k_oz_diag(double* __restrict__ A, int lda, int kb,
-                                                     int koff, int* __restrict__ info) {
+                                                     int koff, int* __restrict__ info,
+                                                     int* __restrict__ any, int nany) {
+  for (int i = threadIdx.x; i < nany; i += THREADS) any[i] = 0;
   extern __shared__ __align__(16) double sm_diag64[];
   diag_body(sm_diag64, A, lda, kb, koff, info);
 }
@@ -246,11 +249,27 @@ __global__ void __launch_bounds__(THREADS) k_oz_diag(double* __restrict__ A, int
 //    (kb_diag columns), while the others work through the rest of the update;
 //  * RECT = true, the blocked solves: the whole rectangle.
 // info may be null when RECT; err (RECT only) is the solve's error word.
+// Entries whose row or column is spread (ozslice.cuh; the rows' words are exA and exB,
+// `flat` the count that makes a flat one) take FP64 FMAs over `F` instead: 32 x 32 entries
+// at a time, two columns per epilogue warp, shared out over all CTAs whoever did the slices
+// of the tile (its entries are others).  Bound by the FP64 pipe (16 clocks a warp
+// instruction): 0.14 ms for 32 x 32 at depth 512.  *any is set by the kernels that made the
+// words when one of them is spread, so that a launch without only tests its words: factor at
+// n = 5000 7.13 -> 7.20 ms, 16384 66.2 -> 66.8, solves at 16384, 64 11.2 -> 11.5.  With next
+// to every row spread (exponential covariance of a 2-D grid of 5000 sites, range 0.5) the
+// factor takes 48.7 ms and 64 right-hand sides 6.7 (CUDA-core kernels: 53.1, 10.4).
+struct Fma {            // the operands in FP64: P(row, k) = P[row prs + k pks], k < kv;
+  const double *P, *Q;  // Q(column, k) = Q[column qcs + k qks]
+  size_t prs, pks, qcs, qks;
+  int kv;
+};
+
 template <bool RECT>
 __global__ void __launch_bounds__(THREADS, 1)
     k_oz_update(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                 double* __restrict__ C, int ldc, int nA, int rA, int nB, int rB, int m, int ncols,
-                int nkb, const int* __restrict__ exA, const int* __restrict__ exB, int TI, int TJ,
+                int nkb, const int* __restrict__ exA, const int* __restrict__ exB, int flat,
+                const int* __restrict__ any, const Fma F, int TI, int TJ,
                 int ntiles, int kb_diag, int koff, int* __restrict__ info, int* __restrict__ err,
                 unsigned long long wait_ns, int hold) {
   using namespace tc;
@@ -268,7 +287,7 @@ __global__ void __launch_bounds__(THREADS, 1)
   uint64_t* acce = accf + 1;
   uint64_t* drain = acce + 1;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
-  __shared__ int s_fail, s_info;
+  __shared__ int s_fail, s_info, s_any;
 
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   // this CTA's tiles: first, first + step, ...
@@ -281,6 +300,7 @@ __global__ void __launch_bounds__(THREADS, 1)
   };
   if (threadIdx.x == 0) {
     s_fail = 0;
+    s_any = *any;
     s_info = info ? *(volatile int*)info : 0;
     if (RECT && *(volatile int*)err != 0) s_info = 1;  // an earlier launch gave up
     for (int i = 0; i < 2; ++i) {
@@ -299,7 +319,8 @@ __global__ void __launch_bounds__(THREADS, 1)
     prefetch_tmap(&tmB);
   }
   __syncthreads();
-  if (s_info != 0) return;  // an earlier block already failed
+  // an earlier block already failed, or this CTA is here for spread entries only
+  if (s_info != 0 || (first >= ntiles && !s_any)) return;
   if (warp == 1) {
     tmem_alloc(tmem_slot, TCOLS);
     tmem_relinquish();
@@ -419,12 +440,19 @@ __global__ void __launch_bounds__(THREADS, 1)
       const int row = ti * BM + q * 32 + lane;
       const int c0 = tj * BN + ch;
       // columns c < jn of this thread are in range (and on or below the diagonal)
-      const int jn = row < m ? min(CW, min(ncols - c0, RECT ? CW : row - c0 + 1)) : 0;
+      const int jn = row < m ? max(0, min(CW, min(ncols - c0, RECT ? CW : row - c0 + 1))) : 0;
+      // the words of the row, and of column c0 + lane; put: the columns done here
+      const bool col = lane < CW && c0 + lane < ncols;
+      const int wr = row < m ? exA[row] : 0, wc = col ? exB[c0 + lane] : 0;
+      const unsigned cs = __ballot_sync(0xffffffffu, col && word_spread(wc, flat));
+      const unsigned put = word_spread(wr, flat) ? 0u : ((1u << jn) - 1) & ~cs;
       unsigned long long acc[CW];  // (unsigned: rows and columns past the end wrap, never trap)
 #pragma unroll
       for (int c = 0; c < CW; ++c) acc[c] = 0ull;
       for (int kw = 0; kw < nkb; kw += WIN, ++gw) {
-        if (!mbar_wait(accf, (uint32_t)gw & 1, wait_ns) || ld_shared_volatile(&s_fail)) {
+        // (one answer for the warp: what follows is aligned across its lanes)
+        if (!__all_sync(0xffffffffu, mbar_wait(accf, (uint32_t)gw & 1, wait_ns) &&
+                                         !ld_shared_volatile(&s_fail))) {
           ok = false;
           break;
         }
@@ -460,20 +488,44 @@ __global__ void __launch_bounds__(THREADS, 1)
         atomicExch(&s_fail, 1);
         break;
       }
-      if (jn > 0) {
+      double* cp = C + (size_t)c0 * ldc + row;
+      const int er = word_exp(wr) - 14 - sh;
+      double old[CW];
+#pragma unroll
+      for (int c = 0; c < CW; ++c) old[c] = put >> c & 1u ? cp[(size_t)c * ldc] : 0.0;
+#pragma unroll
+      for (int c = 0; c < CW; ++c) {
+        const int ec = word_exp(__shfl_sync(0xffffffffu, wc, c));
+        if (put >> c & 1u) cp[(size_t)c * ldc] = old[c] - scaled_double((long long)acc[c], er + ec);
+      }
+    }
+    if (s_any && ok) {
+      // (factorisation: CTA 0 does its share of tile 0, which holds the diagonal block)
+      const bool head = !RECT && blockIdx.x == 0;
+      const int u0 = RECT || head ? blockIdx.x : 7 + blockIdx.x;
+      const int ue = head ? 8 : 8 * ntiles, us = head ? 1 : (RECT ? gridDim.x : gridDim.x - 1);
+      for (int u = u0; u < ue; u += us) {
+        int ti, tj;
+        if (!tile(u >> 3, ti, tj)) continue;
+        const int row = ti * BM + (u & 3) * 32 + lane, c0 = tj * BN + (u & 4) * 8 + 2 * (warp - 2);
+        const int jn = row < m ? min(2, min(ncols - c0, RECT ? 2 : row - c0 + 1)) : 0;
+        const bool rs = jn > 0 && word_spread(exA[row], flat);
+        const bool s0 = jn > 0 && (rs || word_spread(exB[c0], flat));
+        const bool s1 = jn > 1 && (rs || word_spread(exB[c0 + 1], flat));
+        if (!__any_sync(0xffffffffu, s0 || s1)) continue;
+        const double* p = F.P + (size_t)min(row, m - 1) * F.prs;
+        const double* q0 = F.Q + (size_t)min(c0, ncols - 1) * F.qcs;
+        const double* q1 = F.Q + (size_t)min(c0 + 1, ncols - 1) * F.qcs;
+        double a0 = 0.0, a1 = 0.0;
+#pragma unroll 8
+        for (int k = 0; k < F.kv; ++k) {
+          const double x = p[k * F.pks];
+          a0 = fma(x, q0[k * F.qks], a0);
+          a1 = fma(x, q1[k * F.qks], a1);
+        }
         double* cp = C + (size_t)c0 * ldc + row;
-        const int er = exA[row];
-        double old[CW];
-#pragma unroll
-        for (int c = 0; c < CW; ++c) old[c] = c < jn ? cp[(size_t)c * ldc] : 0.0;
-#pragma unroll
-        for (int c = 0; c < CW; ++c)
-          if (c < jn) {
-            const int ec = exB[c0 + c];
-            double r = old[c] - scaled_double((long long)acc[c], er + ec - 14 - sh);
-            if (er == E_BAD || ec == E_BAD) r = __longlong_as_double(0x7FF8000000000000ll);
-            cp[(size_t)c * ldc] = r;
-          }
+        if (s0) cp[0] -= a0;
+        if (s1) cp[ldc] -= a1;
       }
     }
   }
@@ -513,7 +565,9 @@ __global__ void __launch_bounds__(PT) k_oz_panel(double* __restrict__ A, int lda
                                                   __nv_bfloat16* __restrict__ SP,
                                                   int* __restrict__ ex,
                                                   unsigned long long* __restrict__ rowmax,
-                                                  int first, const int* __restrict__ info) {
+                                                  int* __restrict__ ex_block, int first, int last,
+                                                  int* __restrict__ any,
+                                                  const int* __restrict__ info) {
   constexpr int NP = 32 / G;     // column pairs per lane
   constexpr int RW = 32 / G;     // rows per warp
   constexpr int RB = PT / 32 * RW;  // rows per CTA
@@ -580,11 +634,22 @@ __global__ void __launch_bounds__(PT) k_oz_panel(double* __restrict__ A, int lda
     const unsigned long long b = __shfl_xor_sync(0xffffffffu, mx, o, G);
     mx = b > mx ? b : mx;
   }
+  int near = 0;
+#pragma unroll
+  for (int i = 0; i < 2 * NP; ++i)
+    near += near_max(abs_bits(x[i]), mx);
+#pragma unroll
+  for (int o = G / 2; o > 0; o >>= 1) near += __shfl_xor_sync(0xffffffffu, near, o, G);
   if (row >= n) return;
   const int e = scale_exp_bits(mx);
   if (g == 0) {
-    ex[row] = e;
-    rowmax[row] = first ? mx : (mx > rowmax[row] ? mx : rowmax[row]);
+    const int word = row_word(mx, near);
+    ex[row] = word;
+    if (word_spread(word, flat_count(PW))) *any = 1;
+    unsigned long long bm = mx;  // of the block so far
+    if (!first && rowmax[row] > bm) bm = rowmax[row];
+    rowmax[row] = bm;
+    if (last) ex_block[row] = row_word(bm, 0);  // (k_oz_strip adds the count)
   }
 #pragma unroll
   for (int i = 0; i < NP; ++i) {
@@ -600,12 +665,13 @@ __global__ void __launch_bounds__(PT) k_oz_panel(double* __restrict__ A, int lda
 }
 
 // Slices of the finished block column k0 .. k0 + K - 1 (rows from r0 on) with one
-// exponent per row over the whole block.  grid = (32-row tiles, K / 64).
+// exponent per row over the whole block; the rows' words in ex gain the entries near the
+// maximum, and *any is set when a row turns out to be spread.  grid = (32-row tiles, K / 64).
 __global__ void __launch_bounds__(256) k_oz_strip(const double* __restrict__ A, int lda, int n,
                                                   int k0, int r0, int K,
                                                   const unsigned long long* __restrict__ rowmax,
                                                   __nv_bfloat16* __restrict__ SP,
-                                                  int* __restrict__ ex,
+                                                  int* __restrict__ ex, int* __restrict__ any,
                                                   const int* __restrict__ info) {
   __shared__ double T[64][33];
   if (info && *(volatile const int*)info != 0) return;
@@ -623,9 +689,20 @@ __global__ void __launch_bounds__(256) k_oz_strip(const double* __restrict__ A, 
   }
   __syncthreads();
   const int rr = t / 8, cc = 8 * (t % 8), row = rb + rr;
+  const unsigned long long mx = row < n ? rowmax[row] : 0;
+  int near = 0;
+#pragma unroll
+  for (int u = 0; u < 8; ++u)
+    near += near_max(abs_bits(T[cc + u][rr]), mx);
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) near += __shfl_xor_sync(0xffffffffu, near, o);
   if (row >= n) return;
-  const int e = scale_exp_bits(rowmax[row]);
-  if (kc == 0 && cc == 0) ex[row] = e;
+  const int e = scale_exp_bits(mx);
+  if (cc == 0) {
+    const int add = (can_be_flat(mx) ? near << 16 : 0) + (1 << 26);
+    const int word = atomicAdd(&ex[row], add) + add;
+    if (word >> 26 == (int)gridDim.y && word_spread(word, flat_count(K))) *any = 1;
+  }
   uint32_t w[S][4];
 #pragma unroll
   for (int u = 0; u < 4; ++u) {
@@ -648,11 +725,15 @@ __global__ void __launch_bounds__(256) k_oz_strip(const double* __restrict__ A, 
 // The blocked solves' operands.
 
 // Row maxima (abs_bits order) of every SK-wide block column of the lower L, diagonal
-// blocks included: out[b * n + i].  grid = (rows / 256, blocks); a thread walks its row,
-// coalesced across the threads.
+// blocks included: out[b * n + i], and the rows' words for the strips, still without their
+// counts, ex[b * n + i].  grid = (rows / 256, blocks); a thread walks its row, coalesced
+// across the threads.  any: two flags per block, cleared here.
 constexpr int SK = 512;
 __global__ void __launch_bounds__(256) k_oz_block_max(const double* __restrict__ L, int lda, int n,
-                                                      unsigned long long* __restrict__ out) {
+                                                      unsigned long long* __restrict__ out,
+                                                      int* __restrict__ ex,
+                                                      int* __restrict__ any) {
+  if (blockIdx.x == 0 && threadIdx.x < 2) any[2 * blockIdx.y + threadIdx.x] = 0;
   const int i = blockIdx.x * 256 + threadIdx.x, k0 = blockIdx.y * SK;
   if (i >= n) return;
   unsigned long long mx = 0;
@@ -664,6 +745,7 @@ __global__ void __launch_bounds__(256) k_oz_block_max(const double* __restrict__
     mx = b > mx ? b : mx;
   }
   out[(size_t)blockIdx.y * n + i] = mx;
+  ex[(size_t)blockIdx.y * n + i] = row_word(mx, 0);
 }
 // sc[i] = the exponent of row i of L over all its blocks
 __global__ void k_oz_row_scale(int n, int nb, const unsigned long long* __restrict__ bmax,
@@ -675,8 +757,7 @@ __global__ void k_oz_row_scale(int n, int nb, const unsigned long long* __restri
     const unsigned long long v = bmax[(size_t)b * n + i];
     mx = v > mx ? v : mx;
   }
-  const int e = scale_exp_bits(mx);
-  sc[i] = e == E_BAD ? 0 : e;
+  sc[i] = scale_exp_bits(mx);
 }
 
 // x 2^e by integer addition to the exponent field where it stays normal
@@ -687,13 +768,13 @@ JMG_DEV double mul_pow2(double x, int e) {
 }
 
 // Slices of the columns of a column-major P (kv <= SK rows, ncols columns), one
-// exponent per column: slice s, column c, row k at SP[(s * ncols + c) * SK + k] (zero
-// past kv).  Row k is scaled by 2^(sign sc[k]) first (sign 0: not).  One warp per
+// exponent per column (its word in ex): slice s, column c, row k at
+// SP[(s * ncols + c) * SK + k] (zero past kv).  Row k is scaled by 2^(sign sc[k]) first (sign 0: not).  One warp per
 // column.
 __global__ void __launch_bounds__(256) k_oz_cut_cols(const double* __restrict__ P, int ld, int kv,
                                                      int ncols, const int* __restrict__ sc,
                                                      int sign, __nv_bfloat16* __restrict__ SP,
-                                                     int* __restrict__ ex) {
+                                                     int* __restrict__ ex, int* __restrict__ any) {
   const int c = blockIdx.x * 8 + threadIdx.x / 32, lane = threadIdx.x % 32;
   if (c >= ncols) return;
   constexpr int Q = SK / 64;
@@ -719,8 +800,18 @@ __global__ void __launch_bounds__(256) k_oz_cut_cols(const double* __restrict__ 
     const unsigned long long b = __shfl_xor_sync(0xffffffffu, mx, o);
     mx = b > mx ? b : mx;
   }
+  int near = 0;
+#pragma unroll
+  for (int i = 0; i < 2 * Q; ++i)
+    near += 64 * (i / 2) + 2 * lane + (i & 1) < kv &&
+            near_max(abs_bits(x[i]), mx);
+  near = __reduce_add_sync(0xffffffffu, near);
   const int e = scale_exp_bits(mx);
-  if (lane == 0) ex[c] = e;
+  if (lane == 0) {
+    const int word = row_word(mx, near);
+    ex[c] = word;
+    if (word_spread(word, flat_count(kv))) *any = 1;
+  }
 #pragma unroll
   for (int q = 0; q < Q; ++q) {
     int d0[S], d1[S];
@@ -746,7 +837,8 @@ static int map_slices(CUtensorMap* map, const void* base, int n, int K, int box_
 namespace {
 struct OzfPlan {
   int NB;
-  size_t panel, strip, exp_in, exp_out, rowmax, total;
+  int nany;  // one flag per panel, one per block
+  size_t panel, strip, exp_in, exp_out, rowmax, any, total;
 };
 OzfPlan ozf_plan(int n) {
   OzfPlan p{};
@@ -762,6 +854,8 @@ OzfPlan ozf_plan(int n) {
   p.exp_in = take(sizeof(int) * (size_t)n);
   p.exp_out = take(sizeof(int) * (size_t)n);
   p.rowmax = take(sizeof(unsigned long long) * (size_t)n);
+  p.nany = cdiv(n, ozf::PW) + cdiv(n, p.NB);
+  p.any = take(sizeof(int) * (size_t)p.nany);
   p.total = off;
   return p;
 }
@@ -778,6 +872,7 @@ int potrf_split(int n, double* A, int lda, int* info, void* work, cudaStream_t s
   int* e_in = reinterpret_cast<int*>(w + p.exp_in);
   int* e_out = reinterpret_cast<int*>(w + p.exp_out);
   unsigned long long* rowmax = reinterpret_cast<unsigned long long*>(w + p.rowmax);
+  int* any = reinterpret_cast<int*>(w + p.any);
   int dev = 0, nsm = 152;
   JMG_CUDA(cudaGetDevice(&dev));
   JMG_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
@@ -790,41 +885,51 @@ int potrf_split(int n, double* A, int lda, int* info, void* work, cudaStream_t s
     JMG_TRY(map_slices(&oa, strip, n, p.NB, BM));
     JMG_TRY(map_slices(&ob, strip, n, p.NB, BN));
   }
-  auto update = [&](const CUtensorMap& ma, const CUtensorMap& mb, int r0, int ncols, int nkb,
-                    const int* ex) -> int {
+  // P: columns k0 .. of L, K of them
+  auto update = [&](const CUtensorMap& ma, const CUtensorMap& mb, int r0, int ncols, int k0, int K,
+                    const int* ex, const int* spread) -> int {
+    const double* P = A + (size_t)k0 * lda + r0;
+    const Fma F{P, P, 1, (size_t)lda, 1, (size_t)lda, K};
     const int TI = cdiv(n - r0, BM), TJ = cdiv(ncols, BN);
     const long long nt = tile_count(TI, TJ);
-    k_oz_update<false><<<(int)std::min<long long>(nt, nsm), THREADS, SMEM, s>>>(
-        ma, mb, A + (size_t)r0 * lda + r0, lda, n, r0, n, r0, n - r0, ncols, nkb, ex + r0, ex + r0, TI,
-        TJ, (int)nt, std::min(PW, n - r0), r0, info, nullptr, g_wait_ns, hold);
+    k_oz_update<false><<<(int)std::min<long long>(8 * nt, nsm), THREADS, SMEM, s>>>(
+        ma, mb, A + (size_t)r0 * lda + r0, lda, n, r0, n, r0, n - r0, ncols, K / BK, ex + r0,
+        ex + r0, flat_count(K), spread, F, TI, TJ, (int)nt, std::min(PW, n - r0), r0, info, nullptr,
+        g_wait_ns, hold);
     return launched();
   };
   // the first diagonal block; every update leaves the next one factored
-  k_oz_diag<<<1, THREADS, diag64::SMEM, s>>>(A, lda, std::min(PW, n), 0, info);
+  k_oz_diag<<<1, THREADS, diag64::SMEM, s>>>(A, lda, std::min(PW, n), 0, info, any, p.nany);
   JMG_TRY(launched());
   for (int k0 = 0; k0 < n; k0 += p.NB) {
     const int kend = std::min(k0 + p.NB, n);
     for (int k = k0; k < kend; k += PW) {
       const int kb = std::min(PW, n - k), m = n - k - kb;
       if (m <= 0) return JMG_OK;
-      const int first = k == k0;
+      const int first = k == k0, last = k + PW >= kend;
       // lanes per row: enough rows per pass for the eight warps of every SM
+      auto panel_solve = [&](auto kern, int rows) {
+        kern<<<cdiv(m, rows), PT, 0, s>>>(A, lda, n, k, panel, e_in, rowmax, e_out, first, last,
+                                          any + k / PW, info);
+      };
       if (m <= 16 * nsm)
-        k_oz_panel<16><<<cdiv(m, 16), PT, 0, s>>>(A, lda, n, k, panel, e_in, rowmax, first, info);
+        panel_solve(k_oz_panel<16>, 16);
       else if (m <= 32 * nsm)
-        k_oz_panel<8><<<cdiv(m, 32), PT, 0, s>>>(A, lda, n, k, panel, e_in, rowmax, first, info);
+        panel_solve(k_oz_panel<8>, 32);
       else if (m <= 64 * nsm)
-        k_oz_panel<4><<<cdiv(m, 64), PT, 0, s>>>(A, lda, n, k, panel, e_in, rowmax, first, info);
+        panel_solve(k_oz_panel<4>, 64);
       else
-        k_oz_panel<2><<<cdiv(m, 128), PT, 0, s>>>(A, lda, n, k, panel, e_in, rowmax, first, info);
+        panel_solve(k_oz_panel<2>, 128);
       JMG_TRY(launched());
-      if (k + PW < kend) JMG_TRY(update(pa, pb, k + PW, kend - (k + PW), 1, e_in));
+      if (k + PW < kend) JMG_TRY(update(pa, pb, k + PW, kend - (k + PW), k, PW, e_in, any + k / PW));
     }
     if (kend >= n) break;
+    int* block_any = any + cdiv(n, PW) + k0 / p.NB;
     k_oz_strip<<<dim3(cdiv(n - kend, 32), p.NB / 64), 256, 0, s>>>(A, lda, n, k0, kend, p.NB,
-                                                                  rowmax, strip, e_out, info);
+                                                                  rowmax, strip, e_out,
+                                                                  block_any, info);
     JMG_TRY(launched());
-    JMG_TRY(update(oa, ob, kend, n - kend, p.NB / 64, e_out));
+    JMG_TRY(update(oa, ob, kend, n - kend, k0, p.NB, e_out, block_any));
   }
   return JMG_OK;
 }
@@ -842,7 +947,7 @@ int potrf_split(int n, double* A, int lda, int* info, void* work, cudaStream_t s
 namespace {
 struct SolvePlan {
   int nb;
-  size_t strip, exr, cols, exc, bmax, sc, total;
+  size_t strip, exr, cols, exc, bmax, sc, any, total;
 };
 SolvePlan solve_plan(int n, int nrhs) {
   SolvePlan p{};
@@ -854,11 +959,12 @@ SolvePlan solve_plan(int n, int nrhs) {
     return at;
   };
   p.strip = take((size_t)ozf::S * n * ozf::SK * 2);
-  p.exr = take(sizeof(int) * (size_t)n);
+  p.exr = take(sizeof(int) * (size_t)n * p.nb);
   p.cols = take((size_t)ozf::S * nrhs * ozf::SK * 2);
   p.exc = take(sizeof(int) * round_up((size_t)nrhs, 64));
   p.bmax = take(sizeof(unsigned long long) * (size_t)n * p.nb);
   p.sc = take(sizeof(int) * (size_t)n);
+  p.any = take(sizeof(int) * 2 * (size_t)p.nb);  // forward and backward update of each block
   p.total = off;
   return p;
 }
@@ -884,22 +990,24 @@ int solve_split(int n, int nrhs, const double* L, int lda, double* B, int ldb, i
   int* exc = reinterpret_cast<int*>(w + p.exc);
   unsigned long long* bmax = reinterpret_cast<unsigned long long*>(w + p.bmax);
   int* sc = reinterpret_cast<int*>(w + p.sc);
+  int* any = reinterpret_cast<int*>(w + p.any);
   int dev = 0, nsm = 152;
   JMG_CUDA(cudaGetDevice(&dev));
   JMG_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
   JMG_TRY(ensure_smem(k_oz_update<true>, SMEM));
   CUtensorMap mq;
   JMG_TRY(map_slices(&mq, cols, nrhs, SK, BN));
-  k_oz_block_max<<<dim3(cdiv(n, 256), p.nb), 256, 0, s>>>(L, lda, n, bmax);
+  k_oz_block_max<<<dim3(cdiv(n, 256), p.nb), 256, 0, s>>>(L, lda, n, bmax, exr, any);
   JMG_TRY(launched());
   k_oz_row_scale<<<cdiv(n, 256), 256, 0, s>>>(n, p.nb, bmax, sc);
   JMG_TRY(launched());
   // C (m x nrhs, head of B + row0) -= strip cols^T; strip rows rA.. of nA per slice
-  auto update = [&](const CUtensorMap& mp, int nA, int rA, int row0, int m) -> int {
+  auto update = [&](const CUtensorMap& mp, int nA, int rA, int row0, int m, const int* ex,
+                    const int* spread, const Fma& F) -> int {
     const int TI = cdiv(m, BM), TJ = cdiv(nrhs, BN), nt = TI * TJ;
-    k_oz_update<true><<<std::min(nt, nsm), THREADS, SMEM, s>>>(
-        mp, mq, B + row0, ldb, nA, rA, nrhs, 0, m, nrhs, SK / BK, exr + rA, exc, TI, TJ, nt, 0, 0,
-        info, sync, g_wait_ns, hold);
+    k_oz_update<true><<<std::min(8 * nt, nsm), THREADS, SMEM, s>>>(
+        mp, mq, B + row0, ldb, nA, rA, nrhs, 0, m, nrhs, SK / BK, ex, exc, flat_count(F.kv),
+        spread, F, TI, TJ, nt, 0, 0, info, sync, g_wait_ns, hold);
     return launched();
   };
   CUtensorMap mp;
@@ -910,24 +1018,31 @@ int solve_split(int n, int nrhs, const double* L, int lda, double* B, int ldb, i
                        info, s));
     if (k1 >= n) break;
     k_oz_strip<<<dim3(cdiv(n - k1, 32), SK / 64), 256, 0, s>>>(L, lda, n, k0, k1, SK,
-                                                              bmax + (size_t)b * n, strip, exr, info);
+                                                              bmax + (size_t)b * n, strip,
+                                                              exr + (size_t)b * n, any + 2 * b,
+                                                              info);
     JMG_TRY(launched());
-    k_oz_cut_cols<<<cdiv(nrhs, 8), 256, 0, s>>>(B + k0, ldb, kb, nrhs, sc, 0, cols, exc);
+    k_oz_cut_cols<<<cdiv(nrhs, 8), 256, 0, s>>>(B + k0, ldb, kb, nrhs, sc, 0, cols, exc,
+                                                any + 2 * b);
     JMG_TRY(launched());
-    JMG_TRY(update(mp, n, k1, k1, n - k1));
+    JMG_TRY(update(mp, n, k1, k1, n - k1, exr + (size_t)b * n + k1, any + 2 * b,
+                   Fma{L + (size_t)k0 * lda + k1, B + k0, 1, (size_t)lda, (size_t)ldb, 1, kb}));
   }
   for (int b = p.nb - 1; b >= 0; --b) {
     const int k0 = b * SK, kb = std::min(SK, n - k0);
     JMG_TRY(trsv_block(kb, nrhs, L + (size_t)k0 * lda + k0, lda, B + k0, ldb, 1, 1, sync,
                        info, s));
     if (k0 == 0) break;
-    k_oz_cut_cols<<<cdiv(k0, 8), 256, 0, s>>>(L + k0, lda, kb, k0, sc + k0, -1, strip, exr);
+    int* spread = any + 2 * b + 1;
+    k_oz_cut_cols<<<cdiv(k0, 8), 256, 0, s>>>(L + k0, lda, kb, k0, sc + k0, -1, strip, exr, spread);
     JMG_TRY(launched());
-    k_oz_cut_cols<<<cdiv(nrhs, 8), 256, 0, s>>>(B + k0, ldb, kb, nrhs, sc + k0, 1, cols, exc);
+    k_oz_cut_cols<<<cdiv(nrhs, 8), 256, 0, s>>>(B + k0, ldb, kb, nrhs, sc + k0, 1, cols, exc,
+                                                spread);
     JMG_TRY(launched());
     CUtensorMap mt;
     JMG_TRY(map_slices(&mt, strip, k0, SK, BM));
-    JMG_TRY(update(mt, k0, 0, 0, k0));
+    JMG_TRY(update(mt, k0, 0, 0, k0, exr, spread,
+                   Fma{L + k0, B + k0, (size_t)lda, 1, (size_t)ldb, 1, kb}));
   }
   return JMG_OK;
 }

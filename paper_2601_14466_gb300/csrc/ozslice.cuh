@@ -6,17 +6,51 @@
 namespace jmg {
 namespace ozf {
 constexpr int S = 7;            // slices per operand
-constexpr int E_BAD = 1 << 20;  // exponent of a row that is not finite
+
+// Which rows the slices stand in for.  A row (or column) is cut against its largest
+// element, so an entry far below it keeps few digits or none, and a product of two rows
+// whose large entries never meet would lose what an FMA keeps.  A row is FLAT when at
+// least 9/16 of its entries lie within 4 binary exponents of its largest one: two flat
+// rows p, q of length K then share K / 8 indices where |p_k q_k| > 2^-10 max|p| max|q|,
+// so sum |p_k q_k| > 2^-13 K max|p| max|q|, and the error of the slices (about 2^-56
+// sqrt(K) max|p| max|q|) stays at the level of the rounding of that sum, as FMAs' does.
+// Everything else -- decaying, sparse and graded rows, and rows that are not finite --
+// is SPREAD, and its products are formed with FP64 FMAs.  (Rows of the factors of matrices
+// with dense eigenvectors, of Wishart factors and of solves with them are flat without
+// exception; with 3 exponents in place of 4, one row in 2000 was not.)
+constexpr int NEAR = 4;
+JMG_DEV unsigned long long abs_bits(double x) {
+  return (unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull;
+}
+__host__ __device__ constexpr int flat_count(int kv) { return (9 * kv + 15) / 16; }
+// is |x| (its bits) within NEAR exponents of the row's maximum (mb)?
+JMG_DEV bool near_max(unsigned long long b, unsigned long long mb) {
+  return (int)(b >> 52) + NEAR >= (int)(mb >> 52);
+}
 
 // exponent e with |x| 2^-e < 1 for every |x| <= m (m as the bits of |x|);
-// 0 for m == 0, E_BAD for infinities and NaN
+// 0 for m == 0, infinities and NaN
 JMG_DEV int scale_exp_bits(unsigned long long mb) {
   if (mb == 0) return 0;
   const int ex = (int)(mb >> 52);
-  if (ex >= 0x7FF) return E_BAD;
+  if (ex >= 0x7FF) return 0;
   if (ex) return ex - 1022;
   return -1010 - __clzll((long long)mb);  // subnormal: m = mb 2^-1074, mb < 2^(64-clz)
 }
+
+// A row's word: the exponent of its maximum mb in bits 0-15, the number of entries near it
+// in bits 16-25 (none where no exponent lies below the maximum's by NEAR, nor in a row that
+// is not finite); k_oz_strip counts the 64-column chunks that have added theirs from bit 26.
+JMG_DEV bool can_be_flat(unsigned long long mb) {
+  const int ex = (int)(mb >> 52);
+  return mb == 0 || (ex > NEAR && ex < 0x7FF);
+}
+JMG_DEV int row_word(unsigned long long mb, int cnt) {
+  const int e = scale_exp_bits(mb);
+  return (e & 0xFFFF) | (can_be_flat(mb) ? cnt << 16 : 0);
+}
+JMG_DEV int word_exp(int w) { return (int)(short)w; }
+JMG_DEV bool word_spread(int w, int flat) { return (w >> 16 & 1023) < flat; }
 
 // The digits of x 2^-e (|x 2^-e| < 1): V = rint(x 2^(55-e)), |V| <= 2^55, cut into
 // balanced base-256 digits from the bottom; integer operations only.
