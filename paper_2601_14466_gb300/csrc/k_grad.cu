@@ -109,10 +109,16 @@ __global__ void __launch_bounds__(256) k_sym_grad(int n, int nrhs, const double*
 // levels (exact: |sum| <= 7 16 2^14 < 2^24), one conversion and one FP64 addition per
 // entry.  Column k of the pair is scaled by 2^s_k and 2^-s_k first (s_k from the tile's
 // column maxima), so that a pair with a large Bbar and a small X next to one with the
-// opposite costs no digits.  A chunk with an entry that is not finite takes FP64 FMAs
-// from the staged columns, as does everything after a wait that ran out.
-// n = 8192, 16 right-hand sides: 1829 -> 693 us (a tile's phases, not pipelined, take
-// ~25 us; the 537 MB written would take 80), error against 64 bits 0.75 of the FMAs'.
+// opposite costs no digits.
+//
+// Rows of either operand that are spread all the same (ozslice.cuh) take FP64 FMAs from
+// the staged columns, two rows by 16 columns of a warp at a time.  So does the whole
+// product when more than a quarter of its rows are spread, in a chunk of fewer than six
+// right-hand sides (sizes differ by chance there, and the FMAs are few), when an entry is
+// not finite, and after a wait that ran out.
+// n = 8192, 16 right-hand sides: 1829 us with FMAs alone -> 735 (a tile's phases, not
+// pipelined, take ~26 us; the 537 MB written would take 80), error against 64 bits 0.4 of
+// the FMAs'; 2100 when next to every row is spread (128 x 64 tiles, one CTA per SM).
 namespace grad {
 constexpr int BM = 128, BN = 64, TH = 512;
 constexpr int A_TILE = BM * 128, B_TILE = BN * 128;  // rows of 128 bytes, 16 BF16 of them used
@@ -136,7 +142,7 @@ __global__ void __launch_bounds__(grad::TH, 1)
   double* sQ = sP + KC * BM;                                  // [KC][BN]
   __shared__ uint64_t bar, drain;
   __shared__ uint32_t tmem_slot;
-  __shared__ int s_ep[BM], s_eq[BN], s_k[KC];  // row exponents, column shifts
+  __shared__ int s_ep[BM], s_eq[BN], s_k[KC];  // rows' exponents (2 e + spread), column shifts
   const int t = threadIdx.x, warp = t / 32, lane = t % 32;
   // tile b: row tile ti has the column tiles 0 .. 2 ti + 1
   int ti = (int)((sqrtf(4.0f * (float)blockIdx.x + 1.0f) - 1.0f) * 0.5f);
@@ -168,6 +174,7 @@ __global__ void __launch_bounds__(grad::TH, 1)
   bool ok = true;  // uniform over the CTA
   uint32_t phase = 0;
   for (int k0 = 0; k0 < nrhs; k0 += KC) {
+    const int kn = min(KC, nrhs - k0);
 #pragma unroll 1
     for (int half = 0; half < 2; ++half) {
       const double* P = half ? X : Bb;
@@ -194,7 +201,7 @@ __global__ void __launch_bounds__(grad::TH, 1)
 #pragma unroll
         for (int u = 0; u < 2; ++u) sQ[(t / BN + 8 * u) * BN + t % BN] = a[4 + u];
       }
-      const bool slices = __syncthreads_and(fin) && ok;
+      bool slices = __syncthreads_and(fin) && ok && kn >= 6;
       if (slices) {
         {  // column k = warp: shift by half the difference of the maxima's exponents
           unsigned mp = 0, mq = 0;
@@ -209,13 +216,15 @@ __global__ void __launch_bounds__(grad::TH, 1)
           if (lane == 0) s_k[warp] = ((int)(mq >> 20) - (int)(mp >> 20)) / 2;
         }
         __syncthreads();
-        if (t < 2 * (BM + BN)) {  // eight values of a row of P (t < 256) or Q
-          const bool isq = t >= 2 * BM;
-          const int w = isq ? t - 2 * BM : t, row = w / 2, h = 8 * (w & 1);
+        // eight values of a row of P (t < 256) or Q (t < 384)
+        const bool isq = t >= 2 * BM;
+        const int w = isq ? t - 2 * BM : t, row = w / 2, h = 8 * (w & 1);
+        double x[8];
+        int sk[8], e = -(1 << 20);
+        bool spread = false;
+        if (t < 2 * (BM + BN)) {
           const double* src = isq ? sQ + row : sP + row;
           const int ld = isq ? BN : BM;
-          double x[8];
-          int sk[8], e = -(1 << 20);
 #pragma unroll
           for (int u = 0; u < 8; ++u) {
             x[u] = src[(h + u) * ld];
@@ -225,7 +234,18 @@ __global__ void __launch_bounds__(grad::TH, 1)
             if (b) e = max(e, max((int)(b >> 52), 1) - 1022 + sk[u]);
           }
           e = max(e, __shfl_xor_sync(0xffffffffu, e, 1));
-          if (h == 0) (isq ? s_eq : s_ep)[row] = e;
+          int near = 0;  // entries near the row's largest (subnormal ones never)
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            const int f = (__double2hiint(x[u]) >> 20) & 0x7FF;
+            near += f > 0 && f - 1022 + sk[u] + ozf::NEAR >= e;
+          }
+          near += __shfl_xor_sync(0xffffffffu, near, 1);
+          spread = e > -(1 << 20) && near < ozf::flat_count(kn);
+          if (h == 0) (isq ? s_eq : s_ep)[row] = 2 * e + (spread ? 1 : 0);
+        }
+        slices = __syncthreads_count(spread) <= (BM + BN) / 2;  // (two threads per row)
+        if (slices && t < 2 * (BM + BN)) {
           uint32_t d4[S][4];
 #pragma unroll
           for (int u = 0; u < 4; ++u) {
@@ -246,6 +266,8 @@ __global__ void __launch_bounds__(grad::TH, 1)
                 make_uint4(d4[s][0], d4[s][1], d4[s][2], d4[s][3]);
           fence_proxy_async();
         }
+      }
+      if (slices) {
         tc_fence_before();
         __syncthreads();
         if (t == 0 && !hold) {  // (hold, a test hook: no products, the wait below runs out)
@@ -282,11 +304,37 @@ __global__ void __launch_bounds__(grad::TH, 1)
             acc[c] += d < 6 ? y << (sh - 8 * (d < 6 ? d : 0)) : (y + (1 << 7)) >> 8;
           }
         }
-        const int er = s_ep[r] - 14 - sh;
+        const int er = s_ep[r];
+        const unsigned cols = __ballot_sync(0xffffffffu, lane < CW && (s_eq[ch + (lane & 15)] & 1));
+        unsigned rows = __ballot_sync(0xffffffffu, er & 1);  // spread ones of this warp
 #pragma unroll
-        for (int c = 0; c < CW; ++c) v[c] += ozf::scaled_double(acc[c], er + s_eq[ch + c]);
+        for (int c = 0; c < CW; ++c)
+          if (!(er & 1) && !(cols >> c & 1u))
+            v[c] += ozf::scaled_double(acc[c], (er >> 1) + (s_eq[ch + c] >> 1) - 14 - sh);
+        if (cols)
+          for (int k = 0; k < kn; ++k) {
+            const double x = sP[k * BM + r];
+#pragma unroll
+            for (int c = 0; c < CW; ++c)
+              if (cols >> c & 1u) v[c] = fma(x, sQ[k * BN + ch + c], v[c]);
+          }
+        while (rows) {  // lanes 0-15: columns of row r0, lanes 16-31: of row r1
+          const int r0 = __ffs(rows) - 1;
+          rows &= rows - 1;
+          const int r1 = rows ? __ffs(rows) - 1 : r0;
+          rows &= rows - 1;
+          const double* p = sP + q * 32 + (lane < 16 ? r0 : r1);
+          const double* x = sQ + ch + (lane & 15);
+          double s = 0.0;
+          for (int k = 0; k < kn; ++k) s = fma(p[k * BM], x[k * BN], s);
+#pragma unroll
+          for (int c = 0; c < CW; ++c) {
+            const double y = __shfl_sync(0xffffffffu, s, lane == r0 ? c : 16 + c);
+            if ((lane == r0 || lane == r1) && !(cols >> c & 1u)) v[c] += y;
+          }
+        }
       } else {
-        for (int k = 0; k < KC; ++k)
+        for (int k = 0; k < kn; ++k)
 #pragma unroll
           for (int c = 0; c < CW; ++c) v[c] = fma(sP[k * BM + r], sQ[k * BN + ch + c], v[c]);
       }
@@ -324,10 +372,11 @@ int launch_sym_grad(int n, int nrhs, const double* Bb, int ldb, const double* X,
     JMG_CUDA(cudaMemset2DAsync(G, sizeof(double) * ldg, 0, sizeof(double) * n, n, s));
     return JMG_OK;
   }
-  // FP64 work grows with nrhs, a chunk on the tensor cores costs the same from 1 to 16:
-  // n = 8192 nrhs 5 630 / 693 us, 6 744 / 685; n = 2048 5 52 / 53, 8 77 / 53; one wave of
-  // tiles (n <= 1024) 11 31 / 29, 8 24 / 29.
-  if (nrhs >= (n <= 1024 ? 12 : 6)) {
+  // FP64 work grows with nrhs, a chunk on the tensor cores costs about the same from 6 to
+  // 16 (a little more with few, where more rows are spread by chance): n = 8192 nrhs 6 744
+  // / 830 us, 7 860 / 750, 8 970 / 790; n = 2048 6 60 / 75, 8 77 / 69; one wave of tiles (n
+  // <= 1024) 11 31 / 32, 8 24 / 32.
+  if (nrhs >= (n <= 1024 ? 12 : 7)) {
     using namespace grad;
     JMG_TRY(ensure_smem(k_sym_grad_tc, SMEM));
     const long long TI = cdiv(n, BM);

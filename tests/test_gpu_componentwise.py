@@ -91,6 +91,17 @@ def test_solve_keeps_small_entries():
     np.testing.assert_allclose(X, Y.astype(np.float64), rtol=64 * n * U64, atol=0)
 
 
+@pytest.mark.parametrize("n,nrhs", [(65, 12), (300, 16), (513, 21)])
+def test_adjoint_keeps_small_entries(n, nrhs):
+    Y, X = _wide((n, nrhs), 7), _wide((n, nrhs), 8)
+    Y[::3], X[::3] = torch.sign(Y[::3]), torch.sign(X[::3])  # flat rows in between
+    G = jmg.sym_grad(jmg.colmajor_copy(Y.to(DEV)), jmg.colmajor_copy(X.to(DEV))).cpu().numpy()
+    Yl, Xl = Y.numpy().astype(np.longdouble), X.numpy().astype(np.longdouble)
+    want = -(Yl @ Xl.T + Xl @ Yl.T) / 2
+    bound = (2 * nrhs + 2) * U64 * (np.abs(Yl) @ np.abs(Xl).T + np.abs(Xl) @ np.abs(Yl).T)
+    assert np.all(np.abs(G - want) <= bound)
+
+
 @pytest.mark.parametrize("where", ["L", "B"])
 @pytest.mark.parametrize("value", [float("inf"), float("nan")])
 def test_solve_with_entries_that_are_not_finite(where, value):
