@@ -11,17 +11,23 @@ namespace jmg {
 // Factor and solve in one kernel, FP64 arithmetic on T storage.  The factor is
 // kept unscaled: column j holds a_rj, w_j = 1 / a_jj, and u_rj = a_rj w_j goes to
 // the mirrored place above the diagonal, so that
-//   update     a_rc -= a_rj u_cj        (one FMA per element, full warps: the
-//                                        trailing triangle is a tail of the packed
-//                                        column-major order)
+//   update     a_rc -= a_rj u_cj        (one FMA per element, full warps: columns
+//                                        j1 .. j2 are a range of the packed column-major
+//                                        order)
 //   forward    b_k  -= b_j u_kj         (k > j)
 //   backward   x_k   = b_k w_k - sum_{i > k} u_ik x_i
 // need one FP64 instruction per element and no division (the pivot's reciprocal
 // runs on the integer pipe); l_rc = a_rc / sqrt(a_cc) is formed once at the end.
+// Columns come in blocks of JB: a column updates its own block at once, the columns
+// behind it with the block's other columns, as one sum of products subtracted from a_rc
+// once.  An entry is then rounded n / JB + JB times at its own size instead of n times,
+// which set the error: order 128, L 2.8e-16 (root mean square, of its largest entry) with a
+// rounding per column, 1.3e-16 so; order 48 1.7e-16 and 1.2e-16; X 9.4e-16 and 6.2e-16.  It
+// costs 3-5% of the time.
 // Bound by the FP64 pipe (one warp instruction per ~16 clocks and SM) with enough
 // systems resident per SM to cover the column chain: two barriers per column, none
-// in the solve.  1000 FP64 systems, one right-hand side: order 16 30 us, 48 89, 128
-// 1312 (93, 621 and 8890 us with a factor kernel of 256 threads and a solve with one
+// in the solve.  1000 FP64 systems, one right-hand side: order 16 21 us, 48 83, 128
+// 1348 (83, 611 and 8877 us with a factor kernel of 256 threads and a solve with one
 // thread per right-hand side).
 // The solve spreads 32 / KG right-hand sides over a warp, KG lanes each (as many
 // lanes as fill the warps, from 32 for one right-hand side per warp down to 4): the
@@ -29,6 +35,31 @@ namespace jmg {
 // ============================================================================
 namespace bat {
 constexpr int NMAX = 128;
+constexpr int JB = 16;  // columns per block
+// Pivots at the ends of T's range, whose reciprocal is not a normal number of T.  The fast
+// path multiplies by it; this one (not inlined: nothing of it is to cost the fast one
+// registers) divides, with the finished factor, one thread per right-hand side.
+template <typename T>
+JMG_DEV bool out_of_range(T w) {
+  constexpr T least = sizeof(T) == 8 ? (T)0x1p-1022 : (T)0x1p-126f;
+  return !(w >= least && w <= 1 / least);
+}
+template <typename T>
+__device__ __noinline__ void solve_by_division(const T* L, int lda, int n, int nrhs, T* B, int ldb) {
+  for (int q = threadIdx.x; q < nrhs; q += blockDim.x) {
+    T* b = B + (size_t)q * ldb;
+    for (int j = 0; j < n; ++j) {
+      const T y = b[j] / L[(size_t)j * lda + j];
+      b[j] = y;
+      for (int k = j + 1; k < n; ++k) b[k] -= L[(size_t)j * lda + k] * y;
+    }
+    for (int j = n - 1; j >= 0; --j) {
+      T x = b[j];
+      for (int k = j + 1; k < n; ++k) x -= L[(size_t)j * lda + k] * b[k];
+      b[j] = x / L[(size_t)j * lda + j];
+    }
+  }
+}
 // v (component k = g + KG h on lane g of the right-hand side's KG) <- U^-T D^-1 U^-1 v
 // with u_kj = U[k * ld + j], j < k, and w_k = 1 / d_k
 template <typename T, int KG, int H>
@@ -111,38 +142,59 @@ __global__ void __launch_bounds__(KG* H <= 64 ? 128 : 512) k_posv_batched(int n,
   __syncthreads();
   const int nel = n * (n + 1) / 2;
   int fail = n;  // first failing column
-  for (int j = 0; j < n; ++j) {
-    const double d = s[j * ld + j];
-    bool bad = false;
-    // u_j: the warps that hold rows below j (and the first one, for w_j)
-    if (32 * warp < n - 1 - j || warp == 0) {
-      const double w = pivot_rcp(d, &bad);
-      if (t == 0) s_w[j] = w;
-      for (int r = j + 1 + t; r < n; r += nt) s[r * ld + j] = s[j * ld + r] * w;
+  auto column = [&](int c) { return c * n - c * (c - 1) / 2; };  // its start in packed order
+  for (int p = 0; p < n && fail == n; p += bat::JB) {
+    const int pe = min(n, p + bat::JB), e2 = column(pe);
+    for (int j = p; j < pe; ++j) {
+      const double d = s[j * ld + j];
+      bool bad = false;
+      // u_j: the warps that hold rows below j (and the first one, for w_j)
+      if (32 * warp < n - 1 - j || warp == 0) {
+        const double w = pivot_rcp(d, &bad);
+        if (t == 0) s_w[j] = w;
+          for (int r = j + 1 + t; r < n; r += nt) s[r * ld + j] = s[j * ld + r] * w;
+      }
+      if (!(d > 0.0)) {  // (the same value on every thread)
+        fail = j;
+        break;
+      }
+      __syncthreads();
+      if (j + 1 == pe) break;
+      for (int e = column(j + 1) + t; e < e2; e += nt) {
+        const int rc = s_rc[e], c = rc >> 8, r = rc & 255;
+        s[c * ld + r] = fma(-s[j * ld + r], s[c * ld + j], s[c * ld + r]);
+      }
+      __syncthreads();
     }
-    if (!(d > 0.0)) {  // (the same value on every thread)
-      fail = j;
-      break;
-    }
-    __syncthreads();
-    const int c1 = j + 1;
-    for (int e = c1 * n - c1 * (c1 - 1) / 2 + t; e < nel; e += nt) {
+    if (fail < n || pe == n) break;  // (a block with columns behind it is a full one)
+    for (int e = e2 + t; e < nel; e += nt) {
       const int rc = s_rc[e], c = rc >> 8, r = rc & 255;
-      s[c * ld + r] = fma(-s[j * ld + r], s[c * ld + j], s[c * ld + r]);
+      const double *a = s + p * ld + r, *u = s + c * ld + p;
+      double sum = a[0] * u[0];
+#pragma unroll
+      for (int j = 1; j < bat::JB; ++j) sum = fma(a[j * ld], u[j], sum);
+      s[c * ld + r] -= sum;
     }
     __syncthreads();
   }
+  bool odd = false;
   if (t < fail) {
     s_l[t] = sqrt(s[t * ld + t]);
     s_il[t] = 1.0 / s_l[t];
+    odd = bat::out_of_range((T)s_w[t]);
   }
-  __syncthreads();
+  odd = __syncthreads_or(odd);
   for (int c = warp; c < fail; c += nw)
     for (int r = c + lane; r < n; r += 32)
       Ab[(size_t)c * lda + r] = (T)(r == c ? s_l[c] : s[c * ld + r] * s_il[c]);
   if (t == 0) info[blockIdx.x] = fail < n ? fail + 1 : 0;
   if (fail < n) return;
   T* Bb = B + (size_t)blockIdx.x * sB;
+  if (odd) {
+    __syncthreads();  // the factor is in global memory
+    bat::solve_by_division(Ab, lda, n, nrhs, Bb, ldb);
+    return;
+  }
   const int w0 = (warp + blockIdx.x) % nw;  // the first right-hand side takes turns over the quarters
   if constexpr (sizeof(T) == 8) {
     bat::solve_all<T, KG, H>(s, ld, s_w, n, nrhs, Bb, ldb, w0, nw, lane);
@@ -160,7 +212,9 @@ __global__ void __launch_bounds__(KG* H <= 64 ? 128 : 512) k_posv_batched(int n,
 // ============================================================================
 // FP32 storage above order 48: the factors come from k_potrf_diag_batched (k_dense.cu:
 // FP64 in the 32 x 32 diagonal sub-blocks only), the solve runs in FP32 on them, four
-// warps per system, eight above 32 right-hand sides.
+// warps per system, eight above 32 right-hand sides.  U lies behind w: in front of them
+// the same loops took 1.2-1.3 times as long from 32 right-hand sides on (1000 systems of
+// order 56, 70 right-hand sides: 274 -> 205 us, 264 with one thread per right-hand side).
 // ============================================================================
 template <int KG, int H>
 __global__ void __launch_bounds__(256) k_potrs_batched_f32(int n, int nrhs,
@@ -171,17 +225,22 @@ __global__ void __launch_bounds__(256) k_potrs_batched_f32(int n, int nrhs,
   extern __shared__ __align__(16) float sm_bat32[];
   if (info[blockIdx.x] != 0) return;
   const int ld = n | 1;
-  float* U = sm_bat32;         // U[r * ld + c] = l_rc / l_cc
-  float* w = U + n * ld;       // 1 / l_cc^2
-  float* s_l = w + n;          // l_cc
+  float* w = sm_bat32;  // 1 / l_cc^2
+  float* s_l = w + n;   // l_cc
+  float* U = s_l + n;   // U[r * ld + c] = l_rc / l_cc
   const float* Lb = L + (size_t)blockIdx.x * sA;
   const int t = threadIdx.x, nt = blockDim.x, lane = t % 32, warp = t / 32, nw = nt / 32;
+  bool odd = false;
   for (int c = t; c < n; c += nt) {
     const float l = Lb[(size_t)c * lda + c];
     s_l[c] = l;
     w[c] = 1.0f / l / l;
+    odd |= bat::out_of_range(w[c]);
   }
-  __syncthreads();
+  if (__syncthreads_or(odd)) {
+    bat::solve_by_division(Lb, lda, n, nrhs, B + (size_t)blockIdx.x * sB, ldb);
+    return;
+  }
   for (int c = warp; c < n; c += nw)
     for (int r = c + 1 + lane; r < n; r += 32) U[r * ld + c] = Lb[(size_t)c * lda + r] / s_l[c];
   __syncthreads();
