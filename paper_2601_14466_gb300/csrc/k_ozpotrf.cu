@@ -82,26 +82,24 @@ static long long tile_count(int TI, int TJ) {
 }
 
 // ---------------------------------------------------------------------------
-// Diagonal block of kb <= 64 columns, in place, by one CTA of THREADS threads.  A
-// dependent FP64 instruction waits 68 clocks and the pivots are a serial chain:
+// Diagonal block of kb <= 64 columns, in place, by one CTA of THREADS threads, in two
+// halves of 32: a column updates its own half at once, the first half updates the second
+// with one sum of 32 products per entry.  (Against updating all columns at once: half the
+// trailing work beside the chain, and an entry of the second half is rounded 32 times
+// less: error of L at n = 65 1.8e-16 -> 1.4e-16, n = 1024 2.0e-16 -> 1.8e-16, in the same
+// time.)
+// A dependent FP64 instruction waits 68 clocks and the pivots are a serial chain:
 // warp 0 keeps column j in registers (two rows per lane) and in
 // step j updates column j+1, takes pivot j+1 (its reciprocal in integers) and hands
 // u_j = column j / a_jj to the trailing warps (named barrier 1); those apply
-// a_rc -= a_rj u_c to columns j+2 .. , column j+2 first, which they release
+// a_rc -= a_rj u_c to columns j+2 .. of the half, column j+2 first, which they release
 // (named barrier 2: the chain's input of step j+1).  Each barrier is passed the same
-// number of times on both sides (their counts shrink with the trailing warps), and
-// nothing leaves the loop early: the first pivot that is not positive is
-// recorded and the columns from it on are dropped.
+// number of times on both sides, and nothing leaves the loop early: the first pivot that
+// is not positive is recorded and the columns from it on are dropped.
 namespace diag64 {
-// Trailing threads in step j: the trailing work sets the time of the first columns, the
-// chain that of the later ones, where every further warp in the queue of the SM's one
-// FP64 pipe (16 clocks a warp instruction) can hold it up.
-constexpr int J0 = 20;
-JMG_DEV int trail(int j) { return j < J0 ? 480 : 384; }
-// Participants of barrier 1 in step j: the chain warp and every thread that worked in
-// step j-1 (one that leaves arrives there once more, so that the others, who take its
-// elements over, see its last stores).
-JMG_DEV int count1(int j) { return 32 + trail(j > 0 ? j - 1 : 0); }
+constexpr int HB = 32;      // columns of a half
+constexpr int TRAIL = 384;  // trailing threads
+constexpr int BAR = 32 + TRAIL;
 constexpr int LD = PW + 1;
 constexpr int NEL = PW * (PW + 1) / 2;
 constexpr int SMEM = (PW * LD + 2 * PW + 2 * PW) * 8 + NEL * 2;
@@ -147,75 +145,86 @@ JMG_DEV void diag_body(double* sm_d64, double* __restrict__ A, int lda, int kb, 
     for (int r = c + lane; r < PW; r += 32) s_rc[base + r - c] = (unsigned short)((c << 8) | r);
   }
   __syncthreads();
-  if (warp == 0) {
-    double lo = s64[lane], hi = s64[lane + 32];  // column j, rows lane and lane + 32
-    bool bad = false;
-    double w = pivot_rcp(__shfl_sync(0xffffffffu, lo, 0), &bad);
-    int fj = bad ? 0 : -1;  // first failing column
-    for (int j = 0; j + 1 < kb; ++j) {
-      const int j1 = j + 1;
-      const double a1 = __shfl_sync(0xffffffffu, j1 < 32 ? lo : hi, j1 & 31);
-      const double v = a1 * w;  // u of row j+1
-      if (j > 0) bar_sync(2, 32 + trail(j - 1));  // column j+1 done to j-1
-      double* cn = &s64[j1 * LD];
-      double nlo = cn[lane], nhi = cn[lane + 32];
-      double* u = &s_u[(j & 1) * PW];
-      bad = false;
-      if (j1 < 32) {
-        nlo = fma(-lo, v, nlo);
-        const double d = __shfl_sync(0xffffffffu, nlo, j1);
-        u[lane] = lo * w;
-        u[lane + 32] = hi * w;
-        nhi = fma(-hi, v, nhi);
-        cn[lane] = nlo;
-        cn[lane + 32] = nhi;
-        __syncwarp();
-        bar_arrive(1, count1(j));
-        w = pivot_rcp(d, &bad);
-      } else {
-        nhi = fma(-hi, v, nhi);
-        const double d = __shfl_sync(0xffffffffu, nhi, j1 - 32);
-        u[lane + 32] = hi * w;
-        cn[lane + 32] = nhi;
-        __syncwarp();
-        bar_arrive(1, count1(j));
-        w = pivot_rcp(d, &bad);
-      }
-      if (bad && fj < 0) fj = j1;
-      lo = nlo;
-      hi = nhi;
-    }
-    if (lane == 0 && fj >= 0) fail = fj + 1;
-  } else if (warp < 16) {
-    const int tq = t - 32;  // index among the trailing threads
-    for (int j = 0; j + 1 < kb; ++j) {
-      const int nt = trail(j);
-      __syncwarp();
-      if (tq >= nt) {
-        bar_arrive(1, count1(j));
-        break;
-      }
-      bar_sync(1, count1(j));  // u_j and column j in place
-      const double* cj = &s64[j * LD];
-      const double* uj = &s_u[(j & 1) * PW];
-      if (j + 2 < kb) {
-        if (tq >= j + 2 && tq < kb) {
-          double* c2 = &s64[(j + 2) * LD];
-          c2[tq] = fma(-cj[tq], uj[j + 2], c2[tq]);
+  auto column = [](int c) { return c * PW - c * (c - 1) / 2; };  // its start in packed order
+  int fj = -1;  // first failing column (chain warp)
+  for (int p = 0; p < kb; p += HB) {
+    const int pe = min(kb, p + HB);
+    if (warp == 0) {
+      double lo = s64[p * LD + lane], hi = s64[p * LD + lane + 32];  // column j, two rows
+      bool bad = false;
+      double w = pivot_rcp(__shfl_sync(0xffffffffu, p ? hi : lo, 0), &bad);
+      if (bad && fj < 0) fj = p;
+      for (int j = p; j + 1 < pe; ++j) {
+        const int j1 = j + 1;
+        const double a1 = __shfl_sync(0xffffffffu, j1 < 32 ? lo : hi, j1 & 31);
+        const double v = a1 * w;  // u of row j+1
+        if (j > p) bar_sync(2, BAR);  // column j+1 done to j-1
+        double* cn = &s64[j1 * LD];
+        double nlo = cn[lane], nhi = cn[lane + 32];
+        double* u = &s_u[(j & 1) * PW];
+        bad = false;
+        if (j1 < 32) {
+          nlo = fma(-lo, v, nlo);
+          const double d = __shfl_sync(0xffffffffu, nlo, j1);
+          const double uhi = hi * w;
+          u[lane] = lo * w;
+          nhi = fma(-hi, v, nhi);
+          cn[lane] = nlo;
+          cn[lane + 32] = nhi;
+          s64[(lane + 32) * LD + j] = uhi;  // kept for the second half
+          __syncwarp();
+          bar_arrive(1, BAR);
+          w = pivot_rcp(d, &bad);
+        } else {
+          nhi = fma(-hi, v, nhi);
+          const double d = __shfl_sync(0xffffffffu, nhi, j1 - 32);
+          u[lane + 32] = hi * w;
+          cn[lane + 32] = nhi;
+          __syncwarp();
+          bar_arrive(1, BAR);
+          w = pivot_rcp(d, &bad);
         }
-        __syncwarp();
-        bar_arrive(2, 32 + nt);
+        if (bad && fj < 0) fj = j1;
+        lo = nlo;
+        hi = nhi;
       }
-      const int c3 = j + 3;
-      const int e3 = c3 >= PW ? NEL : c3 * PW - c3 * (c3 - 1) / 2;
-      for (int e = e3 + tq; e < NEL; e += nt) {
-        const int rc = s_rc[e], c = rc >> 8, r = rc & 255;
-        if (r >= kb) continue;
-        s64[c * LD + r] = fma(-cj[r], uj[c], s64[c * LD + r]);
+      if (p == 0) s64[(lane + 32) * LD + pe - 1] = hi * w;
+      if (lane == 0 && fj >= 0) fail = fj + 1;
+    } else if (warp <= TRAIL / 32) {
+      const int tq = t - 32;  // index among the trailing threads
+      for (int j = p; j + 1 < pe; ++j) {
+        __syncwarp();
+        bar_sync(1, BAR);  // u_j and column j in place
+        const double* cj = &s64[j * LD];
+        const double* uj = &s_u[(j & 1) * PW];
+        if (j + 2 < pe) {
+          if (tq >= j + 2 && tq < kb) {
+            double* c2 = &s64[(j + 2) * LD];
+            c2[tq] = fma(-cj[tq], uj[j + 2], c2[tq]);
+          }
+          __syncwarp();
+          bar_arrive(2, BAR);
+        }
+        const int e2 = column(pe);
+        for (int e = column(min(j + 3, pe)) + tq; e < e2; e += TRAIL) {
+          const int rc = s_rc[e], c = rc >> 8, r = rc & 255;
+          if (r >= kb) continue;
+          s64[c * LD + r] = fma(-cj[r], uj[c], s64[c * LD + r]);
+        }
       }
     }
+    __syncthreads();
+    if (pe == kb) break;
+    const int e = column(HB) + t;  // second half: 528 entries, one per thread
+    if (e < NEL) {
+      const int rc = s_rc[e], c = rc >> 8, r = rc & 255;
+      double sum = s64[r] * s64[c * LD];
+#pragma unroll 8
+      for (int j = 1; j < HB; ++j) sum = fma(s64[j * LD + r], s64[c * LD + j], sum);
+      s64[c * LD + r] -= sum;
+    }
+    __syncthreads();
   }
-  __syncthreads();
   const int jdone = fail ? fail - 1 : kb;  // columns that are final
   if (t < jdone) {  // l_cc = sqrt(a_cc), l_rc = a_rc / l_cc
     const double l = sqrt(s64[t * LD + t]);
