@@ -17,6 +17,7 @@ from __future__ import annotations
 import ctypes
 import os
 import threading
+import warnings
 from dataclasses import dataclass
 
 import torch
@@ -195,14 +196,17 @@ def workspace_size(op: int, n: int, nrhs: int, opts: Options | None = None,
 def workspace(op: int, n: int, nrhs: int, opts: Options | None, device,
               dtype: int = JMG_F64) -> torch.Tensor:
     """Scratch of one call: enough for its fastest route, or what it needs at least
-    when the device has no room for that."""
+    when the device has no room for that.  The call then takes another route, with other
+    rounding and up to 17 times slower, so a RuntimeWarning says so."""
     need = workspace_size(op, n, nrhs, opts, dtype)
     fast = int(load().jmg_workspace_fast(op, n, nrhs, dtype, ctypes.byref(opts) if opts else None))
     if fast > need:
         try:
             return torch.empty(fast, dtype=torch.uint8, device=device)
         except torch.cuda.OutOfMemoryError:
-            pass
+            warnings.warn("jmg: no room for the %d bytes of scratch of the fast FP64 route (n = %d); "
+                          "the call runs on the FP64 CUDA cores with %d" % (fast, n, need),
+                          RuntimeWarning, stacklevel=3)
     return torch.empty(max(need, 256), dtype=torch.uint8, device=device)
 
 
@@ -219,6 +223,7 @@ def _dtype_code(t: torch.Tensor) -> int:
 
 def potrf_(A: torch.Tensor, *, nb: int = 128, info: torch.Tensor | None = None) -> torch.Tensor:
     """Cholesky factorisation in place: lower(A) <- L (FP64 or FP32, column-major).
+    FP64 above order 64 takes scratch (about 8.1 KB per row, see ``workspace``).
     Returns the device info tensor (int32, 1 element); asynchronous."""
     _need_cuda(A)
     dt = _dtype_code(A)
