@@ -126,7 +126,8 @@ size_t jmg_workspace_size(int op, int n, int nrhs, int dtype, const jmg_options*
  * with a factorisation (potrf, posv, posv_host; n > 64), whose trailing updates
  * then run on the tensor cores in error-free slices (about 8.1 KB per row of A), and
  * with many right-hand sides in a large solve (potrs, posv, posv_host; nrhs > 16,
- * n >= 4096 and n >= 8192 or n * nrhs >= 250000; about as much), whose products do.  `work` has to
+ * n >= 4096 and n >= 8192 or n * nrhs >= 250000; nrhs > 100, n >= 1000 and n * nrhs >=
+ * 150000, or n > 512 and n * nrhs >= 600000; about as much), whose products do.  `work` has to
  * be 256-byte aligned for that; with less, they run on the FP64 CUDA cores. */
 size_t jmg_workspace_fast(int op, int n, int nrhs, int dtype, const jmg_options* opt);
 

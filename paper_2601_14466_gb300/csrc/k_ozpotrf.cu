@@ -983,8 +983,13 @@ size_t ozs_workspace(int n, int nrhs) {
   // Worth it where the one-launch solves are bound by their products.  Both directions,
   // one launch each / blocked: n = 4100, 64 right-hand sides 2.74 / 2.59 ms; 8192, 33:
   // 7.25 / 5.04; 16384, 16: 10.6 / 10.9; 16384, 20: 17.9 / 10.9; 16384, 64: 35.2 / 11.1;
-  // 12001, 100: 37.1 / 8.3.
-  if (nrhs <= 16 || n < 4096 || (n < 8192 && (long long)n * nrhs < 250000)) return 0;
+  // 12001, 100: 37.1 / 8.3.  Smaller orders with many right-hand sides: 600, 500 0.73 / 0.78;
+  // 600, 1000 1.48 / 1.35; 1000, 100 0.44 / 0.53; 1000, 200 0.74 / 0.62; 2000, 300 3.43 / 1.62;
+  // 4000, 200 8.1 / 2.8; 4000, 500 19.7 / 5.4.
+  if (nrhs <= 16) return 0;
+  const long long size = (long long)n * nrhs;
+  const bool many = nrhs > 100 && n > ozf::SK && size >= (n < 1000 ? 600000 : 150000);
+  if (!many && (n < 4096 || (n < 8192 && size < 250000))) return 0;
   return solve_plan(n, nrhs).total;
 }
 

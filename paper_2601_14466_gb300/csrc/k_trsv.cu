@@ -491,6 +491,29 @@ __global__ void __launch_bounds__(trsv::TH, 1)
   }
 }
 
+// Groups per launch.  Every launch keeps all of its CTAs resident (a leader waits for its
+// helpers), so more groups at once leave fewer SMs to help: with gb of them a launch takes
+// about the longer of its chain, 3.9 us a step, and the helpers' products, 4.3 us for 32 x
+// 32 times 16 right-hand sides on one SM, over nsm - gb nl SMs, and 0.6 of the shorter (n =
+// 8000: 4.5 ms modelled and measured for 4 groups at once, 2.45 for 2).  The gb with the
+// least time in all launches.  Both directions, as many groups as fit with one helper each
+// / this: n = 500, 1000 right-hand sides 2.00 / 1.07 ms; 1000, 1000 8.28 / 3.58; 4000, 300
+// 16.8 / 11.9; 8000, 500 270 / 71; up to 64 right-hand sides as before.  Blocks up to LAG
+// have no helpers to wait for: all groups in one launch.
+static int trsv_batch(int groups, int nblk, int lag, int nl, int nsm) {
+  if (nblk <= lag) return std::min(groups, 65535);
+  int best = 1;
+  double least = 0.0;
+  for (int gb = std::min(groups, std::max(1, nsm / (nl + 1))); gb >= 1; --gb) {
+    const double chain = 3.9 * nblk,
+                 products = 4.3 * gb * 0.5 * nblk * nblk / std::max(1, nsm - gb * nl);
+    const double time = cdiv(groups, gb) * (std::max(chain, products) +
+                                            0.6 * std::min(chain, products) + 6.0);
+    if (least == 0.0 || time < least) least = time, best = gb;
+  }
+  return best;
+}
+
 // leaders a group can have (see launch_trsv_persist)
 static int trsv_slots(int nrhs) { return nrhs <= trsv::GR ? trsv::GR : trsv::GR / 4; }
 
@@ -517,18 +540,16 @@ static int trsv_launch(int n, int nrhs, const T* L, int lda, T* B, int ldb, int 
   auto k = k_trsv_persist<T, NR>;
   JMG_TRY(ensure_smem(k, (int)smem));
   // the leaders plus one helper per block when they all fit; the tickets keep the
-  // dependency order either way.  A leader waits for its helpers, so every launch
-  // keeps all of its CTAs resident: groups go in batches, each with its leaders
-  // and at least one helper.
+  // dependency order either way.
   int dev = 0, nsm = 152;
   JMG_CUDA(cudaGetDevice(&dev));
   JMG_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
   const int nl = cdiv(std::min(nrhs, trsv::GR), NR);
   const int want = nl + std::max(0, nblk - trsv::Cfg<T, NR>::LAG);
-  const int batch = std::max(1, std::min(groups, nsm / (nl + 1)));
+  const int batch = trsv_batch(groups, nblk, trsv::Cfg<T, NR>::LAG, nl, nsm);
   for (int g0 = 0; g0 < groups; g0 += batch) {
     const int gn = std::min(batch, groups - g0);
-    const int gx = std::max(nl + 1, std::min(want, nsm / gn));
+    const int gx = want == nl ? nl : std::max(nl + 1, std::min(want, nsm / gn));
     k<<<dim3(gx, gn), trsv::TH, smem, s>>>(n, nrhs, L, lda, B, ldb, trans, g0, slots, tickets, done,
                                            pflag, err, info, g_wait_ns, hold);
     JMG_TRY(launched());
