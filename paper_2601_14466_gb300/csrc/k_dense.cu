@@ -74,10 +74,11 @@ int launch_potf2(float* A, int lda, int kb, int koff, int* info, cudaStream_t s)
 // columns j (x_rj = a_rj / L_jj, then a_rl -= x_rj L_lj for l > j).  Lkk sits in
 // shared memory; threads are (row, column-group) pairs.
 // ============================================================================
-template <typename T, int BR>
-__global__ void __launch_bounds__(256) k_trsm(T* __restrict__ A21, int lda, int m, int kb,
-                                              const T* __restrict__ Lkk,
+__global__ void __launch_bounds__(256) k_trsm(double* __restrict__ A21, int lda, int m, int kb,
+                                              const double* __restrict__ Lkk,
                                               const int* __restrict__ info) {
+  using T = double;
+  constexpr int BR = 32;
   if (*(volatile const int*)info != 0) return;
   extern __shared__ __align__(16) unsigned char sm_trsm[];
   T* Ls = reinterpret_cast<T*>(sm_trsm);  // kb x (kb+1), column-major
@@ -130,19 +131,13 @@ __global__ void __launch_bounds__(256) k_trsm(T* __restrict__ A21, int lda, int 
   }
 }
 
-template <typename T, int BR>
-static int trsm_impl(T* A21, int lda, int m, int kb, const T* Lkk, const int* info,
-                     cudaStream_t s) {
-  if (m <= 0) return JMG_OK;
-  size_t smem = ((size_t)kb * (kb + 1) + (size_t)kb * (BR + 1)) * sizeof(T);
-  auto k = k_trsm<T, BR>;
-  JMG_TRY(ensure_smem(k, (int)smem));
-  k<<<cdiv(m, BR), 256, smem, s>>>(A21, lda, m, kb, Lkk, info);
-  return launched();
-}
 int launch_trsm(double* A21, int lda, int m, int kb, const double* Lkk, const int* info,
                 cudaStream_t s) {
-  return trsm_impl<double, 32>(A21, lda, m, kb, Lkk, info, s);
+  if (m <= 0) return JMG_OK;
+  const size_t smem = ((size_t)kb * (kb + 1) + (size_t)kb * 33) * sizeof(double);
+  JMG_TRY(ensure_smem(k_trsm, (int)smem));
+  k_trsm<<<cdiv(m, 32), 256, smem, s>>>(A21, lda, m, kb, Lkk, info);
+  return launched();
 }
 // 16-bit words of the mixed path's tensor-core operands
 // word pairs (a, b) with a + b < words, ordered by significance
@@ -311,7 +306,7 @@ int launch_trsm(float* A21, int lda, int m, int kb, const float* Lkk, const int*
     return trsm_rows_launch<128, __half>(A21, lda, m, Lkk, info, 0, nullptr, nullptr, 0, s);
   if (kb == 64)
     return trsm_rows_launch<64, __half>(A21, lda, m, Lkk, info, 0, nullptr, nullptr, 0, s);
-  return trsm_impl<float, 64>(A21, lda, m, kb, Lkk, info, s);
+  return JMG_ERR_UNSUPPORTED;  // (a panel with rows below it is always full)
 }
 
 int launch_trsm_words(float* A21, int lda, int m, int kb, const float* Lkk, const int* info,
