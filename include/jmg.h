@@ -124,7 +124,9 @@ size_t jmg_workspace_size(int op, int n, int nrhs, int dtype, const jmg_options*
 /* Bytes of `work` with which the same call takes its fastest route: never less
  * than jmg_workspace_size().  More than that only for plain FP64 calls (prec NATIVE):
  * with a factorisation (potrf, posv, posv_host; n > 64), whose trailing updates
- * then run on the tensor cores in error-free slices (about 8.1 KB per row of A), and
+ * then run on the tensor cores in slices (about 8.1 KB per row of A; rows whose entries
+ * are spread too wide for that keep FP64 FMAs, so that small entries keep the accuracy
+ * these give them), and
  * with many right-hand sides in a large solve (potrs, posv, posv_host; nrhs > 16,
  * n >= 4096 and n >= 8192 or n * nrhs >= 250000; nrhs > 100, n >= 1000 and n * nrhs >=
  * 150000, or n > 512 and n * nrhs >= 600000; about as much), whose products do.  `work` has to

@@ -268,6 +268,10 @@ static int fused_launch(int n, int nrhs, int batch, T* A, int lda, long long sA,
   const size_t nel = (size_t)n * (n + 1) / 2;
   const size_t smem = sizeof(double) * ((size_t)n * (n | 1) + 3 * n) + sizeof(short) * ((nel + 1) / 2 * 2) +
                       (sizeof(T) == 4 ? sizeof(float) * ((size_t)n * (n | 1) + n) : 0);
+  // threads: enough for a column's rows and the trailing triangle of the first columns,
+  // few enough for many systems per SM.  1000 FP64 systems, one right-hand side, half as
+  // many / these / twice as many: order 24 38 / 31 / 30 us, 48 87 / 83 / 128, 80 403 / 365 /
+  // 360, 128 1408 / 1349 / - (order 64 215 / 209 / 181, 96 656 / 610 / 572).
   const int nt = n <= 24 ? 64 : (n <= 64 ? 128 : (n <= 96 ? 256 : 512));
   return by_shape(n, cdiv(nrhs, nt / 32), [&](auto kg, auto h) -> int {
     auto k = k_posv_batched<T, decltype(kg)::value, decltype(h)::value>;
@@ -292,8 +296,9 @@ template <>
 int posv_small_batched<float>(int n, int nrhs, int batch, float* A, int lda, long long sA,
                               float* B, int ldb, long long sB, int* info, cudaStream_t s) {
   if (n > bat::NMAX) return JMG_ERR_UNSUPPORTED;
-  // up to order 48 the factor in FP64 throughout (k_posv_batched; 1000 systems of
-  // order 48, one right-hand side: 93 us against 104 with the factor of larger orders)
+  // up to order 48 the factor in FP64 throughout (k_posv_batched): half the error of the
+  // factor of larger orders (L at order 48 2.5e-8 / 4.9e-8).  1000 systems, one right-hand
+  // side, this / that: order 25 31 / 47 us, 40 61 / 68, 48 88 / 82, 56 164 / 91.
   if (n > 0 && batch > 0 && n <= 48)
     return fused_launch<float>(n, nrhs, batch, A, lda, sA, B, ldb, sB, info, s);
   JMG_CUDA(cudaMemsetAsync(info, 0, sizeof(int) * (size_t)batch, s));

@@ -1,5 +1,5 @@
 // k_ozpotrf.cu -- FP64 Cholesky factorisation with its trailing updates on the
-// BF16 tensor cores, by error-free splitting (Ozaki, Ogita, Oishi and Rump 2012,
+// BF16 tensor cores, by splitting into exact slices (Ozaki, Ogita, Oishi and Rump 2012,
 // "Error-free transformations of matrix multiplication by using fast routines of
 // matrix multiplication and its applications").
 //
@@ -13,20 +13,23 @@
 // stay exact integers below 2^24 (levels 0..4; the last two may round their
 // lowest bit, 2^-54 of the row scales, in the worst case).  Each window is added
 // into one 64-bit integer per output; a single conversion to FP64 and one
-// subtraction from C end the update.  Against the FP64 CUDA-core update this
-// keeps the same 2^-53 relative to the rows of P and rounds C once per update
-// instead of once per product: over random Gram matrices of order 100 .. 3000 the
-// factor's error is 0.8-0.95 of the CUDA-core route's.
+// subtraction from C end the update.  What is cut off is relative to a row's largest
+// entry, so this stands in for FMAs where the rows' large entries meet (flat rows,
+// ozslice.cuh); entries of other rows, the sparse and the decaying ones, take FMAs.
+// Error of the factor against double-double (root mean square), CUDA-core route / this:
+// n = 65 1.4e-16 / 1.4e-16, n = 1024 kappa = 10 2.2e-16 / 1.8e-16, n = 2500 kappa = 1e4
+// 6.1e-15 / 4.0e-15.
 //
 // Two-level right-looking blocking: panels of 64 columns inside blocks of NB = 512,
 // one update of the block's remaining columns per panel (depth 64) and one of the
 // whole trailing matrix per block (depth 512, sliced again with one exponent per
 // row over the block); the CTA that updates the next diagonal block factors it in
 // the same launch, so a panel is two launches.  Factor alone on one GB300, FP64
-// CUDA-core updates -> here: n = 1024 3.66 -> 1.10 ms, 3000 18.6 -> 3.6, 5000
-// 53 -> 7.1, 16384 1260 -> 66.6 ms (there the tensor cores do 28 products of slices
-// for one of FP64: 620 TFLOP/s over the whole factorisation).  Per panel, small
-// trailing matrix: 51 us tile + diagonal block, 19 us panel solve.
+// CUDA-core updates -> here: n = 1024 3.66 -> 1.16 ms, 3000 18.6 -> 3.7, 5000
+// 53 -> 7.2, 16384 1260 -> 66.8 ms (there the tensor cores do 28 products of slices
+// for one of FP64: 620 TFLOP/s over the whole factorisation; blocks of 256 columns
+// 71.2).  Per panel, small trailing matrix: 51 us tile + diagonal block, 19 us panel
+// solve.
 #include <algorithm>
 
 #include "kernels.h"

@@ -28,7 +28,7 @@
 // 16 right-hand sides (28-32 us with one lane per right-hand side substituting and
 // barriers between the phases): both directions at n = 12288, 8 right-hand sides,
 // 24.3 -> 3.6 ms.  From 17 right-hand sides on the helpers' products bound it
-// (n = 16384, 64: 42.8 -> 35.1 ms, 0.98 TFLOP/s of 1.1); large solves then run blocked,
+// (n = 16384, 64: 42.8 -> 33.6 ms, 1.02 TFLOP/s of 1.1); large solves then run blocked,
 // with their products on the tensor cores (solve_split in k_ozpotrf.cu).
 //
 // Roles come from an atomic ticket in order (tickets below the number of leaders
