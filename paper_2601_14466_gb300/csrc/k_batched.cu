@@ -21,9 +21,12 @@ namespace jmg {
 // Columns come in blocks of JB: a column updates its own block at once, the columns
 // behind it with the block's other columns, as one sum of products subtracted from a_rc
 // once.  An entry is then rounded n / JB + JB times at its own size instead of n times,
-// which set the error: order 128, L 2.8e-16 (root mean square, of its largest entry) with a
-// rounding per column, 1.3e-16 so; order 48 1.7e-16 and 1.2e-16; X 9.4e-16 and 6.2e-16.  It
-// costs 3-5% of the time.
+// which set the error (root mean square, of the largest entry): L at order 128 2.8e-16
+// with a rounding per column, 1.6e-16 with blocks of 32, 1.3e-16 with 16, X 9.4e-16, 6.7e-16
+// and 6.2e-16; L at order 48 1.7e-16, 1.5e-16 and 1.2e-16, X 5.9e-16, 5.1e-16 and 4.5e-16 (the
+// blocked kernels before: 1.6, 6.9, 1.5 and 5.4e-16).  Time in the same order, one
+// right-hand side: 1000 systems of order 48 78, 80 and 84 us, 20000 - , 1436 and 1413; 1000
+// of order 128 1302, 1339 and 1348.
 // Bound by the FP64 pipe (one warp instruction per ~16 clocks and SM) with enough
 // systems resident per SM to cover the column chain: two barriers per column, none
 // in the solve.  1000 FP64 systems, one right-hand side: order 16 21 us, 48 83, 128
