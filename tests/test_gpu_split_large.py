@@ -68,3 +68,43 @@ def test_solve_behind_a_failed_factor_leaves_the_right_hand_sides():
     assert st == 0
     assert int(info.item()) == 3001
     assert torch.equal(X, B)
+
+
+def _spiky(n, g):
+    """A lower factor with dense rows, every fifth one spiky (one large entry in sixteen)."""
+    L = torch.randn(n, n, generator=g, dtype=torch.float64, device=DEV).mul_(n ** -0.5).tril_(-1)
+    small = torch.rand(n, n, generator=g, dtype=torch.float64, device=DEV) > 1 / 16
+    small[torch.arange(n, device=DEV) % 5 != 3] = False
+    L[small] *= 1e-9
+    L.diagonal().copy_(2.0 + torch.rand(n, generator=g, dtype=torch.float64, device=DEV))
+    return L
+
+
+@pytest.mark.parametrize("n", [777, 2600])
+def test_factor_with_some_spread_rows(n):
+    # the entries of a tile are shared out: those of spread rows and columns to the FMAs
+    # (other CTAs), the rest to the slices
+    g = torch.Generator(device=DEV).manual_seed(n)
+    L0 = _spiky(n, g)
+    A = L0 @ L0.t()
+    W = jmg.colmajor_copy(A)
+    assert int(jmg.potrf_(W).item()) == 0
+    L = torch.tril(W)
+    R = (A - L @ L.t()).abs().tril()
+    s = A.diagonal().sqrt()
+    # (2 n + 2) u s_i s_j as above, n u s_i s_j for this product
+    assert bool((R <= (3 * n + 2) * U64 * s[:, None] * s[None, :]).all())
+
+
+@pytest.mark.parametrize("n,nrhs", [(4230, 70), (8192, 19)])
+def test_solve_with_some_spread_rows_and_columns(n, nrhs):
+    g = torch.Generator(device=DEV).manual_seed(n)
+    L = _spiky(n, g)
+    B = torch.randn(n, nrhs, generator=g, dtype=torch.float64, device=DEV)
+    B[:, ::3] = 0.0
+    B[torch.randint(0, n, (40,), generator=g, device=DEV), 0] = 1.0  # sparse ones
+    B[n - 1, ::3] = 1.0
+    X = jmg.potrs_(jmg.colmajor_copy(L), jmg.colmajor_copy(B))
+    R = (L @ (L.t() @ X) - B).abs()
+    La = L.abs()
+    assert bool((R <= 4 * (n + 2) * U64 * (La @ (La.t() @ X.abs()) + B.abs())).all())
